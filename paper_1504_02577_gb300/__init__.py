@@ -505,7 +505,10 @@ class Panther:
         torch = self.torch
         rows, R, L, stride = panther_paths_view(self.h.paths)
         with torch.cuda.stream(self.stream):
-            t = _device_view(torch, rows, (R, stride), torch.int32, self.device)[:, :L].contiguous()
+            # clone, not contiguous(): at L == stride the slice is contiguous already
+            # and would be the library's own memory, gone with the handle
+            t = _device_view(torch, rows, (R, stride), torch.int32, self.device)[:, :L].clone(
+                memory_format=torch.contiguous_format)
         self._leave(t)
         return t
 
