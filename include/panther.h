@@ -243,11 +243,12 @@ PANTHER_API panther_status panther_index_view(const panther_index* ix, const int
  * contain u (each path counted once per u), for every u != v; then the k
  * largest by (cnt desc, u asc). Writes out_ids int32[q][k] and
  * out_counts uint32[q][k] (similarity S_RP(v,u) = cnt / R).
- *   q >= 0 (q = 0 is a no-op), 1 <= k <= 128, queries in [0, n). With
- *   k <= 64 every tier runs; with 64 < k <= 128 queries of up to 32 paths
- *   stay in the group tiers and every other query is counted in a per-query
- *   device table and selected with 128-entry lists (slower, same results);
- *   the PLAIN form then runs that path once per query.
+ *   q >= 0 (q = 0 is a no-op), 1 <= k <= 128, queries in [0, n). Batches of
+ *   up to 16,384 queries (1,024 for k > 64) run as one launch with a CTA per
+ *   query, larger ones by tiers; queries with more candidates than a shared
+ *   memory table holds go to the hub tier in both. With k > 64 the hub tier
+ *   uses device tables and 128-entry lists only, and the PLAIN form runs the
+ *   batched one once per query.
  *   flags: PANTHER_TOPK_BATCHED or PANTHER_TOPK_PLAIN, optionally
  *          | PANTHER_IO_HOST (queries/outputs in host memory; the call then
  *          synchronises; batches of 4M queries or more run in four chunks
@@ -256,7 +257,7 @@ PANTHER_API panther_status panther_index_view(const panther_index* ix, const int
  * scratch budget; a batch whose hubs do not fit is processed in several
  * rounds.
  * Host waits: the BATCHED form is not fully asynchronous. After the lane,
- * group and persistent launches it copies the number of hub queries to the
+ * group, warp and CTA launches it copies the number of hub queries to the
  * host and waits for the context stream (once per call); when there are hub
  * queries it waits again to read their path counts and once per hub round
  * (to read which queries need a second, exact pass). The call therefore
@@ -271,9 +272,12 @@ PANTHER_API panther_status panther_topk(panther_ctx* ctx, const panther_index* i
 /* Tier sizes of the last panther_topk call on this context (also set by
  * pantherpp_vectors, which counts through the same tiers):
  *   [0] queries, [1] lane tier, [2] group tiers (8/16/32 lanes per query),
- *   [3] warp tier, [4] CTA tier (both persistent passes), [5] hub queries,
+ *   [3] warp tier, [4] CTA tier (both passes; small batches count here every
+ *       query that is no hub), [5] hub queries,
  *   [6] hub queries counted through the bucketed two-pass tier (per round),
- *   [7] hub queries counted in per-query device tables (per round),
+ *   [7] hub queries counted in per-query device tables (per round). With
+ *       k > 64 [5] and [7] also hold the queries counted in per-query tables
+ *       in shared memory, and [3] and [4] are 0,
  *   [8] hub queries whose buckets overflowed (counted again in tables),
  *   [9] hub queries counted a second time because the first-round
  *       threshold could have dropped a top-k candidate.
@@ -281,7 +285,7 @@ PANTHER_API panther_status panther_topk(panther_ctx* ctx, const panther_index* i
 PANTHER_API panther_status panther_topk_stats(panther_ctx* ctx, int64_t stats[10]);
 
 /* Autotuner for the batched form: runs the batch once per candidate launch
- * shape of the persistent kernel (threads per CTA, shared-table slots, CTAs
+ * shape of the CTA tier's kernel (threads per CTA, shared-table slots, CTAs
  * per SM), times three more runs of each with CUDA events on the context
  * stream, and keeps the fastest shape in the context for later calls.
  * Arguments as panther_topk (device pointers); the outputs hold the batch's

@@ -68,7 +68,7 @@ panther_status panther_create(panther_ctx** out, int device, void* cuda_stream) 
         ctx->own_stream = true;
     }
     if (cudaMalloc(&ctx->d_status, 4 * sizeof(uint32_t)) != cudaSuccess ||
-        cudaMallocHost(&ctx->h_status, 4 * sizeof(uint32_t)) != cudaSuccess ||
+        cudaMallocHost(&ctx->h_status, (4 + 16) * sizeof(uint32_t)) != cudaSuccess ||
         cudaMemset(ctx->d_status, 0, 4 * sizeof(uint32_t)) != cudaSuccess) {
         cudaGetLastError();
         if (ctx->d_status) cudaFree(ctx->d_status);
@@ -76,6 +76,7 @@ panther_status panther_create(panther_ctx** out, int device, void* cuda_stream) 
         delete ctx;
         return PANTHER_ECUDA;
     }
+    ctx->h_counts = (int*)(ctx->h_status + 4);
     // side streams and their events (optional: without them everything runs on `stream`)
     bool side_ok = cudaEventCreateWithFlags(&ctx->fork, cudaEventDisableTiming) == cudaSuccess;
     for (int i = 0; i < 2 && side_ok; ++i)

@@ -1,23 +1,19 @@
 // Co-occurrence counting and top-k (Algorithm 1, Eq. (4)).
 //
 // For query v every path r in P_v contributes 1 to cnt(v,u) for each distinct
-// u != v on the path. Counts accumulate in an open-addressing hash of 64-bit
-// slots (vertex << 32 | count); a slot is claimed with one 64-bit CAS and
-// bumped with one 64-bit add. The top-k by (count desc, id asc) is the k
-// largest of score = count << 32 | (2^32 - 1 - id), kept as a sorted list
-// spread over a warp's registers (rank l in lane l, rank 32+l in lane l's
-// second register) and merged across warps through shared memory.
+// u != v on the path. The top-k by (count desc, id asc) is the k largest of
+// score = count << 32 | (2^32 - 1 - id).
 //
-// Queries are split by the bound cap = min(n-1, |P_v| * T) on their distinct
-// candidates:
-//   warp tier  (cap <= 256):      a warp-private 512-slot table in smem
-//   CTA tier   (cap <= CTA cap):  one CTA, a table filling most of smem
-//   global tier (larger):         a table in device memory, filled by many
-//                                 CTAs, read back in chunks, partial top-k
-//                                 lists merged per query
-// The warp and CTA tiers run in ONE persistent launch whose CTAs pull work
-// from device counters (CTA-tier queries first, then warp-tier queries in
-// chunks), so skewed |P_v| does not leave SMs idle.
+// Queries are split by |P_v| and the bound cap = min(n-1, |P_v| * T) on their
+// distinct candidates:
+//   lane, group tiers (|P_v| <= 6, 32; T <= 7): registers only
+//   warp tier (cap <= WCAP):     one warp, a table of up to WSLOTS slots in smem
+//   CTA tier  (cap <= CTA cap):  one CTA, a table filling its share of smem;
+//                                a second pass with the largest table
+//   hub tier (larger):           tables in device memory or hashed buckets,
+//                                filled by many CTAs, partial lists merged
+// Warp and CTA tiers are persistent launches whose teams pull queries from
+// device counters, so skewed |P_v| does not leave SMs idle.
 #include <algorithm>
 #include <atomic>
 #include <type_traits>
@@ -31,17 +27,18 @@ constexpr uint64_t EMPTY = ~0ull;
 // path ids are unsigned 32-bit (R <= 2^32 - 1, so no valid id is all ones);
 // lanes without a path pass NO_PATH, which every reader rejects with r >= R
 constexpr uint32_t NO_PATH = 0xffffffffu;
-constexpr int WSLOTS = 512;      // warp-tier table slots
-constexpr int WCAP = 256;        // warp-tier candidate bound
+constexpr int WSLOTS = 1024;     // warp-tier table slots
+constexpr int WCAP = 512;        // warp-tier candidate bound
+constexpr int HUB_MIN_CAP = 256; // lowest hub-tier bound of the test routing
 // A query's own path count bounds the work of the tier that takes it: one
 // warp (warp tier) or one CTA (CTA tiers) walks every path of P_v, so a query
 // with few candidates but more paths than these (a small graph with a large
 // R) goes to a wider tier, and beyond CTA_MAX_NP to the hub tier, which
 // splits P_v over many CTAs.
-constexpr int64_t WARP_MAX_NP = int64_t(1) << 16;
+constexpr int64_t WARP_MAX_NP = int64_t(1) << 12;
+constexpr int64_t MID_MAX_NP = int64_t(1) << 14;   // beyond: the pass with the widest CTAs
 constexpr int64_t CTA_MAX_NP = int64_t(1) << 20;
 constexpr int KMAX = 64;
-constexpr int WCHUNK = 16;       // warp-tier queries fetched per atomic
 
 __device__ __forceinline__ uint32_t hslot(uint32_t key, uint32_t nslots) {
     return __umulhi(key * 0x9E3779B1u ^ (key >> 15), nslots);
@@ -72,9 +69,11 @@ __device__ __forceinline__ bool hash_add(unsigned long long* tab, uint32_t nslot
 }
 
 // table size for a query whose distinct candidates are at most cap: about
-// twice cap, a multiple of 32, within [lo, hi]
+// three times cap, a multiple of 32, within [lo, hi]. (Collisions cost more
+// than clearing: with 1.5, 2 and 3 times cap the team kernels took 1.34, 1.10
+// and 1.02 ms on all vertices of 5M, R = 1e7, T = 5.)
 __device__ __forceinline__ uint32_t table_size(int64_t cap, uint32_t lo, uint32_t hi) {
-    int64_t t = ((2 * cap + 31) / 32) * 32;
+    int64_t t = ((3 * cap + 31) / 32) * 32;
     return (uint32_t)(t < lo ? lo : (t > hi ? hi : t));
 }
 
@@ -196,38 +195,6 @@ __device__ __forceinline__ uint64_t slot_score(unsigned long long s) {
     if (s == EMPTY) return 0;
     uint32_t key = (uint32_t)(s >> 32), cnt = (uint32_t)s;
     return ((uint64_t)cnt << 32) | (uint64_t)(0xffffffffu - key);
-}
-
-// Top-k of a warp-private table of ns slots (ns a multiple of 32). With at
-// most 64 filled slots they are compacted in place and sorted once; otherwise
-// every slot is offered to a running list. The table is garbage afterwards.
-__device__ __forceinline__ WarpTopK warp_table_topk(unsigned long long* tab, uint32_t ns, int k) {
-    const unsigned lane = threadIdx.x & 31, lt = (1u << lane) - 1u;
-    int filled = 0;
-    for (uint32_t base = 0; base < ns; base += 32)
-        filled += __popc(__ballot_sync(0xffffffffu, tab[base + lane] != EMPTY));
-    WarpTopK t;
-    if (filled > 64) {
-        for (uint32_t base = 0; base < ns; base += 32) t.offer(slot_score(tab[base + lane]), k);
-        return t;
-    }
-    uint64_t mine[2] = {0, 0};
-    int pos = 0;
-    for (uint32_t base = 0; base < ns; base += 32) {
-        const uint64_t sc = slot_score(tab[base + lane]);
-        const unsigned m = __ballot_sync(0xffffffffu, sc != 0);
-        const int at = pos + __popc(m & lt);
-        // every lane read its slot before the ballot, and at < base + 32
-        if (sc) tab[at] = sc;
-        pos += __popc(m);
-    }
-    __syncwarp();
-    mine[0] = lane < (unsigned)filled ? tab[lane] : 0;
-    mine[1] = 32 + lane < (unsigned)filled ? tab[32 + lane] : 0;
-    warp_sort64_desc(mine[0], mine[1]);
-    t.a = mine[0];
-    t.b = mine[1];
-    return t;
 }
 
 struct OutRef {
@@ -861,8 +828,8 @@ struct Tiers {
 constexpr int CL_PER = 16;
 
 __global__ void __launch_bounds__(256) classify_kernel(const int32_t* __restrict__ queries, int64_t q, PathsRef P,
-                                                       int64_t ccap, int64_t ccap_big, bool lane_ok, int group_max,
-                                                       bool all_hub,
+                                                       int64_t wcap, int64_t ccap, int64_t ccap_big, bool lane_ok,
+                                                       int group_max,
                                                        Tiers tiers, OutRef o, uint32_t* status) {
     __shared__ unsigned tot[8];
     __shared__ int base[8];
@@ -888,9 +855,9 @@ __global__ void __launch_bounds__(256) classify_kernel(const int32_t* __restrict
                     else if (np <= 8 && np <= group_max) t = 4;
                     else if (np <= 16 && np <= group_max) t = 5;
                     else if (np <= 32 && np <= group_max) t = 6;
-                    else if (all_hub) t = 2;     // k > 64: the rest in device tables
-                    else if (np > CTA_MAX_NP) t = 2;
-                    else t = (cap <= WCAP && np <= WARP_MAX_NP) ? 0 : (cap <= ccap ? 1 : (cap <= ccap_big ? 7 : 2));
+                    else if (np > CTA_MAX_NP || cap > ccap_big) t = 2;
+                    else if (cap <= wcap && np <= WARP_MAX_NP) t = 0;
+                    else t = (cap <= ccap && np <= MID_MAX_NP) ? 1 : 7;
                 }
             }
             if (t < 0) {
@@ -1017,278 +984,761 @@ __device__ void cta_select(unsigned long long* tab, uint32_t nslots, unsigned lo
     __syncthreads();
 }
 
-// CTA-wide: count one query into the shared table and write its top-k
-template <int STRIDE>
-__device__ void cta_query(const PathsRef& P, int32_t v, int64_t qi, unsigned long long* tab, uint32_t max_slots,
-                          unsigned long long* lists, const OutRef& o, uint32_t* status) {
-    int64_t a = P.off[v], b = P.off[v + 1];
-    const uint32_t nslots = table_size((b - a) * (P.L - 1), 1024, max_slots);
-    for (uint32_t s = threadIdx.x; s < nslots; s += blockDim.x) tab[s] = EMPTY;
-    __syncthreads();
-    bool ok = true;
-    for (int64_t base = a + (threadIdx.x & ~31u); base < b; base += blockDim.x) {   // warp-uniform
-        const int64_t e = base + (threadIdx.x & 31);
-        const bool act = e < b;
-        ok &= insert_path_conv<STRIDE>(P, act ? P.pid[e] : NO_PATH, v, tab, nslots, act);
-    }
-    if (!ok) flag_status(status, ST_HASH_FULL);
-    __syncthreads();
-    cta_select<false>(tab, nslots, lists, o.k, [&](const WarpTopK& t) { write_list(t, o, qi); });
+// ------------------------------------------------------- team tiers ---
+// Queries beyond the lane and group tiers whose table fits in shared memory:
+// a team (one warp, or a whole CTA) counts a query in an open-addressing
+// table of two 32-bit words per slot, key[] (a vertex, or EMPTYK) and ext[]
+// (its occurrences beyond the first, so most slots' ext is never touched),
+// and then ranks its top-k.
+//
+// What bounds it: issue slots and shared-memory latency, not DRAM (warp tier
+// at T = 10: 66% issue active, DRAM at 6%). All vertices, top-10, one GB300:
+// 5M vertices, R = 1e7, T = 5: these three kernels 1.02 ms, where 64-bit
+// slots scanned twice per query took 5.73 (untuned shape; 2.4 tuned); 1M
+// vertices, R = 2e6, T = 10: 2.04 against 12.4 ms. Two things
+// keep the instruction count low. (1) The first probes of all of a path's
+// entries are issued together, as one 32-bit compare-and-swap each (a slot of
+// key and count in one 64-bit word needs a load, a 64-bit CAS and a 64-bit
+// add, which shared memory has only as a CAS loop), and only the few that
+// collide walk on. (2) An entry that is counted the second time lists its
+// slot, so the candidates with a count of 2 or more are known without
+// scanning the table; usually they fill the top-k, and the table (mostly
+// single occurrences) is never read again. Only a query with fewer than k
+// such candidates looks for the smallest ids among the single ones.
+constexpr uint32_t EMPTYK = 0xffffffffu;
+
+__host__ __device__ constexpr int team_items(bool cta) { return cta ? 256 : 128; }   // 64-bit scores ranked at once
+// shared bytes of a team with tables of up to `slots` slots
+__host__ __device__ constexpr size_t team_bytes(bool cta, uint32_t slots) {
+    return (size_t)slots * 8 + (size_t)slots / 2 + (size_t)team_items(cta) * 8 + 32;
 }
 
-template <int STRIDE>
-__device__ void warp_query(const PathsRef& P, int32_t v, int64_t qi, unsigned long long* tab, const OutRef& o,
-                           uint32_t* status) {
-    unsigned lane = threadIdx.x & 31;
-    int64_t a = P.off[v], b = P.off[v + 1];
-    const uint32_t ns = table_size((b - a) * (P.L - 1), 64, WSLOTS);
-    for (uint32_t s = lane; s < ns; s += 32) tab[s] = EMPTY;
-    __syncwarp();
-    bool ok = true;
-    for (int64_t base = a; base < b; base += 32) {                   // warp-uniform trip count
-        const int64_t e = base + lane;
-        const bool act = e < b;
-        ok &= insert_path_conv<STRIDE>(P, act ? P.pid[e] : NO_PATH, v, tab, ns, act);
-    }
-    if (!ok) flag_status(status, ST_HASH_FULL);
-    __syncwarp();
-    WarpTopK t = warp_table_topk(tab, ns, o.k);
-    write_list(t, o, qi);
-    __syncwarp();
+struct TeamMem {
+    uint32_t* key;           // [slots]
+    uint32_t* ext;           // [slots]
+    uint16_t* rep;           // [slots / 4] slots counted at least twice, while they fit
+    unsigned long long* buf; // [team_items] scores to rank; also a 256-bin histogram
+    unsigned* ctr;           // [0] repeated slots, [2..6] scratch
+    uint32_t ns;             // slots of this query
+    uint32_t rep_cap;
+};
+
+template <bool CTA>
+__device__ __forceinline__ TeamMem team_mem(void* base, uint32_t slots) {
+    TeamMem M;
+    M.buf = (unsigned long long*)base;
+    M.ctr = (unsigned*)(M.buf + team_items(CTA));
+    M.key = M.ctr + 8;
+    M.ext = M.key + slots;
+    M.rep = (uint16_t*)(M.ext + slots);
+    M.ns = slots;
+    M.rep_cap = slots / 4;
+    return M;
 }
 
+template <bool CTA>
+__device__ __forceinline__ void team_sync() {
+    if (CTA) __syncthreads(); else __syncwarp();
+}
+template <bool CTA>
+__device__ __forceinline__ int team_rank() { return CTA ? (int)threadIdx.x : (int)(threadIdx.x & 31); }
+template <bool CTA>
+__device__ __forceinline__ int team_size() { return CTA ? (int)blockDim.x : 32; }
 
-// ------------------------------------------------- narrow warp tier ---
-// When every vertex id fits in 32 - cb bits and every warp-tier count in cb
-// bits, a slot is one 32-bit word key << cb | count: half the table, 32-bit
-// atomics, and 32-bit keys to sort.
-constexpr uint32_t EMPTY32 = 0xffffffffu;
+// one more occurrence of the vertex in slot s
+__device__ __forceinline__ void team_bump(const TeamMem& M, uint32_t s) {
+    if (atomicAdd(&M.ext[s], 1u) == 0u) {
+        const unsigned at = atomicAdd(&M.ctr[0], 1u);
+        if (at < M.rep_cap) M.rep[at] = (uint16_t)s;
+    }
+}
 
-__device__ __forceinline__ bool hash_add32_conv(uint32_t* tab, uint32_t nslots, uint32_t key, int cb, bool active) {
-    uint32_t s = active ? hslot(key, nslots) : 0;
-    bool pending = active, ok = true;
-    uint32_t probes = 0;
-    const uint32_t mine_word = (key << cb) | 1u;
-    while (__any_sync(0xffffffffu, pending)) {
-        if (pending) {
-            uint32_t cur = tab[s];
-            bool mine = cur != EMPTY32 && (cur >> cb) == key;
-            if (cur == EMPTY32) {
-                uint32_t prev = atomicCAS(&tab[s], EMPTY32, mine_word);
-                if (prev == EMPTY32) pending = false;
-                else mine = (prev >> cb) == key;
-            }
-            if (mine) {
-                atomicAdd(&tab[s], 1u);
-                pending = false;
-            }
-            if (pending) {
-                s = (s + 1 == nslots) ? 0 : s + 1;
-                if (++probes >= nslots) {
-                    pending = false;
-                    ok = false;
-                }
-            }
+// walk on from slot s (exclusive) until u is counted. Bounded by the table
+// size: a full table clears ok.
+__device__ __forceinline__ void team_probe(const TeamMem& M, uint32_t u, uint32_t s, bool& ok) {
+    for (uint32_t probes = 1; probes < M.ns; ++probes) {
+        s = (s + 1 == M.ns) ? 0 : s + 1;
+        const uint32_t p = atomicCAS(&M.key[s], EMPTYK, u);
+        if (p == EMPTYK) return;
+        if (p == u) {
+            team_bump(M, s);
+            return;
         }
     }
-    return ok;
+    ok = false;
 }
 
+// Shared-memory atomics under a predicate (the result register keeps its value
+// where p is false). Written as predicated instructions: an `if` around each
+// of them costs a divergent branch and a reconvergence per entry.
+__device__ __forceinline__ uint32_t shared_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void cas_if(bool p, uint32_t& r, uint32_t addr, uint32_t cmp, uint32_t val) {
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %1, 0;\n\t@q atom.shared.cas.b32 %0, [%2], %3, %4;\n\t}"
+                 : "+r"(r) : "r"((uint32_t)p), "r"(addr), "r"(cmp), "r"(val) : "memory");
+}
+__device__ __forceinline__ void inc_if(bool p, uint32_t& r, uint32_t addr) {
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %1, 0;\n\t@q atom.shared.add.u32 %0, [%2], 1;\n\t}"
+                 : "+r"(r) : "r"((uint32_t)p), "r"(addr) : "memory");
+}
+
+// Count up to N vertices per lane (u[j] = NO_VERTEX: none). Straight-line for the common case: the first probes
+// are in flight together, then the second probes of those that collided, then
+// the counts of those that met their own key; what still collides (a few
+// lanes) walks on in a loop. An entry's state is what its last probe returned:
+// EMPTYK (claimed, or nothing to count), its own key (to be counted), or
+// another key.
+constexpr uint32_t NO_VERTEX = 0x7fffffffu;            // n < 2^31
+
+template <int N>
+__device__ __forceinline__ void team_place(const TeamMem& M, const uint32_t (&u)[N], bool& ok) {
+    const uint32_t kbase = shared_addr(M.key), xoff = shared_addr(M.ext) - kbase, end = kbase + 4u * M.ns;
+    uint32_t at[N], pr[N], old[N];
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+        pr[j] = EMPTYK;
+        at[j] = kbase + 4u * hslot(u[j], M.ns);
+        cas_if(u[j] != NO_VERTEX, pr[j], at[j], EMPTYK, u[j]);
+    }
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+        const bool col = pr[j] != EMPTYK && pr[j] != u[j];
+        if (col) {
+            at[j] += 4u;
+            at[j] = at[j] == end ? kbase : at[j];
+        }
+        cas_if(col, pr[j], at[j], EMPTYK, u[j]);
+    }
+    unsigned live = 0, first = 0;                      // bit j: still colliding; counted the second time now
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+        const bool own = pr[j] == u[j];
+        old[j] = 1u;
+        inc_if(own, old[j], at[j] + xoff);
+        live |= (!own && pr[j] != EMPTYK) ? 1u << j : 0u;
+    }
+#pragma unroll
+    for (int j = 0; j < N; ++j) first |= old[j] == 0u ? 1u << j : 0u;
+    if (first) {                                       // list the slots
+        unsigned pos = atomicAdd(&M.ctr[0], (unsigned)__popc(first));
+#pragma unroll
+        for (int j = 0; j < N; ++j)
+            if ((first >> j) & 1u) {
+                if (pos < M.rep_cap) M.rep[pos] = (uint16_t)((at[j] - kbase) >> 2);
+                ++pos;
+            }
+    }
+    while (live) {                                     // two collisions in a row: one entry at a time
+        const int jj = __ffs(live) - 1;
+        live &= live - 1;
+        uint32_t w = u[0], a = at[0];
+#pragma unroll
+        for (int q = 1; q < N; ++q) {
+            w = jj == q ? u[q] : w;
+            a = jj == q ? at[q] : a;
+        }
+        team_probe(M, w, (a - kbase) >> 2, ok);
+    }
+    __syncwarp();
+}
+
+// How a warp walks P_v, a round at a time. Rows of up to 32 entries: a lane
+// takes four entries, ceil((T+1)/4) lanes a path. With a whole row per lane a
+// query of fewer than 32 paths (most of the warp tier's) leaves lanes idle,
+// and the unrolled code of 8 to 32 entries, their probes and comparisons,
+// overflows the instruction cache: at T = 10 (1,000,003 vertices, R = 2e6) the
+// warp tier took 2.96 ms that way and 1.46 ms this way, at T = 5 the three
+// kernels 1.21 and 1.10 ms. Rows of 64 or 128: the warp takes 32 paths' ids
+// and walks them one by one (team_insert_long).
 template <int STRIDE>
-__device__ __forceinline__ bool insert_path32(const PathsRef& P, uint32_t r, int32_t v, uint32_t* tab, uint32_t nslots,
-                                              int cb, bool active) {
-    active &= r < (uint64_t)P.R;
-    int32_t x[STRIDE];
-    const int4* src = (const int4*)(P.rows + (uint64_t)(active ? r : 0u) * STRIDE);
-#pragma unroll
-    for (int k = 0; k < STRIDE / 4; ++k) {
-        int4 q = active ? __ldg(src + k) : make_int4(-1, -1, -1, -1);
-        x[4 * k] = q.x; x[4 * k + 1] = q.y; x[4 * k + 2] = q.z; x[4 * k + 3] = q.w;
+struct Walk {
+    static constexpr int XN = 4;                       // entries held per lane
+    int ppr;                                           // paths per round
+    int sub, c4;                                       // this lane's path of the round, its first entry
+    __device__ __forceinline__ Walk(const PathsRef& P) {
+        const int lane = threadIdx.x & 31;
+        if (STRIDE <= 32) {
+            const int lanes = (P.L + 3) >> 2;
+            ppr = 32 / lanes;
+            sub = lane / lanes;
+            c4 = 4 * (lane - sub * lanes);
+            if (sub >= ppr) sub = 1 << 30;             // spare lanes: past any list
+        } else {
+            ppr = 32;
+            sub = lane;
+            c4 = 0;
+        }
     }
-    bool ok = true;
-#pragma unroll
-    for (int j = 0; j < STRIDE; ++j) {
-        bool take = active && j < P.L && x[j] != v;
-#pragma unroll
-        for (int i = 0; i < j; ++i) take &= (x[i] != x[j]);
-        if (__any_sync(0xffffffffu, take)) ok &= hash_add32_conv(tab, nslots, (uint32_t)x[j], cb, take);
+    // this lane's entries of path r (-1 everywhere when r is no path)
+    __device__ __forceinline__ void load(const PathsRef& P, uint32_t r, int32_t (&x)[XN]) const {
+        if constexpr (STRIDE > 32) return;
+        const bool act = r < (uint64_t)P.R;
+        const int4* src = (const int4*)(P.rows + (uint64_t)(act ? r : 0u) * STRIDE + c4);
+        const int4 q = (act && c4 < P.L) ? __ldg(src) : make_int4(-1, -1, -1, -1);
+        x[0] = q.x; x[1] = q.y; x[2] = q.z; x[3] = q.w;
     }
-    return ok;
+    // count the distinct vertices u != v of the round's paths
+    __device__ __forceinline__ void count(const PathsRef& P, const int32_t (&x)[XN], int32_t v, const TeamMem& M,
+                                          bool& ok) const {
+        uint32_t u[XN];
+        bool t[XN];
+#pragma unroll
+        for (int j = 0; j < XN; ++j) {
+            t[j] = x[j] >= 0 && x[j] != v && c4 + j < P.L;
+#pragma unroll
+            for (int i = 0; i < j; ++i) t[j] = t[j] && x[i] != x[j];
+        }
+        for (int d = 4; d < P.L; d += 4) {             // and the path's earlier lanes
+            int32_t y[XN];
+#pragma unroll
+            for (int k = 0; k < XN; ++k) {
+                y[k] = __shfl_up_sync(0xffffffffu, x[k], d >> 2);
+                if (c4 < d) y[k] = -1;
+            }
+#pragma unroll
+            for (int j = 0; j < XN; ++j)
+#pragma unroll
+                for (int k = 0; k < XN; ++k) t[j] = t[j] && x[j] != y[k];
+        }
+#pragma unroll
+        for (int j = 0; j < XN; ++j) u[j] = t[j] ? (uint32_t)x[j] : NO_VERTEX;
+        team_place<XN>(M, u, ok);
+    }
+};
+
+// rows of 64 or 128 entries: the warp takes its lanes' paths one at a time,
+// lane l holding entries l, l+32, ... (as insert_paths_warp)
+template <int STRIDE>
+__device__ __forceinline__ void team_insert_long(const PathsRef& P, uint32_t r, int32_t v, const TeamMem& M,
+                                                     bool& ok) {
+    constexpr int NR = STRIDE / 32;
+    const unsigned lane = threadIdx.x & 31, lt = (1u << lane) - 1u;
+    unsigned pend = __ballot_sync(0xffffffffu, r < (uint64_t)P.R);
+    while (pend) {                                     // warp-uniform
+        const int src = __ffs(pend) - 1;
+        pend &= pend - 1;
+        const uint32_t rr = __shfl_sync(0xffffffffu, r, src);
+        const int32_t* row = P.rows + (uint64_t)rr * STRIDE;
+        int32_t y[NR];
+#pragma unroll
+        for (int m = 0; m < NR; ++m) y[m] = __ldg(row + m * 32 + lane);
+#pragma unroll
+        for (int m = 0; m < NR; ++m) {
+            if (m * 32 >= P.L) break;                  // warp-uniform: the rest is padding
+            bool take = m * 32 + (int)lane < P.L && y[m] >= 0 && y[m] != v;
+            take &= (__match_any_sync(0xffffffffu, y[m]) & lt) == 0;
+#pragma unroll
+            for (int mm = 0; mm < m; ++mm)
+#pragma unroll 8
+                for (int sl = 0; sl < 32; ++sl) take &= __shfl_sync(0xffffffffu, y[mm], sl) != y[m];
+            if (take) {
+                const uint32_t u = (uint32_t)y[m], s = hslot(u, M.ns);
+                const uint32_t p = atomicCAS(&M.key[s], EMPTYK, u);
+                if (p == u) team_bump(M, s);
+                else if (p != EMPTYK) team_probe(M, u, s, ok);
+            }
+            __syncwarp();
+        }
+    }
 }
 
-// sort key of a narrow slot: count high, then ascending id (0 = empty)
-__device__ __forceinline__ uint32_t slot_score32(uint32_t w, int cb) {
-    if (w == EMPTY32) return 0;
-    const uint32_t kb = 32 - cb, kmask = (1u << kb) - 1u;   // 1 <= cb <= 16
-    return ((w & ((1u << cb) - 1u)) << kb) | (kmask - (w >> cb));
-}
-
-__device__ __forceinline__ uint64_t widen_score(uint32_t sc, int cb) {
-    if (!sc) return 0;
-    const uint32_t kb = 32 - cb, kmask = (1u << kb) - 1u;
-    const uint32_t cnt = sc >> kb, id = kmask - (sc & kmask);
+__device__ __forceinline__ uint64_t score_of(uint32_t id, uint32_t cnt) {
     return ((uint64_t)cnt << 32) | (uint64_t)(0xffffffffu - id);
 }
 
-// bitonic sort, descending, of the 64 32-bit keys (a: rank lane, b: rank 32 + lane)
-__device__ __forceinline__ void warp_sort64_desc32(uint32_t& a, uint32_t& b) {
-    const unsigned lane = threadIdx.x & 31;
-#pragma unroll
-    for (int kk = 2; kk <= 64; kk <<= 1) {
-#pragma unroll
-        for (int j = kk >> 1; j > 0; j >>= 1) {
-            if (j == 32) {
-                const bool desc = (lane & kk) == 0;
-                const uint32_t hi = max(a, b), lo = min(a, b);
-                a = desc ? hi : lo;
-                b = desc ? lo : hi;
-            } else {
-                const uint32_t pa = __shfl_xor_sync(0xffffffffu, a, j);
-                const uint32_t pb = __shfl_xor_sync(0xffffffffu, b, j);
-                const bool lower = (lane & j) == 0;
-                const bool da = kk == 64 || (lane & kk) == 0;
-                const bool db = kk == 64 || ((32 + lane) & kk) == 0;
-                a = (lower == da) ? max(a, pa) : min(a, pa);
-                b = (lower == db) ? max(b, pb) : min(b, pb);
+__device__ __forceinline__ void put_rank(const OutRef& o, int64_t qi, unsigned rank, uint32_t id, uint32_t cnt) {
+    const int64_t at = qi * o.k + rank;
+    if (o.ids) o.ids[at] = (int32_t)id;
+    o.cnt[at] = cnt;
+}
+
+// The z distinct scores in buf take ranks rank0, rank0 + 1, ... by comparison;
+// those below rank0 + limit go out. With `idbits` > 0 every score is one
+// 32-bit word (count above the id's complement), else count << 32 | ~id.
+template <bool CTA>
+__device__ __forceinline__ void team_rank_out(const TeamMem& M, unsigned z, unsigned limit, unsigned rank0, int idbits,
+                                              const OutRef& o, int64_t qi) {
+    for (unsigned i = team_rank<CTA>(); i < z; i += team_size<CTA>()) {
+        unsigned rank = 0, j = 0;
+        uint32_t id, cnt;
+        if (idbits) {
+            const uint32_t* b32 = (const uint32_t*)M.buf;
+            const uint32_t s = b32[i], mask = (1u << idbits) - 1u;
+#pragma unroll 1
+            for (; j + 4 <= z; j += 4) {
+                const uint4 q = *(const uint4*)(b32 + j);
+                rank += (q.x > s ? 1u : 0u) + (q.y > s ? 1u : 0u) + (q.z > s ? 1u : 0u) + (q.w > s ? 1u : 0u);
             }
+#pragma unroll 1
+            for (; j < z; ++j) rank += b32[j] > s ? 1u : 0u;
+            id = mask - (s & mask);
+            cnt = s >> idbits;
+        } else {
+            const uint64_t s = M.buf[i];
+#pragma unroll 2
+            for (; j < z; ++j) rank += M.buf[j] > s ? 1u : 0u;
+            id = 0xffffffffu - (uint32_t)s;
+            cnt = (uint32_t)(s >> 32);
         }
+        if (rank < limit) put_rank(o, qi, rank0 + rank, id, cnt);
     }
 }
 
-__device__ __forceinline__ uint32_t warp_sort32_desc32(uint32_t a) {
+__device__ __forceinline__ void put_score(const TeamMem& M, unsigned at, uint32_t id, uint32_t cnt, int idbits) {
+    if (idbits) ((uint32_t*)M.buf)[at] = (cnt << idbits) | (((1u << idbits) - 1u) - id);
+    else M.buf[at] = score_of(id, cnt);
+}
+
+// one-byte monotone code of an id distance: exact below 16, then eight steps
+// per doubling (at most 231 below 2^31), and the smallest distance of a code
+__host__ __device__ __forceinline__ uint32_t dist_code(uint32_t x) {
+    if (x < 16) return x;
+    uint32_t e = 4;
+#ifdef __CUDA_ARCH__
+    e = 31u - (uint32_t)__clz(x);
+#else
+    while ((x >> (e + 1)) != 0) ++e;
+#endif
+    return 8u * (e - 2u) + ((x >> (e - 3u)) & 7u);
+}
+__host__ __device__ __forceinline__ uint32_t dist_floor(uint32_t c) {
+    if (c < 16) return c;
+    return (8u + c % 8u) << (c / 8u - 1u);
+}
+
+// 256-bin histogram in the scratch, scanned by warp 0 in the given direction:
+// finds the bin where the running total first reaches `need` (the last bin
+// with entries if it never does) and publishes {bin, total before it, total
+// with it} in ctr[4..6]. Every thread of the team calls it; ends with a sync.
+template <bool CTA, bool DOWN>
+__device__ __forceinline__ void team_find_bin(const TeamMem& M, unsigned need) {
+    const uint32_t* h = (const uint32_t*)M.buf;
+    team_sync<CTA>();
+    if (!CTA || threadIdx.x < 32) {
+        const unsigned lane = threadIdx.x & 31;
+        uint32_t c[8], sum = 0;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const unsigned b = lane * 8 + i;
+            c[i] = h[DOWN ? 255 - b : b];
+            sum += c[i];
+        }
+        uint32_t inc = sum;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, inc, d);
+            if ((int)lane >= d) inc += y;
+        }
+        const uint32_t total = __shfl_sync(0xffffffffu, inc, 31);
+        const uint32_t want = need < total ? need : total;
+        uint32_t run = inc - sum;
+        if (run < want && want <= inc) {               // one lane
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                if (run < want && want <= run + c[i]) {
+                    const unsigned b = lane * 8 + i;
+                    M.ctr[4] = DOWN ? 255 - b : b;
+                    M.ctr[5] = run;
+                    M.ctr[6] = run + c[i];
+                }
+                run += c[i];
+            }
+        }
+    }
+    team_sync<CTA>();
+}
+
+template <bool CTA>
+__device__ __forceinline__ void team_clear_hist(const TeamMem& M) {
+    uint32_t* h = (uint32_t*)M.buf;
+    team_sync<CTA>();
+    for (int i = team_rank<CTA>(); i < 256; i += team_size<CTA>()) h[i] = 0;
+    if (team_rank<CTA>() == 0) {
+        M.ctr[2] = 0;
+        M.ctr[3] = 0xffffffffu;
+    }
+    team_sync<CTA>();
+}
+
+// bitonic sort of one key per lane, ascending
+__device__ __forceinline__ uint32_t warp_sort32_asc(uint32_t a) {
     const unsigned lane = threadIdx.x & 31;
 #pragma unroll
     for (int kk = 2; kk <= 32; kk <<= 1) {
 #pragma unroll
         for (int j = kk >> 1; j > 0; j >>= 1) {
             const uint32_t pa = __shfl_xor_sync(0xffffffffu, a, j);
-            const bool lower = (lane & j) == 0;
-            const bool da = kk == 32 || (lane & kk) == 0;
-            a = (lower == da) ? max(a, pa) : min(a, pa);
+            const bool lower = (lane & j) == 0, asc = kk == 32 || (lane & kk) == 0;
+            a = (lower == asc) ? min(a, pa) : max(a, pa);
         }
     }
     return a;
 }
 
-// returns false (and does nothing) when the query has 2^cb - 1 or more paths:
-// its counts might not fit, or a slot might read as empty
-template <int STRIDE>
-__device__ bool warp_query32(const PathsRef& P, int32_t v, int64_t qi, uint32_t* tab, const OutRef& o, int cb,
-                             uint32_t* status) {
-    if constexpr (STRIDE > 32) return false;              // long rows: the wide form
-    const unsigned lane = threadIdx.x & 31, lt = (1u << lane) - 1u;
-    const int64_t a = P.off[v], b = P.off[v + 1];
-    if (b - a >= (int64_t(1) << cb) - 1) return false;
-    const uint32_t ns = table_size((b - a) * (P.L - 1), 64, WSLOTS);
-    for (uint32_t s = lane; s < ns; s += 32) tab[s] = EMPTY32;
-    __syncwarp();
-    bool ok = true;
-    for (int64_t base = a; base < b; base += 32) {                   // warp-uniform trip count
-        const int64_t e = base + lane;
-        const bool act = e < b;
-        ok &= insert_path32<STRIDE>(P, act ? P.pid[e] : NO_PATH, v, tab, ns, cb, act);
-    }
-    if (!ok) flag_status(status, ST_HASH_FULL);
-    __syncwarp();
-    // top-k: the slots with count >= c* are compacted in place and sorted
-    // once. c* = 1 when at most 64 slots are filled; otherwise the k-th
-    // largest count, found bit by bit (counts are below 2^cb) by counting the
-    // slots at or above a threshold on a register copy of the table. More
-    // than 64 slots at or above c* (many ties at c*): every slot is offered to
-    // a running list instead.
-    constexpr int NR = WSLOTS / 32;
-    const uint32_t cmask = (1u << cb) - 1u;
-    uint32_t wv[NR];
-#pragma unroll
-    for (int g = 0; g < NR; ++g) wv[g] = (uint32_t)g * 32u < ns ? tab[g * 32 + lane] : EMPTY32;
-    auto at_least = [&](uint32_t c) {
-        int s = 0;
-#pragma unroll
-        for (int g = 0; g < NR; ++g)
-            s += __popc(__ballot_sync(0xffffffffu, wv[g] != EMPTY32 && (wv[g] & cmask) >= c));
-        return s;
+// Candidates with exactly the count `cnt`: the scores of those with the
+// smallest ids go to buf, at least `want` of them (all when there are no more)
+// and at most its capacity. Returns {in buf, the query's candidates with this
+// count up to `want`}. Many candidates are narrowed first. A warp takes the
+// want-th smallest of its lanes' own minima as a bound (an upper bound of the
+// want-th smallest id; few lie below it). Else a histogram of coded distances
+// from the smallest id finds the bin that holds the want-th; while the ids up
+// to that bin do not fit, the search goes on inside the bin (at most an eighth
+// of its distance wide, and one id per bin below 16).
+template <bool CTA>
+__device__ __forceinline__ uint2 team_level(const TeamMem& M, uint32_t cnt, unsigned want, bool counts_only,
+                                            int idbits) {
+    const int t = team_rank<CTA>(), nt = team_size<CTA>();
+    const unsigned room = idbits ? 2 * team_items(CTA) : team_items(CTA);
+    auto each = [&](auto f) {                          // f(id) for this thread's share
+#pragma unroll 1
+        for (unsigned s = 4 * t; s < M.ns; s += 4 * nt) {
+            const uint4 u = *(const uint4*)(M.key + s), x = *(const uint4*)(M.ext + s);
+            if (u.x != EMPTYK && x.x + 1u == cnt) f(u.x);
+            if (u.y != EMPTYK && x.y + 1u == cnt) f(u.y);
+            if (u.z != EMPTYK && x.z + 1u == cnt) f(u.z);
+            if (u.w != EMPTYK && x.w + 1u == cnt) f(u.w);
+        }
     };
-    uint32_t cstar = 1;
-    int filled = at_least(1);
-    if (filled > 64) {
-        cstar = 0;
-        for (int bit = cb - 1; bit >= 0; --bit)                       // warp-uniform
-            if (at_least(cstar | (1u << bit)) >= o.k) cstar |= 1u << bit;
-        filled = at_least(cstar);
-    }
-    WarpTopK t;
-    if (filled > 64) {
-#pragma unroll
-        for (int g = 0; g < NR; ++g)
-            if ((uint32_t)g * 32u < ns) t.offer(widen_score(slot_score32(wv[g], cb), cb), o.k);
-    } else {
-        int pos = 0;
-#pragma unroll
-        for (int g = 0; g < NR; ++g) {
-            const bool pass = wv[g] != EMPTY32 && (wv[g] & cmask) >= cstar;
-            const unsigned m = __ballot_sync(0xffffffffu, pass);
-            if (pass) tab[pos + __popc(m & lt)] = slot_score32(wv[g], cb);   // the table is in registers
-            pos += __popc(m);
-        }
-        __syncwarp();
-        uint32_t ka = lane < (unsigned)filled ? tab[lane] : 0u;
-        uint32_t kb2 = 32 + lane < (unsigned)filled ? tab[32 + lane] : 0u;
-        if (filled <= 32) {
-            ka = warp_sort32_desc32(ka);
-            kb2 = 0;
-        } else {
-            warp_sort64_desc32(ka, kb2);
-        }
-        t.a = widen_score(ka, cb);
-        t.b = widen_score(kb2, cb);
-    }
-    write_list(t, o, qi);
+    uint32_t mn = 0x7fffffffu, lo = 0, hi = 0x7fffffffu;
+    unsigned e = 0;
+    each([&](uint32_t id) {
+        mn = min(mn, id);
+        ++e;
+    });
     __syncwarp();
-    return true;
+    e = __reduce_add_sync(0xffffffffu, e);
+    if (CTA) {
+        __syncthreads();
+        if (t == 0) M.ctr[2] = 0;
+        __syncthreads();
+        if ((t & 31) == 0) atomicAdd(&M.ctr[2], e);
+        __syncthreads();
+        e = M.ctr[2];
+    }
+    const unsigned r = min(want, e);
+    if (r == 0 || counts_only) return make_uint2(0u, r);
+    bool refine = e > 64;
+    if (!CTA && e > 24 && r <= 32) {
+        hi = __shfl_sync(0xffffffffu, warp_sort32_asc(mn), r - 1);
+        refine = false;
+    }
+    unsigned z;
+#pragma unroll 1
+    for (;;) {
+        if (refine) {
+            unsigned before = 0;                       // members below lo: fewer than r, all taken
+            hi = 0x7fffffffu;
+#pragma unroll 1
+            for (;;) {
+                team_clear_hist<CTA>(M);
+                mn = 0xffffffffu;
+                each([&](uint32_t id) { mn = (id >= lo && id <= hi) ? min(mn, id) : mn; });
+                __syncwarp();
+                mn = __reduce_min_sync(0xffffffffu, mn);
+                if (CTA) {
+                    if ((t & 31) == 0) atomicMin(&M.ctr[3], mn);
+                    __syncthreads();
+                    mn = M.ctr[3];
+                }
+                each([&](uint32_t id) {
+                    if (id >= lo && id <= hi) atomicAdd((uint32_t*)M.buf + dist_code(id - mn), 1u);
+                });
+                __syncwarp();
+                team_find_bin<CTA, false>(M, r - before);
+                const uint32_t b = M.ctr[4];
+                z = before + M.ctr[6];
+                before += M.ctr[5];
+                hi = min(hi, mn + dist_floor(b + 1) - 1u);
+                lo = mn + dist_floor(b);
+                if (z <= room) break;
+            }
+        }
+        team_sync<CTA>();
+        if (t == 0) M.ctr[2] = 0;
+        team_sync<CTA>();
+        each([&](uint32_t id) {
+            if (id <= hi) {
+                const unsigned at = atomicAdd(&M.ctr[2], 1u);
+                if (at < room) put_score(M, at, id, cnt, idbits);
+            }
+        });
+        team_sync<CTA>();
+        z = M.ctr[2];
+        if (z <= room || refine) break;
+        refine = true;                                 // the lanes' minima were no good bound
+        team_sync<CTA>();
+    }
+    return make_uint2(min(z, room), r);
 }
 
-struct PersistArgs {
+// The counted table's top-k by (count desc, id asc) -> row qi of the output.
+// Every thread of the team calls it with the counting finished (synchronised).
+// Step 0 ranks the candidates counted at least twice, or those above a count
+// that too many share; step 1 adds the smallest ids at that count (1, when
+// fewer than k were counted twice).
+template <bool CTA>
+__device__ __forceinline__ void team_select(const TeamMem& M, const OutRef& o, int64_t qi, int idbits) {
+    const unsigned k = (unsigned)o.k, m = M.ctr[0], items = team_items(CTA);
+    const int t = team_rank<CTA>(), nt = team_size<CTA>();
+    unsigned done = 0, level = 1;
+#pragma unroll 1
+    for (int step = 0; step < 2; ++step) {
+        unsigned z = 0, take = 0;
+        if (step == 1) {
+            const uint2 got = team_level<CTA>(M, level, k - done, o.ids == nullptr, idbits);
+            z = got.x;
+            take = got.y;
+            if (!o.ids)                                // counts only: no ids to rank
+                for (unsigned i = t; i < take; i += nt) o.cnt[qi * o.k + done + i] = level;
+        } else if (m <= M.rep_cap && (m <= 64u || (m <= k && m <= items))) {
+            for (unsigned i = t; i < m; i += nt) {     // few: the list itself
+                const unsigned s = M.rep[i];
+                put_score(M, i, M.key[s], M.ext[s] + 1u, idbits);
+            }
+            z = m;
+            take = min(m, k);
+        } else {
+            // f(id, count) for this thread's share of the candidates counted
+            // at least twice: the list, or the table when the list overflowed
+            auto each_rep = [&](auto f) {
+                const bool listed = m <= M.rep_cap;
+                const unsigned cnt = listed ? m : M.ns;
+#pragma unroll 1
+                for (unsigned i = t; i < cnt; i += nt) {
+                    const unsigned s = listed ? (unsigned)M.rep[i] : i;
+                    const uint32_t u = M.key[s], x = M.ext[s];
+                    if (u != EMPTYK && x) f(u, x + 1u);
+                }
+            };
+            team_clear_hist<CTA>(M);
+            each_rep([&](uint32_t, uint32_t c) { atomicAdd((uint32_t*)M.buf + path_code(c), 1u); });
+            __syncwarp();
+            team_find_bin<CTA, true>(M, k);
+            const uint32_t b = M.ctr[4];
+            const unsigned above = M.ctr[5], upto = M.ctr[6];   // above bin b (fewer than k), and with it
+            if (b >= 128u && upto > items) {
+                // a coded bin of large counts holds more than the buffer: one rank at a time
+                if (!CTA || threadIdx.x < 32) {
+                    const unsigned lane = threadIdx.x & 31;
+                    uint64_t last = ~0ull;
+                    for (unsigned rk = 0; rk < k; ++rk) {
+                        uint64_t best = 0;
+                        for (unsigned s = lane; s < M.ns; s += 32) {
+                            const uint32_t u = M.key[s], x = M.ext[s];
+                            const uint64_t sc = (u != EMPTYK && x) ? score_of(u, x + 1u) : 0ull;
+                            best = (sc < last && sc > best) ? sc : best;
+                        }
+#pragma unroll
+                        for (int d = 16; d; d >>= 1) best = umax64(best, __shfl_xor_sync(0xffffffffu, best, d));
+                        if (lane == 0) put_rank(o, qi, rk, 0xffffffffu - (uint32_t)best, (uint32_t)(best >> 32));
+                        last = best;
+                    }
+                }
+                done = k;                              // more than k candidates here
+                break;
+            }
+            // all of bin b with those above it, or (many share the count b) only those above
+            const bool split = b < 128u && upto > 64u;
+            const uint32_t from = split ? b + 1 : b;
+            if (split) level = b;
+            team_clear_hist<CTA>(M);
+            each_rep([&](uint32_t id, uint32_t c) {
+                if (path_code(c) >= from) {
+                    const unsigned at = atomicAdd(&M.ctr[2], 1u);
+                    if (at < items) put_score(M, at, id, c, idbits);
+                }
+            });
+            z = split ? above : upto;
+            take = min(z, k);
+        }
+        team_sync<CTA>();
+        team_rank_out<CTA>(M, z, take, done, idbits, o, qi);
+        done += take;
+        if (done >= k) break;
+        team_sync<CTA>();
+    }
+    for (unsigned i = done + t; i < k; i += nt) put_rank(o, qi, i, 0xffffffffu, 0u);
+}
+
+// the table of a query with np paths, emptied
+template <bool CTA>
+__device__ __forceinline__ void team_clear(const PathsRef& P, int64_t np, TeamMem& M, uint32_t max_slots) {
+    const int t = team_rank<CTA>(), nt = team_size<CTA>();
+    int64_t cap = np * (P.L - 1);
+    if (cap > P.n - 1) cap = P.n - 1;
+    M.ns = table_size(cap, 64, max_slots);
+    const int4 e4 = make_int4(-1, -1, -1, -1), z4 = make_int4(0, 0, 0, 0);
+    for (uint32_t i = t; i < M.ns / 4; i += nt) {
+        ((int4*)M.key)[i] = e4;
+        ((int4*)M.ext)[i] = z4;
+    }
+    if (t == 0) M.ctr[0] = 0;
+}
+
+// the counts are complete: rank and write the row
+template <bool CTA>
+__device__ __forceinline__ void team_finish(const PathsRef& P, int64_t np, const TeamMem& M, bool ok, const OutRef& o,
+                                            int64_t qi, uint32_t* status) {
+    if (!ok) flag_status(status, ST_HASH_FULL);
+    team_sync<CTA>();
+    // a count never exceeds np: with the id it fits 32 bits when there is room above the id bits
+    const int idbits = 32 - __clz((int)(P.n - 1) | 1);
+    team_select<CTA>(M, o, qi, (np >> (32 - idbits)) == 0 ? idbits : 0);
+    team_sync<CTA>();
+}
+
+// count one query (paths [a, b) of the index) with a CTA and write its row
+template <int STRIDE>
+__device__ __forceinline__ void cta_query(const PathsRef& P, int32_t v, int64_t qi, int64_t a, int64_t b, TeamMem M,
+                                          uint32_t max_slots, const OutRef& o, uint32_t* status) {
+    const Walk<STRIDE> W(P);
+    team_clear<true>(P, b - a, M, max_slots);
+    // this warp's rounds: the ids of the round after next and the rows of the
+    // next one are loaded while a round is counted
+    const int64_t first = a + (int64_t)(threadIdx.x >> 5) * W.ppr, step = (int64_t)(blockDim.x >> 5) * W.ppr;
+    uint32_t r0 = first + W.sub < b ? P.pid[first + W.sub] : NO_PATH;
+    uint32_t r1 = first + step + W.sub < b ? P.pid[first + step + W.sub] : NO_PATH;
+    bool ok = true;
+    int32_t x[Walk<STRIDE>::XN], y[Walk<STRIDE>::XN];
+    W.load(P, r0, x);
+    __syncthreads();
+    for (int64_t base = first; base < b; base += step) {
+        const int64_t e2 = base + 2 * step + W.sub;
+        const uint32_t r2 = e2 < b ? P.pid[e2] : NO_PATH;
+        if constexpr (STRIDE > 32) {
+            team_insert_long<STRIDE>(P, r0, v, M, ok);
+            r0 = r1;
+        } else {
+            W.load(P, r1, y);
+            W.count(P, x, v, M, ok);
+#pragma unroll
+            for (int j = 0; j < Walk<STRIDE>::XN; ++j) x[j] = y[j];
+        }
+        r1 = r2;
+    }
+    team_finish<true>(P, b - a, M, ok, o, qi, status);
+}
+
+// What a query needs: 1 a team with a table of up to `ccap` candidates, 7 the
+// pass with the largest tables, 2 the hub tier, 0 nothing (no candidates),
+// -1 not a vertex
+__device__ __forceinline__ int query_tier(const PathsRef& P, int64_t v, int64_t ccap, int64_t ccap_big, int64_t* a,
+                                          int64_t* b) {
+    if (v < 0 || v >= P.n) return -1;
+    *a = P.off[v];
+    *b = P.off[v + 1];
+    const int64_t np = *b - *a, cap = min(np * (P.L - 1), P.n - 1);
+    if (cap <= 0) return 0;
+    if (np > CTA_MAX_NP || cap > ccap_big) return 2;
+    return cap <= ccap && np <= MID_MAX_NP ? 1 : 7;
+}
+
+struct TeamArgs {
     PathsRef P;
     const int32_t* queries;
-    Tiers tiers;
+    const int32_t* list;     // query indices of this tier
+    const int* count;        // their number
+    int* fetch;              // next one to take
     OutRef o;
-    uint32_t cta_slots;
+    uint32_t slots;          // largest table
     uint32_t* status;
-    int narrow_cb;   // > 0: warp tier on 32-bit slots with this many count bits
 };
 
+// one warp per query, up to 16 queries per fetch (fewer when the list is
+// short: every warp gets some); lane j reads query j's vertex and path range
 template <int STRIDE>
-__global__ void __launch_bounds__(1024, 1) persistent_kernel(PersistArgs A) {
-    extern __shared__ unsigned long long smem[];
-    unsigned long long* lists = smem + A.cta_slots;     // 64 entries per warp after the table
-    __shared__ int s_item;
-    const int nC = A.tiers.count[1], nW = A.tiers.count[0];
-    // CTA tier first: the largest items, one query per fetch
-    for (;;) {
-        if (threadIdx.x == 0) s_item = atomicAdd(&A.tiers.count[4], 1);
-        __syncthreads();
-        int it = s_item;
-        __syncthreads();
-        if (it >= nC) break;
-        int64_t qi = A.tiers.list[1][it];
-        int32_t v = A.queries ? A.queries[qi] : (int32_t)qi;
-        cta_query<STRIDE>(A.P, v, qi, smem, A.cta_slots, lists, A.o, A.status);
-    }
-    // warp tier, WCHUNK queries per fetch
-    unsigned lane = threadIdx.x & 31;
-    unsigned long long* wt = smem + (threadIdx.x >> 5) * WSLOTS;
+__global__ void __launch_bounds__(128) warp_tier_kernel(TeamArgs A) {
+    extern __shared__ __align__(16) unsigned char tsm[];
+    TeamMem M = team_mem<false>(tsm + (threadIdx.x >> 5) * team_bytes(false, A.slots), A.slots);
+    const unsigned lane = threadIdx.x & 31;
+    const Walk<STRIDE> W(A.P);
+    const int n = *A.count;
+    const int warps = (int)(gridDim.x * (blockDim.x >> 5));
+    const int chunk = max(1, min(16, n / (4 * warps)));
     for (;;) {
         int it = 0;
-        if (lane == 0) it = atomicAdd(&A.tiers.count[3], WCHUNK);
+        if (lane == 0) it = atomicAdd(A.fetch, chunk);
         it = __shfl_sync(0xffffffffu, it, 0);
-        if (it >= nW) break;
-        int end = it + WCHUNK < nW ? it + WCHUNK : nW;
-        for (int j = it; j < end; ++j) {
-            int64_t qi = A.tiers.list[0][j];
-            int32_t v = A.queries ? A.queries[qi] : (int32_t)qi;
-            if (!A.narrow_cb || !warp_query32<STRIDE>(A.P, v, qi, (uint32_t*)wt, A.o, A.narrow_cb, A.status))
-                warp_query<STRIDE>(A.P, v, qi, wt, A.o, A.status);
+        if (it >= n) break;
+        const int cnt = min(chunk, n - it);
+        int32_t mq = 0, mv = 0;
+        int64_t ma = 0, mb = 0;
+        if ((int)lane < cnt) {
+            mq = A.list[it + lane];
+            mv = A.queries ? A.queries[mq] : mq;
+            ma = A.P.off[mv];
+            mb = A.P.off[mv + 1];
         }
+        // The chunk's rounds of paths, query after query: the ids of the
+        // round after next and the rows of the next one are loaded while a
+        // round is counted, across the border of two queries too (most
+        // queries have a single round).
+        int jn = 0;                                    // the round the next ids are loaded for
+        int64_t pn = __shfl_sync(0xffffffffu, ma, 0), en = __shfl_sync(0xffffffffu, mb, 0);
+        auto next_ids = [&]() {
+            const uint32_t r = pn + W.sub < en ? A.P.pid[pn + W.sub] : NO_PATH;
+            pn += W.ppr;
+            if (pn >= en && jn < cnt) {                // warp-uniform
+                ++jn;
+                const int jj = jn < cnt ? jn : 0;
+                pn = __shfl_sync(0xffffffffu, ma, jj);
+                en = jn < cnt ? __shfl_sync(0xffffffffu, mb, jj) : pn;
+            }
+            return r;
+        };
+        int32_t x[Walk<STRIDE>::XN], y[Walk<STRIDE>::XN];
+        uint32_t r0 = next_ids(), r1 = next_ids();
+        W.load(A.P, r0, x);
+        for (int j = 0; j < cnt; ++j) {
+            const int64_t qi = __shfl_sync(0xffffffffu, mq, j);
+            const int32_t v = __shfl_sync(0xffffffffu, mv, j);
+            const int64_t np = __shfl_sync(0xffffffffu, mb - ma, j);
+            team_clear<false>(A.P, np, M, A.slots);
+            __syncwarp();
+            bool ok = true;
+            for (int64_t i = 0; i < np; i += W.ppr) {
+                const uint32_t r2 = next_ids();
+                if constexpr (STRIDE > 32) {
+                    team_insert_long<STRIDE>(A.P, r0, v, M, ok);
+                    r0 = r1;
+                } else {
+                    W.load(A.P, r1, y);
+                    W.count(A.P, x, v, M, ok);
+#pragma unroll
+                    for (int c = 0; c < Walk<STRIDE>::XN; ++c) x[c] = y[c];
+                }
+                r1 = r2;
+            }
+            team_finish<false>(A.P, np, M, ok, A.o, qi, A.status);
+        }
+    }
+}
+
+// one CTA per query; thread 0 fetches the next query while the current one is counted
+// (MAXT: the largest CTA it is launched with, 512 unless the caller's shape asks for 1,024)
+template <int STRIDE, int MAXT>
+__global__ void __launch_bounds__(MAXT) cta_tier_kernel(TeamArgs A) {
+    extern __shared__ __align__(16) unsigned char tsm[];
+    const TeamMem M = team_mem<true>(tsm, A.slots);
+    __shared__ int s_it;
+    __shared__ int32_t s_q, s_v;
+    __shared__ int64_t s_a, s_b;
+    const int n = *A.count;
+    if (threadIdx.x == 0) s_it = atomicAdd(A.fetch, 1);
+    for (;;) {
+        if (threadIdx.x == 0 && s_it < n) {
+            s_q = A.list[s_it];
+            s_v = A.queries ? A.queries[s_q] : s_q;
+            s_a = A.P.off[s_v];
+            s_b = A.P.off[s_v + 1];
+        }
+        __syncthreads();
+        if (s_it >= n) break;
+        const int64_t qi = s_q, a = s_a, b = s_b;
+        const int32_t v = s_v;
+        int next = 0;
+        if (threadIdx.x == 0) next = atomicAdd(A.fetch, 1);
+        cta_query<STRIDE>(A.P, v, qi, a, b, M, A.slots, A.o, A.status);
+        if (threadIdx.x == 0) s_it = next;             // every thread has read the shared values: cta_query ends with a barrier
     }
 }
 
@@ -1297,8 +1747,8 @@ __global__ void __launch_bounds__(1024, 1) persistent_kernel(PersistArgs A) {
 template <int STRIDE>
 __global__ void __launch_bounds__(1024, 1) single_kernel(PathsRef P, const int32_t* __restrict__ queries, int64_t qi, OutRef o,
                               uint32_t cta_slots, unsigned long long* gtab, uint32_t gslots, uint32_t* status) {
-    extern __shared__ unsigned long long smem[];
-    unsigned long long* lists = smem + cta_slots;       // 64 entries per warp after the table
+    extern __shared__ __align__(16) unsigned char tsm[];
+    unsigned long long* lists = (unsigned long long*)tsm;   // 64 entries per warp (global table only)
     int64_t v = queries ? queries[qi] : qi;
     if (v < 0 || v >= P.n) {
         if (threadIdx.x == 0) flag_status(status, ST_BAD_QUERY);
@@ -1311,7 +1761,8 @@ __global__ void __launch_bounds__(1024, 1) single_kernel(PathsRef P, const int32
     int64_t np = P.off[v + 1] - P.off[v];
     int64_t cap = np * (P.L - 1);
     if (cap * 10 <= (int64_t)cta_slots * 7) {
-        cta_query<STRIDE>(P, (int32_t)v, qi, smem, cta_slots, lists, o, status);
+        cta_query<STRIDE>(P, (int32_t)v, qi, P.off[v], P.off[v + 1], team_mem<true>(tsm, cta_slots), cta_slots, o,
+                          status);
         return;
     }
     // global table: gtab is EMPTY on entry and left EMPTY on exit
@@ -1348,6 +1799,39 @@ __global__ void __launch_bounds__(1024, 1) single_kernel(PathsRef P, const int32
 }
 
 // ------------------------------------------------------- global tier ---
+// Small batches: one CTA per query in one launch, without the classification
+// and the other tiers (whose launches cost more than the work): a query is
+// answered, padded, or listed for the pass with the largest tables or the hubs.
+// counts as in Tiers: [1] answered here, [2] hubs, [10] largest tables.
+template <int STRIDE>
+__global__ void __launch_bounds__(512) small_batch_kernel(PathsRef P, const int32_t* __restrict__ queries, int64_t q,
+                                                          int64_t ccap, int64_t ccap_big, uint32_t slots,
+                                                          int32_t* __restrict__ hubs, int32_t* __restrict__ bigs,
+                                                          int* __restrict__ counts, OutRef o, uint32_t* status) {
+    extern __shared__ __align__(16) unsigned char tsm[];
+    const TeamMem M = team_mem<true>(tsm, slots);
+    for (int64_t i = blockIdx.x; i < q; i += gridDim.x) {
+        const int64_t v = queries ? (int64_t)queries[i] : i;
+        int64_t a = 0, b = 0;
+        const int tier = query_tier(P, v, ccap, ccap_big, &a, &b);      // the same for every thread
+        if (tier == 1) {
+            if (threadIdx.x == 0) atomicAdd(&counts[1], 1);
+            cta_query<STRIDE>(P, (int32_t)v, i, a, b, M, slots, o, status);
+            continue;
+        }
+        if (threadIdx.x == 0) {
+            if (tier == 2) hubs[atomicAdd(&counts[2], 1)] = (int32_t)i;
+            else if (tier == 7) bigs[atomicAdd(&counts[10], 1)] = (int32_t)i;
+            else if (tier < 0) {
+                flag_status(status, ST_BAD_QUERY);
+                atomicMin(status + 1, (uint32_t)i);
+            }
+        }
+        if (tier <= 0)
+            for (unsigned r = threadIdx.x; r < (unsigned)o.k; r += blockDim.x) put_rank(o, i, r, 0xffffffffu, 0u);
+    }
+}
+
 struct GPlan {
     const int32_t* qidx;      // [ng] query index of each global query in this round
     const int64_t* tab_off;   // [ng] first slot of its table in the arena
@@ -1396,38 +1880,6 @@ __global__ void g_count_kernel(PathsRef P, const int32_t* __restrict__ queries, 
     if (!ok) flag_status(status, ST_HASH_FULL);
 }
 
-// 64 < k <= 128 sends every query of the batch to device tables; queries of
-// at most WARP_NP paths are counted by one warp each instead of a CTA per
-// 512 paths
-constexpr int64_t WARP_NP = 2048;
-
-template <int STRIDE>
-__global__ void __launch_bounds__(256) g_count_warp_kernel(PathsRef P, const int32_t* __restrict__ queries, GPlan G,
-                                                           unsigned long long* arena, uint32_t* status) {
-    const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (gw >= G.ng) return;                           // warp-uniform
-    const int g = (int)gw;
-    const int64_t qi = G.qidx[g];
-    const int32_t v = queries ? queries[qi] : (int32_t)qi;
-    const int64_t a = P.off[v], b = P.off[v + 1];
-    if (b - a > WARP_NP) return;                      // counted by g_count_kernel
-    unsigned long long* tab = arena + G.tab_off[g];
-    const uint32_t ns = G.tab_n[g];
-    const uint32_t thr = G.thr ? G.thr[g] : 0;
-    const unsigned lane = threadIdx.x & 31;
-    bool ok = true;
-    if constexpr (STRIDE > 32) {
-        for (int64_t base = a; base < b; base += 32) {            // warp-uniform
-            const int64_t e = base + lane;
-            const bool act = e < b;
-            ok &= insert_paths_warp<STRIDE>(P, act ? P.pid[e] : NO_PATH, v, tab, ns, act, thr);
-        }
-    } else {
-        for (int64_t e = a + lane; e < b; e += 32) ok &= insert_path<STRIDE, false>(P, P.pid[e], v, tab, ns, thr);
-    }
-    if (!ok) flag_status(status, ST_HASH_FULL);
-}
-
 // partial top-k of one chunk of one table; empties the slots it read
 __global__ void __launch_bounds__(512) g_select_kernel(GPlan G, unsigned long long* arena, int k,
                                                        unsigned long long* partial) {
@@ -1459,41 +1911,7 @@ __global__ void __launch_bounds__(256) g_merge_cta_kernel(GPlan G, const unsigne
     if (w == 0) write_list(t, o, G.qidx[g]);
 }
 
-__global__ void g_merge_kernel(GPlan G, const unsigned long long* __restrict__ partial, OutRef o) {
-    int g = blockIdx.x;
-    if (g >= G.ng || threadIdx.x >= 32) return;
-    WarpTopK t;
-    unsigned lane = threadIdx.x;
-    for (int64_t it = G.sel_off[g]; it < G.sel_off[g + 1]; ++it) {
-        t.offer(partial[it * KMAX + lane], o.k);
-        if (o.k > 32) t.offer(partial[it * KMAX + 32 + lane], o.k);
-    }
-    write_list(t, o, G.qidx[g]);
-}
-
-// 64 < k <= 128: tables of at most SMALL4 slots are selected whole by one
-// warp (most queries of a batch: their tables are sized to twice their
-// candidate bound, from 64 slots); larger ones in chunks (partial 128-lists),
-// then one merge per query
-constexpr uint32_t SMALL4 = 2048;
-
-__global__ void __launch_bounds__(256) g_small4_kernel(GPlan G, unsigned long long* arena, OutRef o) {
-    const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (gw >= G.ng) return;                           // warp-uniform
-    const int g = (int)gw;
-    const uint32_t ns = G.tab_n[g];
-    if (ns > SMALL4) return;
-    unsigned long long* tab = arena + G.tab_off[g];
-    const unsigned lane = threadIdx.x & 31;
-    WarpTopK4 t;
-    for (uint32_t base = 0; base < ns; base += 32) {  // ns is a power of two >= 64
-        uint64_t sc = slot_score(tab[base + lane]);
-        if (sc) tab[base + lane] = EMPTY;
-        t.offer(sc, o.k);
-    }
-    write_list4(t, o, G.qidx[g]);
-}
-
+// 64 < k <= 128: partial 128-lists per chunk of a table, then one merge per query
 __global__ void __launch_bounds__(512) g_select4_kernel(GPlan G, unsigned long long* arena, int k,
                                                         unsigned long long* partial) {
     __shared__ unsigned long long lists[16 * KMAX4];
@@ -1525,7 +1943,6 @@ __global__ void __launch_bounds__(256) g_merge4_kernel(GPlan G, const unsigned l
                                                        OutRef o) {
     __shared__ unsigned long long lists[8 * KMAX4];
     const int g = blockIdx.x;
-    if (G.tab_n[g] <= SMALL4) return;                 // answered by g_small4_kernel
     const int w = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const unsigned lane = threadIdx.x & 31;
     WarpTopK4 t;
@@ -1716,7 +2133,10 @@ static void launch_lane(bool narrow, bool l6, bool k12, unsigned blocks, cudaStr
 // ------------------------------------------------------------ host side ---
 constexpr int BIG_T = 512;
 constexpr uint32_t BIG_SLOTS = 24576;
-constexpr size_t BIG_SMEM = (size_t)BIG_SLOTS * 8 + (size_t)(BIG_T / 32) * KMAX * 8;
+constexpr size_t BIG_SMEM = team_bytes(true, BIG_SLOTS);
+constexpr int WARP_T = 128;      // threads of a warp-tier CTA (one query per warp)
+constexpr size_t WARP_SMEM = (size_t)(WARP_T / 32) * team_bytes(false, WSLOTS);
+static_assert(WARP_SMEM <= 48 * 1024, "the warp tier needs no shared-memory attribute");
 
 struct TopkShape {
     int threads;
@@ -1726,20 +2146,66 @@ struct TopkShape {
 
 static TopkShape topk_shape(panther_ctx* ctx) {
     TopkShape s;
-    s.threads = ctx->topk_threads ? ctx->topk_threads : 1024;
-    s.cta_slots = ctx->topk_cta_slots ? (uint32_t)ctx->topk_cta_slots : 24576;
-    s.blocks_per_sm = ctx->topk_blocks_per_sm ? ctx->topk_blocks_per_sm : 1;
-    // warp tables must fit in the same dynamic area
-    uint32_t need = (uint32_t)(s.threads / 32) * WSLOTS;
-    if (s.cta_slots < need) s.cta_slots = need;
+    s.threads = ctx->topk_threads ? ctx->topk_threads : 128;
+    s.cta_slots = ctx->topk_cta_slots ? (uint32_t)ctx->topk_cta_slots : 3840;
+    s.blocks_per_sm = ctx->topk_blocks_per_sm ? ctx->topk_blocks_per_sm : 6;
     return s;
 }
 
+// The shared-memory attribute of the CTA kernels (room for the largest table)
+// applies to the current device only: it is set once per device (bit `device`
+// of the mask). Contexts on several host threads (the serving workers) may get
+// here together; setting it twice is harmless.
 template <int STRIDE>
-static panther_status set_smem_attr(panther_ctx* ctx, size_t bytes) {
-    PCK(ctx, cudaFuncSetAttribute(persistent_kernel<STRIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
-    PCK(ctx, cudaFuncSetAttribute(single_kernel<STRIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+static panther_status set_smem_attr(panther_ctx* ctx) {
+    static std::atomic<uint64_t> done{0};
+    const uint64_t bit = ctx->device < 64 ? (uint64_t(1) << ctx->device) : 0;
+    if (bit && (done.load(std::memory_order_acquire) & bit)) return PANTHER_OK;
+    PCK(ctx, cudaFuncSetAttribute(cta_tier_kernel<STRIDE, 512>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BIG_SMEM));
+    PCK(ctx, cudaFuncSetAttribute(cta_tier_kernel<STRIDE, 1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BIG_SMEM));
+    PCK(ctx, cudaFuncSetAttribute(small_batch_kernel<STRIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BIG_SMEM));
+    PCK(ctx, cudaFuncSetAttribute(single_kernel<STRIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BIG_SMEM));
+    done.fetch_or(bit, std::memory_order_acq_rel);
     return PANTHER_OK;
+}
+
+// small_batch_kernel up to this many queries (k <= 64, k > 64). 1M vertices,
+// T = 5, one-launch form against the tiers: R = 33,123, k = 5: 76 / 106 us for
+// 16 queries, 100 / 130 for 4,000, 136 / 155 for 16,000, 261 / 154 for 64,000;
+// R = 2e6, k = 10: 97 / 134, 282 / 330, 479 / 479, 1,192 / 1,057 us.
+constexpr int64_t SMALL_Q = 16384, SMALL_Q_WIDE = 1024;
+
+template <int STRIDE>
+static void launch_small(panther_ctx* ctx, const PathsRef& P, const int32_t* queries, int64_t q, const Tiers& tiers,
+                         const OutRef& o, const TopkShape& sh, int64_t ccap, int64_t ccap_big) {
+    cudaStream_t s = ctx->stream;
+    int* c = tiers.count;
+    const unsigned blocks = (unsigned)std::min<int64_t>(q, (int64_t)ctx->num_sms * sh.blocks_per_sm);
+    const int threads = std::min(sh.threads, 512);
+    small_batch_kernel<STRIDE><<<blocks, threads, team_bytes(true, sh.cta_slots), s>>>(
+        P, queries, q, ccap, ccap_big, sh.cta_slots, tiers.list[2], tiers.list[7], c, o, ctx->d_status);
+    const TeamArgs big{P, queries, tiers.list[7], c + 10, c + 13, o, BIG_SLOTS, ctx->d_status};
+    cta_tier_kernel<STRIDE, 512><<<(unsigned)std::min<int64_t>(q, ctx->num_sms), BIG_T, BIG_SMEM, s>>>(big);
+    ctx->launches += 2;
+}
+
+// the warp tier, the CTA tier at the context's shape and the pass with the
+// largest tables (their lists: tiers 0, 1 and 7)
+template <int STRIDE>
+static void launch_teams(panther_ctx* ctx, const PathsRef& P, const int32_t* queries, const Tiers& tiers,
+                         const OutRef& o, const TopkShape& sh) {
+    cudaStream_t s = ctx->stream;
+    int* c = tiers.count;
+    const TeamArgs big{P, queries, tiers.list[7], c + 10, c + 13, o, BIG_SLOTS, ctx->d_status};
+    cta_tier_kernel<STRIDE, 512><<<(unsigned)ctx->num_sms, BIG_T, BIG_SMEM, s>>>(big);
+    const TeamArgs mid{P, queries, tiers.list[1], c + 1, c + 4, o, sh.cta_slots, ctx->d_status};
+    const unsigned blocks = (unsigned)(ctx->num_sms * sh.blocks_per_sm);
+    const size_t smem = team_bytes(true, sh.cta_slots);
+    if (sh.threads <= 512) cta_tier_kernel<STRIDE, 512><<<blocks, sh.threads, smem, s>>>(mid);
+    else cta_tier_kernel<STRIDE, 1024><<<blocks, sh.threads, smem, s>>>(mid);
+    const TeamArgs wrp{P, queries, tiers.list[0], c, c + 3, o, WSLOTS, ctx->d_status};
+    warp_tier_kernel<STRIDE><<<(unsigned)(ctx->num_sms * 5), WARP_T, WARP_SMEM, s>>>(wrp);
+    ctx->launches += 3;
 }
 
 struct HubQuery {
@@ -1898,8 +2364,7 @@ static panther_status hub_tables(panther_ctx* ctx, const PathsRef& P, const int3
         int64_t used = 0;
         while (pos < hubs.size()) {
             const HubQuery& h = hubs[pos];
-            // k > 64 sends every query here: small ones get small tables
-            uint32_t slots = table_slots(hub_bound(P, h, above), k > KMAX ? 64u : 1024u);
+            uint32_t slots = table_slots(hub_bound(P, h, above), 1024u);
             if (!rq.empty() && used + slots > budget_slots) break;
             rq.push_back(h.qi);
             rt.push_back(h.thr);
@@ -1907,8 +2372,8 @@ static panther_status hub_tables(panther_ctx* ctx, const PathsRef& P, const int3
             roff.push_back(used);
             rn.push_back(slots);
             used += slots;
-            ioff.push_back(ioff.back() + ((k > KMAX && h.np <= WARP_NP) ? 0 : ceil_div(h.np, G_PATHS)));
-            soff.push_back(soff.back() + ((k > KMAX && slots <= SMALL4) ? 0 : ceil_div(slots, G_SLOTS)));
+            ioff.push_back(ioff.back() + ceil_div(h.np, G_PATHS));
+            soff.push_back(soff.back() + ceil_div(slots, G_SLOTS));
             ++pos;
         }
         if (used > arena_slots) {
@@ -1942,28 +2407,14 @@ static panther_status hub_tables(panther_ctx* ctx, const PathsRef& P, const int3
         ctx->hub_arena_clean = false;   // until the select pass of this round has run
         GPlan G{(const int32_t*)(dplan + o_q), (const int64_t*)(dplan + o_o), (const uint32_t*)(dplan + o_n),
                 (const int64_t*)(dplan + o_i), (const int64_t*)(dplan + o_s), rng, (const uint32_t*)(dplan + o_t)};
+        if (stride == 8) g_count_kernel<8><<<(unsigned)ioff.back(), 256, 0, s>>>(P, queries, G, arena, ctx->d_status);
+        else if (stride == 16) g_count_kernel<16><<<(unsigned)ioff.back(), 256, 0, s>>>(P, queries, G, arena, ctx->d_status);
+        else if (stride == 32) g_count_kernel<32><<<(unsigned)ioff.back(), 256, 0, s>>>(P, queries, G, arena, ctx->d_status);
+        else if (stride == 64) g_count_kernel<64><<<(unsigned)ioff.back(), 256, 0, s>>>(P, queries, G, arena, ctx->d_status);
+        else g_count_kernel<128><<<(unsigned)ioff.back(), 256, 0, s>>>(P, queries, G, arena, ctx->d_status);
         if (k > KMAX) {
-            const unsigned gwb = (unsigned)ceil_div((int64_t)rng * 32, 256);
-            if (stride == 8) g_count_warp_kernel<8><<<gwb, 256, 0, s>>>(P, queries, G, arena, ctx->d_status);
-            else if (stride == 16) g_count_warp_kernel<16><<<gwb, 256, 0, s>>>(P, queries, G, arena, ctx->d_status);
-            else if (stride == 32) g_count_warp_kernel<32><<<gwb, 256, 0, s>>>(P, queries, G, arena, ctx->d_status);
-            else if (stride == 64) g_count_warp_kernel<64><<<gwb, 256, 0, s>>>(P, queries, G, arena, ctx->d_status);
-            else g_count_warp_kernel<128><<<gwb, 256, 0, s>>>(P, queries, G, arena, ctx->d_status);
-            ctx->launches++;
-        }
-        if (ioff.back() > 0) {
-            if (stride == 8) g_count_kernel<8><<<(unsigned)ioff.back(), 256, 0, s>>>(P, queries, G, arena, ctx->d_status);
-            else if (stride == 16) g_count_kernel<16><<<(unsigned)ioff.back(), 256, 0, s>>>(P, queries, G, arena, ctx->d_status);
-            else if (stride == 32) g_count_kernel<32><<<(unsigned)ioff.back(), 256, 0, s>>>(P, queries, G, arena, ctx->d_status);
-            else if (stride == 64) g_count_kernel<64><<<(unsigned)ioff.back(), 256, 0, s>>>(P, queries, G, arena, ctx->d_status);
-            else g_count_kernel<128><<<(unsigned)ioff.back(), 256, 0, s>>>(P, queries, G, arena, ctx->d_status);
-        }
-        if (k > KMAX) {
-            g_small4_kernel<<<(unsigned)ceil_div((int64_t)rng * 32, 256), 256, 0, s>>>(G, arena, o);
-            if (soff.back() > 0) {
-                g_select4_kernel<<<(unsigned)soff.back(), 512, 0, s>>>(G, arena, k, partial);
-                g_merge4_kernel<<<rng, 256, 0, s>>>(G, partial, o);
-            }
+            g_select4_kernel<<<(unsigned)soff.back(), 512, 0, s>>>(G, arena, k, partial);
+            g_merge4_kernel<<<rng, 256, 0, s>>>(G, partial, o);
         } else {
             g_select_kernel<<<(unsigned)soff.back(), 512, 0, s>>>(G, arena, k, partial);
             g_merge_cta_kernel<<<rng, 256, 0, s>>>(G, partial, o);
@@ -1995,27 +2446,21 @@ panther_status topk_run(panther_ctx* ctx, const panther_index* ix, const panther
                         int64_t q, int k, int32_t* ids, uint32_t* cnt, bool plain) {
     cudaStream_t s = ctx->stream;
     TopkShape sh = topk_shape(ctx);
-    const size_t smem = (size_t)sh.cta_slots * 8 + (size_t)(sh.threads / 32) * KMAX * 8;
-    // the attribute is process-wide (contexts of several threads share it):
-    // always the larger of this shape and the big-table pass
-    const size_t attr = std::max(smem, BIG_SMEM);
     panther_status st;
-    if (p->stride == 8) st = set_smem_attr<8>(ctx, attr);
-    else if (p->stride == 16) st = set_smem_attr<16>(ctx, attr);
-    else if (p->stride == 32) st = set_smem_attr<32>(ctx, attr);
-    else if (p->stride == 64) st = set_smem_attr<64>(ctx, attr);
-    else st = set_smem_attr<128>(ctx, attr);
+    if (p->stride == 8) st = set_smem_attr<8>(ctx);
+    else if (p->stride == 16) st = set_smem_attr<16>(ctx);
+    else if (p->stride == 32) st = set_smem_attr<32>(ctx);
+    else if (p->stride == 64) st = set_smem_attr<64>(ctx);
+    else st = set_smem_attr<128>(ctx);
     if (st) return st;
     PathsRef P{p->rows, p->R, p->L, ix->off, ix->pid, ix->n, ix->cls};
     OutRef o{ids, cnt, k};
-    int64_t ccap = (int64_t)sh.cta_slots * 7 / 10;
-    // queries above the tuned shape's table but within a 24,576-slot one take a
-    // second persistent pass with one 1,024-thread CTA per SM
-    int64_t ccap_big = sh.cta_slots < BIG_SLOTS ? (int64_t)BIG_SLOTS * 7 / 10 : ccap;
-    if (ctx->dbg_hub_min_cap > 0) {   // test routing: a lower hub-tier bound
-        ccap = std::min(ccap, std::max<int64_t>(ctx->dbg_hub_min_cap, WCAP));
-        ccap_big = std::min(ccap_big, ccap);
-    }
+    // tables are at most 0.7 full; queries above the shape's table but within a
+    // 24,576-slot one take a second pass with one 512-thread CTA per SM
+    const int64_t wcap = WCAP, ccap = (int64_t)sh.cta_slots * 7 / 10;
+    int64_t ccap_big = (int64_t)BIG_SLOTS * 7 / 10;
+    if (ctx->dbg_hub_min_cap > 0)     // test routing: a lower hub-tier bound
+        ccap_big = std::min(ccap_big, std::max<int64_t>(ctx->dbg_hub_min_cap, HUB_MIN_CAP));
     for (int i = 0; i < 10; ++i) ctx->topk_stats[i] = 0;
     ctx->topk_stats[0] = q;
 
@@ -2039,17 +2484,11 @@ panther_status topk_run(panther_ctx* ctx, const panther_index* ix, const panther
         fill_empty_kernel<<<ctx->num_sms * 4, 256, 0, s>>>(gtab, gslots);
         ctx->launches++;
         for (int64_t i = 0; i < q; ++i) {
-            if (p->stride == 8)
-                single_kernel<8><<<1, sh.threads, smem, s>>>(P, queries, i, o, sh.cta_slots, gtab, gslots, ctx->d_status);
-            else if (p->stride == 16)
-                single_kernel<16><<<1, sh.threads, smem, s>>>(P, queries, i, o, sh.cta_slots, gtab, gslots, ctx->d_status);
-            else if (p->stride == 32)
-                single_kernel<32><<<1, sh.threads, smem, s>>>(P, queries, i, o, sh.cta_slots, gtab, gslots, ctx->d_status);
-            else if (p->stride == 64)
-                single_kernel<64><<<1, sh.threads, smem, s>>>(P, queries, i, o, sh.cta_slots, gtab, gslots, ctx->d_status);
-            else
-                single_kernel<128><<<1, sh.threads, smem, s>>>(P, queries, i, o, sh.cta_slots, gtab, gslots,
-                                                              ctx->d_status);
+            if (p->stride == 8) single_kernel<8><<<1, 1024, BIG_SMEM, s>>>(P, queries, i, o, BIG_SLOTS, gtab, gslots, ctx->d_status);
+            else if (p->stride == 16) single_kernel<16><<<1, 1024, BIG_SMEM, s>>>(P, queries, i, o, BIG_SLOTS, gtab, gslots, ctx->d_status);
+            else if (p->stride == 32) single_kernel<32><<<1, 1024, BIG_SMEM, s>>>(P, queries, i, o, BIG_SLOTS, gtab, gslots, ctx->d_status);
+            else if (p->stride == 64) single_kernel<64><<<1, 1024, BIG_SMEM, s>>>(P, queries, i, o, BIG_SLOTS, gtab, gslots, ctx->d_status);
+            else single_kernel<128><<<1, 1024, BIG_SMEM, s>>>(P, queries, i, o, BIG_SLOTS, gtab, gslots, ctx->d_status);
             ctx->launches++;
         }
         dev_free(ctx, gtab);
@@ -2057,16 +2496,12 @@ panther_status topk_run(panther_ctx* ctx, const panther_index* ix, const panther
         return PANTHER_OK;
     }
 
-    int32_t* lists = nullptr;
     int* counts = nullptr;
-    if ((st = dev_alloc(ctx, (void**)&lists, sizeof(int32_t) * 8 * (size_t)q)) ||
-        (st = dev_alloc(ctx, (void**)&counts, sizeof(int) * 16))) {
-        dev_free(ctx, lists);
-        return st;
-    }
+    if ((st = dev_alloc(ctx, (void**)&counts, sizeof(int) * 16 + sizeof(int32_t) * 8 * (size_t)q))) return st;
+    int32_t* const lists = counts + 16;
     Tiers tiers{{lists, lists + q, lists + 2 * q, lists + 3 * q, lists + 4 * q, lists + 5 * q, lists + 6 * q, lists + 7 * q},
                 counts};
-    const bool all_hub = k > KMAX;                      // 64 < k <= 128: device tables only
+    const bool wide_k = k > KMAX;                       // 64 < k <= 128: hub queries in device tables only
     // largest |P_v| the group tiers take: ids must fit below 2^group_ub(G)
     // (any k: G = 8 ranks at most 56 candidates, larger groups rank directly)
     const int group_max = p->stride != 8 ? 0
@@ -2074,85 +2509,76 @@ panther_status topk_run(panther_ctx* ctx, const panther_index* ix, const panther
                           : ix->n <= (int64_t(1) << group_ub(16)) ? 16 : 0;
     const bool lane_ok = p->stride == 8 && k <= LANE_K;
     PCK(ctx, cudaMemsetAsync(counts, 0, sizeof(int) * 16, s));
-    classify_kernel<<<(unsigned)ceil_div(q, 256 * CL_PER), 256, 0, s>>>(queries, q, P, ccap, ccap_big, lane_ok,
-                                                                         group_max, all_hub, tiers, o, ctx->d_status);
-    ctx->launches++;
-    // the lane and group tiers are independent of the persistent passes: they
-    // run on the side streams (joined back into `s` below)
-    const bool side = ctx->side[0] != nullptr;
-    cudaStream_t s0 = side ? ctx->side[0] : s, s1 = side ? ctx->side[1] : s;
-    if (side) {
-        PCK(ctx, cudaEventRecord(ctx->fork, s));
-        PCK(ctx, cudaStreamWaitEvent(s0, ctx->fork, 0));
-        PCK(ctx, cudaStreamWaitEvent(s1, ctx->fork, 0));
-    }
-    if (lane_ok) {
-        launch_lane(ix->n <= (int64_t(1) << 29), P.L == 6, k <= 12, (unsigned)(ctx->num_sms * 8), s0, P, queries,
-                    lists + 3 * q, counts, o);
+    if (q <= (wide_k ? SMALL_Q_WIDE : SMALL_Q)) {
+        if (p->stride == 8) launch_small<8>(ctx, P, queries, q, tiers, o, sh, ccap, ccap_big);
+        else if (p->stride == 16) launch_small<16>(ctx, P, queries, q, tiers, o, sh, ccap, ccap_big);
+        else if (p->stride == 32) launch_small<32>(ctx, P, queries, q, tiers, o, sh, ccap, ccap_big);
+        else if (p->stride == 64) launch_small<64>(ctx, P, queries, q, tiers, o, sh, ccap, ccap_big);
+        else launch_small<128>(ctx, P, queries, q, tiers, o, sh, ccap, ccap_big);
+    } else {
+        classify_kernel<<<(unsigned)ceil_div(q, 256 * CL_PER), 256, 0, s>>>(queries, q, P, wcap, ccap, ccap_big, lane_ok,
+                                                                             group_max, tiers, o, ctx->d_status);
         ctx->launches++;
-    }
-    if (group_max >= 16) {
-        group_kernel<8><<<(unsigned)(ctx->num_sms * 8), 256, 0, s0>>>(P, queries, lists + 4 * q, counts, 6, o);
-        group_kernel<16><<<(unsigned)(ctx->num_sms * 8), 256, 0, s1>>>(P, queries, lists + 5 * q, counts, 7, o);
-        ctx->launches += 2;
-    }
-    if (group_max >= 32) {
-        group_kernel<32><<<(unsigned)(ctx->num_sms * 8), 256, 0, s1>>>(P, queries, lists + 6 * q, counts, 8, o);
-        ctx->launches++;
-    }
-    if (side) {
-        PCK(ctx, cudaEventRecord(ctx->join[0], s0));
-        PCK(ctx, cudaEventRecord(ctx->join[1], s1));
-    }
-    // narrow warp tier: ids below 2^(32 - cb) with cb bits for the largest
-    // warp-tier count (a count never exceeds the query's number of paths)
-    int cb = 1;
-    while ((1 << cb) <= WCAP / std::max(1, P.L - 1)) ++cb;
-    const int narrow_cb = (cb <= 16 && ix->n <= (int64_t(1) << (32 - cb))) ? cb : 0;   // ids < 2^(32-cb)
-    PersistArgs A{P, queries, tiers, o, sh.cta_slots, ctx->d_status, narrow_cb};
-    unsigned blocks = (unsigned)(ctx->num_sms * sh.blocks_per_sm);
-    if (!all_hub) {
-    if (p->stride == 8) persistent_kernel<8><<<blocks, sh.threads, smem, s>>>(A);
-    else if (p->stride == 16) persistent_kernel<16><<<blocks, sh.threads, smem, s>>>(A);
-    else if (p->stride == 32) persistent_kernel<32><<<blocks, sh.threads, smem, s>>>(A);
-    else if (p->stride == 64) persistent_kernel<64><<<blocks, sh.threads, smem, s>>>(A);
-    else persistent_kernel<128><<<blocks, sh.threads, smem, s>>>(A);
-    ctx->launches++;
-    if (ccap_big > ccap) {
-        // CTA tier only: its list is tier 7's, its counters start at [9]
-        Tiers big{{lists, lists + 7 * q, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr}, counts + 9};
-        PersistArgs B{P, queries, big, o, BIG_SLOTS, ctx->d_status, 0};
-        const unsigned bb = (unsigned)ctx->num_sms;
-        if (p->stride == 8) persistent_kernel<8><<<bb, BIG_T, BIG_SMEM, s>>>(B);
-        else if (p->stride == 16) persistent_kernel<16><<<bb, BIG_T, BIG_SMEM, s>>>(B);
-        else if (p->stride == 32) persistent_kernel<32><<<bb, BIG_T, BIG_SMEM, s>>>(B);
-        else if (p->stride == 64) persistent_kernel<64><<<bb, BIG_T, BIG_SMEM, s>>>(B);
-        else persistent_kernel<128><<<bb, BIG_T, BIG_SMEM, s>>>(B);
-        ctx->launches++;
-    }
-    }   // !all_hub
-    if (side) {
-        PCK(ctx, cudaStreamWaitEvent(s, ctx->join[0], 0));
-        PCK(ctx, cudaStreamWaitEvent(s, ctx->join[1], 0));
+        // the lane and group tiers are independent of the persistent passes: they
+        // run on the side streams (joined back into `s` below)
+        const bool side = ctx->side[0] != nullptr;
+        cudaStream_t s0 = side ? ctx->side[0] : s, s1 = side ? ctx->side[1] : s;
+        if (side) {
+            PCK(ctx, cudaEventRecord(ctx->fork, s));
+            PCK(ctx, cudaStreamWaitEvent(s0, ctx->fork, 0));
+            PCK(ctx, cudaStreamWaitEvent(s1, ctx->fork, 0));
+        }
+        if (lane_ok) {
+            launch_lane(ix->n <= (int64_t(1) << 29), P.L == 6, k <= 12, (unsigned)(ctx->num_sms * 8), s0, P, queries,
+                        lists + 3 * q, counts, o);
+            ctx->launches++;
+        }
+        if (group_max >= 16) {
+            group_kernel<8><<<(unsigned)(ctx->num_sms * 8), 256, 0, s0>>>(P, queries, lists + 4 * q, counts, 6, o);
+            group_kernel<16><<<(unsigned)(ctx->num_sms * 8), 256, 0, s1>>>(P, queries, lists + 5 * q, counts, 7, o);
+            ctx->launches += 2;
+        }
+        if (group_max >= 32) {
+            group_kernel<32><<<(unsigned)(ctx->num_sms * 8), 256, 0, s1>>>(P, queries, lists + 6 * q, counts, 8, o);
+            ctx->launches++;
+        }
+        if (side) {
+            PCK(ctx, cudaEventRecord(ctx->join[0], s0));
+            PCK(ctx, cudaEventRecord(ctx->join[1], s1));
+        }
+        if (p->stride == 8) launch_teams<8>(ctx, P, queries, tiers, o, sh);
+        else if (p->stride == 16) launch_teams<16>(ctx, P, queries, tiers, o, sh);
+        else if (p->stride == 32) launch_teams<32>(ctx, P, queries, tiers, o, sh);
+        else if (p->stride == 64) launch_teams<64>(ctx, P, queries, tiers, o, sh);
+        else launch_teams<128>(ctx, P, queries, tiers, o, sh);
+        if (side) {
+            PCK(ctx, cudaStreamWaitEvent(s, ctx->join[0], 0));
+            PCK(ctx, cudaStreamWaitEvent(s, ctx->join[1], 0));
+        }
     }
     PCK(ctx, cudaGetLastError());
 
     // global tier: read its size (one synchronisation), then run in rounds
-    int h_counts[16];
+    int* h_counts = ctx->h_counts;                      // pinned: the copy is a plain DMA
     PCK(ctx, cudaMemcpyAsync(h_counts, counts, sizeof(int) * 16, cudaMemcpyDeviceToHost, s));
     PCK(ctx, cudaStreamSynchronize(s));
     const int ng = h_counts[2];
     ctx->topk_stats[1] = lane_ok ? h_counts[5] : 0;
     ctx->topk_stats[2] = (int64_t)h_counts[6] + h_counts[7] + h_counts[8];
-    ctx->topk_stats[3] = h_counts[0];
-    ctx->topk_stats[4] = (int64_t)h_counts[1] + (ccap_big > ccap ? h_counts[10] : 0);
-    ctx->topk_stats[5] = ng;
+    if (wide_k) {
+        // reported as queries counted in per-query tables, wherever these lie
+        ctx->topk_stats[7] = (int64_t)h_counts[0] + h_counts[1] + h_counts[10];
+        ctx->topk_stats[5] = ctx->topk_stats[7] + ng;
+    } else {
+        ctx->topk_stats[3] = h_counts[0];
+        ctx->topk_stats[4] = (int64_t)h_counts[1] + h_counts[10];
+        ctx->topk_stats[5] = ng;
+    }
     if (ng > 0) {
         std::vector<int32_t> gq(ng);
         std::vector<int64_t> npv(ng);
         int64_t* d_np = nullptr;
         if ((st = dev_alloc(ctx, (void**)&d_np, sizeof(int64_t) * ng))) {
-            dev_free(ctx, lists);
             dev_free(ctx, counts);
             return st;
         }
@@ -2173,7 +2599,7 @@ panther_status topk_run(panther_ctx* ctx, const panther_index* ix, const panther
         std::vector<HubQuery> hubs(ng);
         for (int i = 0; i < ng; ++i) {
             int64_t t = (int64_t)((double)npv[i] * HUB_PRUNE / std::max(k, 10));
-            hubs[i] = HubQuery{gq[i], npv[i], (t < 2 || all_hub) ? 0u : path_code(t)};
+            hubs[i] = HubQuery{gq[i], npv[i], (t < 2 || wide_k) ? 0u : path_code(t)};
         }
         // queries with a small filtered candidate bound count straight into a
         // device table (it stays in L2); the others go through the buckets
@@ -2184,7 +2610,7 @@ panther_status topk_run(panther_ctx* ctx, const panther_index* ix, const panther
                 bool table = h.thr > 0 && hub_bound(P, h, above) <= HUB_TABLE_BOUND;
                 if (ctx->dbg_hub_route == 1) table = false;
                 if (ctx->dbg_hub_route == 2) table = true;
-                if (all_hub) table = true;                 // the buckets keep 64-entry lists
+                if (wide_k) table = true;                 // the buckets keep 64-entry lists
                 (table ? tq : bq).push_back(h);
             }
             panther_status r = PANTHER_OK;
@@ -2201,12 +2627,10 @@ panther_status topk_run(panther_ctx* ctx, const panther_index* ix, const panther
         std::vector<HubQuery> none;
         if (!st && !again.empty()) st = hub_tables(ctx, P, queries, o, k, again, above, none);
         if (st) {
-            dev_free(ctx, lists);
             dev_free(ctx, counts);
             return st;
         }
     }
-    dev_free(ctx, lists);
     dev_free(ctx, counts);
     return PANTHER_OK;
 }
@@ -2285,8 +2709,8 @@ extern "C" panther_status panther_tune_topk(panther_ctx* ctx, const panther_inde
     if (ix->n != p->n || ix->R != p->R) return set_err(ctx, PANTHER_EINVAL, "index and paths do not belong together");
     cudaSetDevice(ctx->device);
     struct Shape { int threads, slots, bps; };
-    const Shape cand[] = {{1024, 24576, 1}, {512, 12288, 2}, {256, 6144, 4}, {256, 4096, 6},
-                          {512, 24576, 1}, {256, 8192, 3}, {128, 3072, 8}, {128, 4096, 6}};
+    const Shape cand[] = {{128, 3840, 6}, {128, 3072, 7}, {128, 6144, 4}, {256, 3840, 6},
+                          {256, 6144, 4}, {256, 8192, 3}, {512, 12288, 2}, {512, 24576, 1}};
     cudaEvent_t a, b;
     PCK(ctx, cudaEventCreate(&a));
     PCK(ctx, cudaEventCreate(&b));
@@ -2333,7 +2757,7 @@ extern "C" panther_status panther_tune_topk(panther_ctx* ctx, const panther_inde
 extern "C" panther_status panther_set_topk_shape(panther_ctx* ctx, int threads, int table_slots, int ctas_per_sm) {
     if (!ctx) return PANTHER_EINVAL;
     if ((threads != 128 && threads != 256 && threads != 512 && threads != 1024) || table_slots % 32 != 0 ||
-        table_slots < threads / 32 * WSLOTS || table_slots > 24576 || ctas_per_sm < 1 || ctas_per_sm > 8)
+        table_slots < threads / 32 * 512 || table_slots > 24576 || ctas_per_sm < 1 || ctas_per_sm > 8)
         return set_err(ctx, PANTHER_EINVAL, "unsupported top-k launch shape");
     ctx->topk_threads = threads;
     ctx->topk_cta_slots = table_slots;
