@@ -20,19 +20,20 @@
 // If every entry of a and of b is <= 256, the BF16 inputs are exact and every
 // partial sum is an integer of magnitude < 2^24, so y_hat = y exactly.
 //
-// Selection (one thread per query row of the tile) keeps the k best keys in
-// shared memory: exact pairs insert (y, id); other pairs are kept while their
-// lower bound y_hat - E does not exceed the k-th key, insert (y_hat + E, id)
-// and are appended to a per-query shortlist. Afterwards every kept candidate
-// is re-ranked with exact uint64 arithmetic on the integer vectors, so the
-// answer is exact. Candidates (and queries) are stored exact rows first, so
-// whole 256-candidate tiles take the one-compare fast path.
+// Selection (two threads per query row of the tile, half of the columns each)
+// keeps the k best keys in shared memory: exact pairs insert (y, id); other
+// pairs are kept while their lower bound y_hat - E does not exceed the k-th
+// key, insert (y_hat + E, id) and are appended to a per-query shortlist.
+// Afterwards every kept candidate is re-ranked with exact uint64 arithmetic on
+// the integer vectors, so the answer is exact. Candidates (and queries) are
+// stored exact rows first, so whole 256-candidate tiles take the fast path:
+// the minimum of 32 columns, which comes with the TMEM load.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <math.h>
 
 #include <algorithm>
-#include <vector>
+#include <numeric>
 
 #include "internal.cuh"
 
@@ -69,37 +70,49 @@ __device__ __forceinline__ uint32_t round8(uint32_t x) {
     return q << sh;                  // may carry to 2^(p+1): still 8 significant bits
 }
 
-// minimum of three floats in one instruction (the values are finite here)
-__device__ __forceinline__ float fmin3(float a, float b, float c) {
-    float r;
-    asm("min.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
-    return r;
-}
-
 __device__ __forceinline__ uint16_t bf16_bits_of(float f) {   // f exactly representable
     return (uint16_t)(__float_as_uint(f) >> 16);
 }
 
-// per-vertex statistics and the exact-row flag
-__global__ void vec_stats_kernel(const uint32_t* __restrict__ theta, int64_t n, int D, uint64_t* __restrict__ norm2,
-                                 float* __restrict__ nrm, uint8_t* __restrict__ exact, int64_t* __restrict__ flag,
-                                 unsigned* __restrict__ maxv) {
-    int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (v >= n) return;
-    uint64_t s = 0;
-    uint32_t mx = 0;
-    for (int d = 0; d < D; ++d) {
-        uint32_t x = theta[v * D + d];
-        s += (uint64_t)x * x;
-        mx = x > mx ? x : mx;
+// per-vertex statistics and the exact-row flag: eight lanes per row (coalesced
+// sectors and several rows in flight per warp; a thread per row strides by D),
+// one maximum per warp
+__global__ void __launch_bounds__(256) vec_stats_kernel(const uint32_t* __restrict__ theta, int64_t n, int D,
+                                                        uint64_t* __restrict__ norm2, float* __restrict__ nrm,
+                                                        uint8_t* __restrict__ exact, int64_t* __restrict__ flag,
+                                                        unsigned* __restrict__ maxv) {
+    const int sub = threadIdx.x & 7;
+    const int64_t nrows = (int64_t)gridDim.x * blockDim.x / 8;
+    uint32_t top = 0;
+    for (int64_t v = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / 8; __any_sync(0xffffffffu, v < n);
+         v += nrows) {
+        uint64_t s = 0;
+        uint32_t mx = 0;
+        if (v < n) {
+#pragma unroll 8
+            for (int d = sub; d < D; d += 8) {
+                const uint32_t x = theta[v * D + d];
+                s += (uint64_t)x * x;
+                mx = x > mx ? x : mx;
+            }
+        }
+#pragma unroll
+        for (int o = 4; o; o >>= 1) {
+            s += __shfl_xor_sync(0xffffffffu, s, o);
+            mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        }
+        top = max(top, mx);
+        if (sub == 0 && v < n) {
+            norm2[v] = s;
+            const float r = sqrtf(__ull2float_ru(s));
+            nrm[v] = r * (1.0f + 1.0f / (1 << 21));
+            const uint8_t e = mx <= MAX_EXACT;
+            exact[v] = e;
+            flag[v] = e;
+        }
     }
-    norm2[v] = s;
-    float r = sqrtf(__ull2float_ru(s));
-    nrm[v] = r * (1.0f + 1.0f / (1 << 21));
-    uint8_t e = mx <= MAX_EXACT;
-    exact[v] = e;
-    flag[v] = e;
-    atomicMax(maxv, mx);
+    top = __reduce_max_sync(0xffffffffu, top);
+    if ((threadIdx.x & 31) == 0 && top) atomicMax(maxv, top);
 }
 
 // position of every vertex: exact rows first (id ascending), then the rest
@@ -112,68 +125,77 @@ __global__ void vec_perm_kernel(const uint8_t* __restrict__ exact, const int64_t
     pos[v] = p;
 }
 
-// B rows (candidate role) in permuted order + SoA candidate info
-__global__ void vec_brow_kernel(const uint32_t* __restrict__ theta, const uint64_t* __restrict__ norm2,
-                                const float* __restrict__ nrm, const int32_t* __restrict__ perm, VecMeta M,
-                                uint16_t* __restrict__ B, int32_t* __restrict__ cid, float* __restrict__ cnrm,
-                                float* __restrict__ cncf) {
-    int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+// B rows (candidate role) in permuted order + SoA candidate info: eight lanes
+// per row, each writing eight columns as one 16-byte store (1.5M rows of D = 50:
+// 961 us with a thread per row, 320 with a warp per row)
+__global__ void __launch_bounds__(256) vec_brow_kernel(const uint32_t* __restrict__ theta,
+                                                       const uint64_t* __restrict__ norm2,
+                                                       const float* __restrict__ nrm,
+                                                       const int32_t* __restrict__ perm, VecMeta M,
+                                                       uint16_t* __restrict__ B, int32_t* __restrict__ cid,
+                                                       float* __restrict__ cnrm, float* __restrict__ cncf) {
+    const int64_t p = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / 8;
+    const int sub = threadIdx.x & 7;
     if (p >= M.npad) return;
-    uint16_t* row = B ? B + p * KN_K : nullptr;      // no BF16 rows when D > 56 (FP32 form only)
-    if (p >= M.n) {
-        // padding: y = 2^40 for every query, id -1 (never selected)
-        if (row) {
-            for (int d = 0; d < KN_K; ++d) row[d] = 0;
-            row[M.D] = bf16_bits_of(1099511627776.0f);
+    const bool pad = p >= M.n;
+    const int32_t v = pad ? -1 : perm[p];
+    const uint64_t n2 = pad ? 0 : norm2[v];
+    if (B) {                                         // no BF16 rows when D > 56 (FP32 form only)
+        uint32_t c[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const int d = sub * 8 + j;
+            c[j] = !pad && d < M.D ? theta[(int64_t)v * M.D + d] : 0u;
         }
-        cid[p] = -1;
-        cnrm[p] = 0.f;
-        cncf[p] = 1099511627776.0f;
-        return;
+        uint32_t out[4];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const int d = sub * 8 + j;
+            float f = -2.0f * (float)round8(c[j]);
+            if (pad) f = d == M.D ? 1099511627776.0f : 0.f;   // padding: y = 2^40 for every query, id -1
+            else if (d >= M.D) f = d < M.D + 8 ? ldexpf((float)((n2 >> (8 * (d - M.D))) & 255ull), 8 * (d - M.D)) : 0.f;
+            const uint32_t b = bf16_bits_of(f);
+            out[j / 2] = j & 1 ? out[j / 2] | (b << 16) : b;
+        }
+        ((uint4*)(B + p * KN_K))[sub] = make_uint4(out[0], out[1], out[2], out[3]);
     }
-    int32_t v = perm[p];
-    for (int d = 0; row && d < KN_K; ++d) {
-        float f = 0.f;
-        if (d < M.D) f = -2.0f * (float)round8(theta[(int64_t)v * M.D + d]);
-        else if (d < M.D + 8) {
-            int i = d - M.D;
-            uint64_t piece = (norm2[v] >> (8 * i)) & 255ull;
-            f = ldexpf((float)piece, 8 * i);
-        }
-        row[d] = bf16_bits_of(f);
-    }
-    cid[p] = v;
-    cnrm[p] = nrm[v];
-    cncf[p] = __ull2float_ru(norm2[v]);
-}
-
-// A rows (query role) for a list of query slots
-__global__ void vec_arow_kernel(const uint32_t* __restrict__ theta, const int32_t* __restrict__ qv, int64_t qpad,
-                                int D, uint16_t* __restrict__ A) {
-    int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= qpad) return;
-    uint16_t* row = A + s * KN_K;
-    int32_t v = qv[s];
-    for (int d = 0; d < KN_K; ++d) {
-        float f = 0.f;
-        if (v >= 0) {
-            if (d < D) f = (float)round8(theta[(int64_t)v * D + d]);
-            else if (d < D + 8) f = 1.0f;
-        }
-        row[d] = bf16_bits_of(f);
+    if (sub == 0) {
+        cid[p] = v;
+        cnrm[p] = pad ? 0.f : nrm[v];
+        cncf[p] = pad ? 1099511627776.0f : __ull2float_ru(n2);
     }
 }
 
-__global__ void tile_flags_kernel(const uint8_t* __restrict__ exact, const int32_t* __restrict__ ids, int64_t count,
-                                  int tile, uint8_t* __restrict__ out, int64_t ntiles) {
-    int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= ntiles) return;
-    uint8_t all = 1;
-    for (int64_t i = t * tile; i < (t + 1) * tile && i < count; ++i) {
-        int32_t v = ids[i];
-        if (v >= 0 && !exact[v]) all = 0;
+// A rows (query role) for a list of query slots, a warp per row
+__global__ void __launch_bounds__(256) vec_arow_kernel(const uint32_t* __restrict__ theta,
+                                                       const int32_t* __restrict__ qv, int64_t qpad, int D,
+                                                       uint16_t* __restrict__ A) {
+    const int64_t s = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    if (s >= qpad) return;                           // warp-uniform
+    const int32_t v = qv[s];
+    auto col = [&](int d) -> uint32_t {
+        float f = 0.f;
+        if (v >= 0 && d < D) f = (float)round8(theta[(int64_t)v * D + d]);
+        else if (v >= 0 && d < D + 8) f = 1.0f;
+        return bf16_bits_of(f);
+    };
+    ((uint32_t*)(A + s * KN_K))[lane] = col(2 * lane) | (col(2 * lane + 1) << 16);
+}
+
+// out[t] = every id of tile t is padding or an exact row (a warp per tile)
+__global__ void __launch_bounds__(256) tile_flags_kernel(const uint8_t* __restrict__ exact,
+                                                         const int32_t* __restrict__ ids, int64_t count, int tile,
+                                                         uint8_t* __restrict__ out, int64_t ntiles) {
+    const int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (t >= ntiles) return;                         // warp-uniform
+    bool all = true;
+    for (int64_t i = t * tile + (threadIdx.x & 31); i < (t + 1) * tile && i < count; i += 32) {
+        const int32_t v = ids[i];
+        all &= v < 0 || exact[v] != 0;
     }
-    out[t] = all;
+    all = __all_sync(0xffffffffu, all);
+    if ((threadIdx.x & 31) == 0) out[t] = all ? 1 : 0;
 }
 
 // ----------------------------------------------------------- PTX helpers ---
@@ -263,23 +285,27 @@ __device__ __forceinline__ void umma_commit(uint32_t bar) {
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
-// 32 columns of this thread's TMEM lane into r (asynchronous: wait before use)
-__device__ __forceinline__ void tmem_ld32_async(uint32_t taddr, uint32_t (&r)[32]) {
+// 32 columns of this thread's TMEM lane into r and the smallest of them as
+// floats into m (asynchronous: wait before use). The minimum comes with the
+// load: taken by FMNMX instructions it was three quarters of the selection
+// warps' work.
+__device__ __forceinline__ void tmem_ld32_min_async(uint32_t taddr, uint32_t (&r)[32], float& m) {
     asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
+        "tcgen05.ld.red.sync.aligned.32x32b.x32.min.f32 "
         "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-        "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+        "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, %32, [%33];"
         : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
           "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
           "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-          "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+          "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31]),
+          "=f"(m)
         : "r"(taddr));
 }
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 // ties the registers to a point after the wait, so no use is scheduled before it
-__device__ __forceinline__ void reg_fence(uint32_t (&r)[32]) {
+__device__ __forceinline__ void reg_fence(uint32_t (&r)[32], float& m) {
     asm volatile(""
-                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
+                 : "+f"(m), "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
                    "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]),
                    "+r"(r[15]), "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]),
                    "+r"(r[22]), "+r"(r[23]), "+r"(r[24]), "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]),
@@ -345,36 +371,133 @@ __device__ __noinline__ Row take_bounded(Row r, const RowConst& c, float y, floa
     return r;
 }
 
-// one group of 32 screened values y (columns pos0 .. pos0+31)
-__device__ __forceinline__ Row select_group(Row r, const RowConst& c, const float (&y)[32], bool fast,
-                                            const int32_t* cid, const float* cnrm, const float* cncf, int64_t pos0,
-                                            int64_t nexact) {
-    if (c.qid < 0) return r;
-    if (fast) {
-        // exact tiles hold exact rows in ascending id order, after every row
-        // already in the list, so a candidate tied with the k-th key never
-        // wins its tie: only y < thr can enter. The minimum of the 32 values
-        // decides whether any can: three-input minima, 16 instructions.
-        float t11[11];
+// smallest upper bound of a group's keys (SEED), from the smallest of its
+// values when the tile is exact (+inf when it holds padding only: exact keys
+// lie below 2^24, padding's is 2^40)
+__device__ __forceinline__ float seed_exact(float m) {
+    return m < 1099511627776.0f ? m : __int_as_float(0x7f800000);
+}
+__device__ __forceinline__ float seed_bounded(const RowConst& c, const uint32_t (&y)[32], const int32_t* cid,
+                                              const float* cnrm, const float* cncf) {
+    float m = __int_as_float(0x7f800000);
 #pragma unroll
-        for (int j = 0; j < 10; ++j) t11[j] = fmin3(y[3 * j], y[3 * j + 1], y[3 * j + 2]);
-        t11[10] = fminf(y[30], y[31]);
-        const float m = fminf(fmin3(fmin3(t11[0], t11[1], t11[2]), fmin3(t11[3], t11[4], t11[5]),
-                                    fmin3(t11[6], t11[7], t11[8])),
-                              fminf(t11[9], t11[10]));
-        if (m < r.thr) {
+    for (int j = 0; j < 32; ++j) {
+        const float E = fmaf(c.anrm, cnrm[j], fmaf(KN_BETA, cncf[j], 1.0f)) * 1.0001f;
+        if (cid[j] >= 0) m = fminf(m, __fadd_ru(__uint_as_float(y[j]), E));
+    }
+    return m;
+}
+
+// One group of 32 screened values y of an exact tile, for the 32 rows of a
+// warp (every lane calls it; `live` marks query rows). Exact tiles hold exact
+// rows in ascending id order, after every row already in the list, so a
+// candidate tied with the k-th key never wins its tie: only y < thr can enter.
+// Mostly one row of the warp has one such candidate, so the warp inserts it
+// together, lane l holding entry l of the row's list: an insertion by the
+// row's own lane is a chain of up to k loads and stores the tile's other warps
+// soon wait for, and a call there saves the group's registers.
+__device__ __forceinline__ Row select_exact(Row r, const RowConst& c, const uint32_t (&y)[32], const int32_t* cid,
+                                            bool live, float2* warp_lists) {
+    const int lane = threadIdx.x & 31;
+    int last = -1;
+    for (;;) {
+        // this row's next column below thr
+        float key = 0.f;
+        int at = -1;
 #pragma unroll
-            for (int j = 0; j < 32; ++j)
-                if (y[j] < r.thr) r = take_exact(r, c, y[j], cid[j]);
-        }
-    } else {
-#pragma unroll
-        for (int j = 0; j < 32; ++j) {
-            float E = fmaf(c.anrm, cnrm[j], fmaf(KN_BETA, cncf[j], 1.0f)) * 1.0001f;
-            if (__fsub_rd(y[j], E) <= r.thr) r = take_bounded(r, c, y[j], E, cid[j], pos0 + j < nexact);
+        for (int j = 31; j >= 0; --j)
+            if (__uint_as_float(y[j]) < r.thr && j > last) {
+                key = __uint_as_float(y[j]);
+                at = j;
+            }
+        unsigned rows = __ballot_sync(0xffffffffu, live && at >= 0);
+        if (!rows) return r;
+        const int id = at >= 0 ? cid[at] : -1;
+        last = at >= 0 ? at : 32;
+        rows &= __ballot_sync(0xffffffffu, id >= 0 && id != c.self);
+        while (rows) {                               // warp-uniform
+            const int l = __ffs(rows) - 1;
+            rows &= rows - 1;
+            const float nk = __shfl_sync(0xffffffffu, key, l);
+            const int ni = __shfl_sync(0xffffffffu, id, l), n = __shfl_sync(0xffffffffu, r.n, l);
+            float2* list = warp_lists + l * (KN_SPLIT * KN_KMAX);
+            float2 e = make_float2(0.f, 0.f);
+            if (lane < n) e = list[lane];
+            const bool before = lane < n && (e.x < nk || (e.x == nk && __float_as_int(e.y) < ni));
+            const int pos = __popc(__ballot_sync(0xffffffffu, before));
+            float2 up;
+            up.x = __shfl_up_sync(0xffffffffu, e.x, 1);
+            up.y = __shfl_up_sync(0xffffffffu, e.y, 1);
+            const int n1 = n < c.k ? n + 1 : n;
+            e = lane < pos ? e : lane == pos ? make_float2(nk, __int_as_float(ni)) : up;
+            __syncwarp();
+            if (lane >= pos && lane < n1) list[lane] = e;
+            __syncwarp();
+            const float wk = __shfl_sync(0xffffffffu, e.x, c.k - 1);
+            const float wi = __shfl_sync(0xffffffffu, e.y, c.k - 1);
+            if (lane == l) {
+                r.n = n1;
+                if (n1 == c.k) {
+                    r.thr = wk;
+                    r.thr_id = __float_as_int(wi);
+                }
+            }
         }
     }
+}
+
+// one group of 32 screened values y (columns pos0 .. pos0+31) with error bounds
+__device__ __forceinline__ Row select_bounded(Row r, const RowConst& c, const uint32_t (&y)[32], const int32_t* cid,
+                                              const float* cnrm, const float* cncf, int64_t pos0, int64_t nexact) {
+#pragma unroll
+    for (int j = 0; j < 32; ++j) {
+        const float E = fmaf(c.anrm, cnrm[j], fmaf(KN_BETA, cncf[j], 1.0f)) * 1.0001f;
+        if (__fsub_rd(__uint_as_float(y[j]), E) <= r.thr)
+            r = take_bounded(r, c, __uint_as_float(y[j]), E, cid[j], pos0 + j < nexact);
+    }
     return r;
+}
+
+// The screen's work, query tiles x candidate tiles in query-tile order, is cut
+// into G equal runs, one per CTA: a run crosses query tiles and a query tile is
+// cut into at most `nseg` segments, each with lists of its own. (Whole query
+// tiles per CTA leave SMs idle when their number is a little above a multiple
+// of the SM count: 157 tiles on 152 SMs took two waves.) With G = 0 a CTA
+// takes whole query tiles in turn (nseg = 1; the FP32 form's own candidate
+// ranges are nseg segments of every tile).
+struct Split {
+    int64_t nqt, nct, G;
+    int64_t nseg;
+    __host__ __device__ int64_t begin(int64_t g) const { return g * (nqt * nct) / G; }
+    __host__ __device__ int64_t owner(int64_t unit) const { return ((unit + 1) * G - 1) / (nqt * nct); }
+    __host__ __device__ int64_t first(int64_t qt) const { return G ? owner(qt * nct) : 0; }
+    __host__ __device__ int64_t segments(int64_t qt) const {
+        return G ? owner((qt + 1) * nct - 1) - owner(qt * nct) + 1 : nseg;
+    }
+};
+
+// work item j of CTA c: a query tile, its segment and the candidate tiles of it
+struct Item {
+    int64_t qt, seg, ct0, ct1;
+};
+__device__ __forceinline__ bool split_item(const Split& W, int64_t c, int64_t grid, int64_t j, Item* it) {
+    if (!W.G) {
+        it->qt = c + j * grid;
+        it->seg = 0;
+        it->ct0 = 0;
+        it->ct1 = W.nct;
+        return it->qt < W.nqt;
+    }
+    const int64_t u0 = W.begin(c), u1 = W.begin(c + 1);
+    if (u0 >= u1) return false;
+    const int64_t qt = u0 / W.nct + j;
+    const int64_t a = qt * W.nct;
+    if (a >= u1) return false;
+    it->qt = qt;
+    it->seg = c - W.first(qt);
+    it->ct0 = u0 > a ? u0 - a : 0;
+    it->ct1 = u1 < a + W.nct ? u1 - a : W.nct;
+    return true;
 }
 
 struct ScreenArgs {
@@ -382,18 +505,20 @@ struct ScreenArgs {
     const float* cnrm;       // [npad]
     const float* cncf;       // [npad]
     const uint8_t* ctile;    // [npad/256] all-exact flags
-    int64_t nct;             // candidate tiles
+    Split W;                 // nct of it: candidate tiles screened (SEED: of the sample)
+    uint32_t seed_step, seed_mul;   // SEED: tile j of the sample is candidate tile (j * mul mod nct) * step
+    const float* thr0;       // [qpad] upper bound of the k-th key, or null
     int64_t nexact;          // exact candidate positions
     const int32_t* qv;       // [qpad] query vertex per slot (-1 pad)
     const float* qnrm;       // [qpad]
     const uint8_t* qexact;   // [qpad]
     const uint8_t* qtile;    // [qpad/128] all-exact flags
-    int64_t nqt;
-    int64_t nchunk;          // candidate ranges per query tile (work item = tile x range)
     int k;
-    float2* lists;           // [qpad][nchunk][KN_SPLIT][k]
-    int32_t* shortlist;      // [qpad][nchunk][KN_SPLIT][KN_SCAP]
-    int32_t* scount;         // [qpad][nchunk][KN_SPLIT]
+    float2* lists;           // [qpad][nseg][KN_SPLIT][k]
+    int32_t* shortlist;      // [qpad][nseg][KN_SPLIT][KN_SCAP]
+    int32_t* scount;         // [qpad][nseg][KN_SPLIT]
+    float* smin;             // SEED: [qpad][nseg][KN_SPLIT][seed_keys]
+    int seed_keys;           // SEED: minima written per segment and column slice: 20, 4 or 1
     int* overflow;           // [qpad]
     uint32_t* status;
     bool exclude_self;       // queries and candidates are the same vertices
@@ -411,11 +536,33 @@ constexpr uint32_t SM_BAR = SM_LIST + KN_M * KN_SPLIT * KN_KMAX * 8;   // barrie
 constexpr uint32_t SM_TOTAL = SM_BAR + 256;
 constexpr uint32_t KN_SMEM_BYTES = SM_TOTAL + 1024;
 
-// DUMP = true is the measurement form (pantherpp_debug_screen): it also
-// writes every screened value y_hat to S.dump; DUMP = false is the k-NN path.
-template <bool DUMP>
+// SCREEN is the k-NN path. DUMP is the measurement form
+// (pantherpp_debug_screen): it also writes every screened value y_hat to
+// S.dump. SEED screens a sample of the candidate tiles first, in an order
+// scattered over them, to bound each query's k-th key from above (S.thr0 of
+// the SCREEN launch). Without it a query meets the candidates by ascending id,
+// which real ids make a bad order (low ids, high degrees: every candidate is
+// nearer than all before it and enters the list). 48 queries against 1M
+// vertices: 589 us without the sample and with insertions by single lanes, 10 +
+// 74 now; 20,011 against 1.5M: 17.4 ms, 0.13 + 4.16 now (5.7 with single-lane
+// insertions, 3.1 with none). Taking all tiles in the scattered order was 18 ms:
+// the few candidates that enter then no longer come in the same tiles for many
+// rows, and ties at the k-th key enter by id. The sample keeps no
+// lists (a new list takes every candidate of its first tiles): only the minima
+// of SEED_T * 4 disjoint shares of each segment's column slice, whose
+// (k+1)-th smallest over the query bounds its k-th key (one of them may be the
+// query itself).
+constexpr int SEED_T = 5;
+enum { SCREEN = 0, DUMP_FORM = 1, SEED = 2 };
+
+template <int MODE>
 __global__ void __launch_bounds__(KN_THREADS, 1)
     screen_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, ScreenArgs S) {
+    constexpr bool DUMP = MODE == DUMP_FORM;
+    auto tile_at = [&](int64_t ct) -> int64_t {
+        if (MODE != SEED) return ct;
+        return (int64_t)((uint64_t)((uint32_t)ct) * S.seed_mul % (uint32_t)S.W.nct) * S.seed_step;
+    };
     extern __shared__ uint8_t smraw[];
     const uint32_t raw = smem_u32(smraw);
     const uint32_t base = (raw + 1023) & ~1023u;
@@ -468,17 +615,17 @@ __global__ void __launch_bounds__(KN_THREADS, 1)
             int64_t it = 0;
             int j = 0;
             bool ok = true;
-            for (int64_t wi = blockIdx.x; wi < S.nqt * S.nchunk && ok; wi += gridDim.x, ++j) {
-                const int64_t qt = wi / S.nchunk, ch = wi % S.nchunk;
-                const int64_t ct0 = ch * S.nct / S.nchunk, ct1 = (ch + 1) * S.nct / S.nchunk;
+            Item w;
+            for (; ok && split_item(S.W, blockIdx.x, gridDim.x, j, &w); ++j) {
                 if (!mbar_wait(AEMPTY, (j & 1) ^ 1, S.status, abort_flag)) {
                     ok = false;
                     break;
                 }
                 mbar_expect_tx(AFULL, KN_M * KN_K * 2);
-                tma_load_2d(base + SM_A, &tmA, 0, (int)(qt * KN_M), AFULL);
+                tma_load_2d(base + SM_A, &tmA, 0, (int)(w.qt * KN_M), AFULL);
                 last_a = j & 1;
-                for (int64_t ct = ct0; ct < ct1; ++ct, ++it) {
+                for (int64_t c = w.ct0; c < w.ct1; ++c, ++it) {
+                    const int64_t ct = tile_at(c);
                     int s = (int)(it % KN_STAGES);
                     uint32_t ph = (uint32_t)((it / KN_STAGES) & 1);
                     if (!mbar_wait(EMPTY(s), ph ^ 1, S.status, abort_flag)) { ok = false; break; }
@@ -497,12 +644,11 @@ __global__ void __launch_bounds__(KN_THREADS, 1)
         if (lane == 0) {
             int64_t it = 0;
             int j = 0;
-            for (int64_t wi = blockIdx.x; wi < S.nqt * S.nchunk; wi += gridDim.x, ++j) {
-                const int64_t ch = wi % S.nchunk;
-                const int64_t ct0 = ch * S.nct / S.nchunk, ct1 = (ch + 1) * S.nct / S.nchunk;
+            Item w;
+            for (; split_item(S.W, blockIdx.x, gridDim.x, j, &w); ++j) {
                 if (!mbar_wait(AFULL, j & 1, S.status, abort_flag)) break;
                 bool ok = true;
-                for (int64_t ct = ct0; ct < ct1; ++ct, ++it) {
+                for (int64_t ct = w.ct0; ct < w.ct1; ++ct, ++it) {
                     int s = (int)(it % KN_STAGES);
                     uint32_t ph = (uint32_t)((it / KN_STAGES) & 1);
                     int b = (int)(it & 1);
@@ -531,74 +677,124 @@ __global__ void __launch_bounds__(KN_THREADS, 1)
         const int half = (warp - 2) >> 2;         // column slice of every tile this warp screens
         const int row = quarter * 32 + lane;
         float2* mylist = (float2*)(gbase + SM_LIST) + (row * KN_SPLIT + half) * KN_KMAX;
-        int64_t it = 0;
-        for (int64_t wi = blockIdx.x; wi < S.nqt * S.nchunk; wi += gridDim.x) {
-            const int64_t qt = wi / S.nchunk, ch = wi % S.nchunk;
-            const int64_t ct0 = ch * S.nct / S.nchunk, ct1 = (ch + 1) * S.nct / S.nchunk;
-            const int64_t slot = qt * KN_M + row;
-            Row r{__int_as_float(0x7f800000), 0x7fffffff, 0, 0};
-            const int64_t state = (slot * S.nchunk + ch) * KN_SPLIT + half;
+        uint32_t it = 0;
+        Item w;
+        for (int64_t wj = 0; split_item(S.W, blockIdx.x, gridDim.x, wj, &w); ++wj) {
+            const int64_t slot = w.qt * KN_M + row;
+            // keys up to thr0 (the k-th key is no larger) enter until k are held
+            Row r{S.thr0 ? nextafterf(S.thr0[slot], __int_as_float(0x7f800000)) : __int_as_float(0x7f800000),
+                  0x7fffffff, 0, 0};
+            const int64_t state = (slot * S.W.nseg + w.seg) * KN_SPLIT + half;
             const RowConst rc{S.qv[slot], S.exclude_self ? S.qv[slot] : -2, S.qexact[slot] != 0,
-                              KN_ALPHA * S.qnrm[slot], mylist, S.shortlist + state * KN_SCAP, S.overflow + slot, S.k};
-            const bool qtile_exact = S.qtile[qt] != 0;
+                              KN_ALPHA * S.qnrm[slot], mylist,
+                              S.shortlist + state * KN_SCAP, S.overflow + slot, S.k};
+            const bool qtile_exact = S.qtile[w.qt] != 0;
+            float acc[SEED_T * 4];
+            int turn = 0;
+            if (MODE == SEED)
+#pragma unroll
+                for (int i = 0; i < SEED_T * 4; ++i) acc[i] = __int_as_float(0x7f800000);
             bool ok = true;
-            for (int64_t ct = ct0; ct < ct1; ++ct, ++it) {
-                int s = (int)(it % KN_STAGES);
-                uint32_t ph = (uint32_t)((it / KN_STAGES) & 1);
-                int b = (int)(it & 1);
-                uint32_t pb = (uint32_t)((it >> 1) & 1);
-                if (!mbar_wait(FULL(s), ph, S.status, abort_flag) || !mbar_wait(TFULL(b), pb, S.status, abort_flag)) {
+            bool flag = S.ctile[tile_at(w.ct0)] != 0;    // of the coming tile, loaded a tile ahead
+            for (int64_t c = w.ct0; c < w.ct1; ++c, ++it) {
+                const int64_t ct = tile_at(c);
+                const int s = (int)(it % KN_STAGES);
+                const uint32_t ph = (it / KN_STAGES) & 1;
+                const int b = (int)(it & 1);
+                const uint32_t pb = (it >> 1) & 1;
+                const bool fast = qtile_exact && flag;
+                if (c + 1 < w.ct1) flag = S.ctile[tile_at(c + 1)] != 0;
+                if (!__all_sync(0xffffffffu, mbar_wait(TFULL(b), pb, S.status, abort_flag))) {
                     ok = false;
                     break;
                 }
                 tc_fence_after();
                 const uint8_t* info = gbase + SM_INFO + s * (KN_N * 12);
-                const int32_t* cid = (const int32_t*)info;
-                const float* cnrm = (const float*)(info + KN_N * 4);
-                const float* cncf = (const float*)(info + KN_N * 8);
-                const bool fast = qtile_exact && S.ctile[ct];
-                const uint32_t tbase = tmem + ((uint32_t)(quarter * 32) << 16) + b * KN_N;
-                {
-                    const int h = half;                   // 128 columns per selection warp
-                    uint32_t u0[32], u1[32], u2[32], u3[32];
-                    __syncwarp();
-                    tmem_ld32_async(tbase + h * 128 + 0, u0);
-                    tmem_ld32_async(tbase + h * 128 + 32, u1);
-                    tmem_ld32_async(tbase + h * 128 + 64, u2);
-                    tmem_ld32_async(tbase + h * 128 + 96, u3);
-                    tmem_wait_ld();
-                    reg_fence(u0);
-                    reg_fence(u1);
-                    reg_fence(u2);
-                    reg_fence(u3);
-                    float y[32];
-#define KN_GROUP(U, G)                                                                                   \
-    {                                                                                                    \
-        _Pragma("unroll") for (int j = 0; j < 32; ++j) y[j] = __uint_as_float(U[j]);                     \
-        const int c0 = h * 128 + (G) * 32;                                                               \
-        if (DUMP && rc.qid >= 0) {                                                                       \
-            float* dst = S.dump + (int64_t)S.qidx[slot] * S.npad + ct * KN_N + c0;                       \
-            _Pragma("unroll") for (int j = 0; j < 32; ++j) dst[j] = y[j];                                \
-        }                                                                                                \
-        r = select_group(r, rc, y, fast, cid + c0, cnrm + c0, cncf + c0, ct * KN_N + c0, S.nexact);      \
-    }
-                    KN_GROUP(u0, 0)
-                    KN_GROUP(u1, 1)
-                    KN_GROUP(u2, 2)
-                    KN_GROUP(u3, 3)
-#undef KN_GROUP
-                }
+                const int c0 = half * 128;                // 128 columns per selection warp
+                const int32_t* cid = (const int32_t*)info + c0;
+                const float* cnrm = (const float*)(info + KN_N * 4) + c0;
+                const float* cncf = (const float*)(info + KN_N * 8) + c0;
+                const uint32_t tbase = tmem + ((uint32_t)(quarter * 32) << 16) + b * KN_N + c0;
+                // the candidates' ids and norms of stage s, seen through its
+                // barrier (complete: the MMAs that filled TFULL waited for it)
+                auto info_ready = [&]() { return mbar_wait(FULL(s), ph, S.status, abort_flag); };
+                uint32_t u[4][32];
+                float m[4];
+                __syncwarp();
+#pragma unroll
+                for (int g = 0; g < 4; ++g) tmem_ld32_min_async(tbase + g * 32, u[g], m[g]);
+                tmem_wait_ld();
+#pragma unroll
+                for (int g = 0; g < 4; ++g) reg_fence(u[g], m[g]);
+                // the values are in registers: the buffer goes back to the MMA
+                // warp now, so that selection overlaps the next tile's MMAs
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) {
-                    mbar_arrive(TEMPTY(b));
-                    mbar_arrive(EMPTY(s));
+                if (lane == 0) mbar_arrive(TEMPTY(b));
+                if (DUMP && rc.qid >= 0) {
+#pragma unroll
+                    for (int g = 0; g < 4; ++g) {
+                        float* dst = S.dump + (int64_t)S.qidx[slot] * S.npad + ct * KN_N + c0 + g * 32;
+#pragma unroll
+                        for (int i = 0; i < 32; ++i) dst[i] = __uint_as_float(u[g][i]);
+                    }
                 }
+                if constexpr (MODE == SEED) {
+                    float v[4];
+#pragma unroll
+                    for (int g = 0; g < 4; ++g) v[g] = seed_exact(m[g]);
+                    if (!fast && info_ready()) {
+#pragma unroll
+                        for (int g = 0; g < 4; ++g)
+                            v[g] = seed_bounded(rc, u[g], cid + g * 32, cnrm + g * 32, cncf + g * 32);
+                    }
+#pragma unroll
+                    for (int i = 0; i < SEED_T * 4; ++i)
+                        if (turn == i / 4) acc[i] = fminf(acc[i], v[i & 3]);
+                    turn = turn + 1 == SEED_T ? 0 : turn + 1;
+                } else if (fast) {                        // warp-uniform
+                    const bool live = rc.qid >= 0;
+                    const float mt = live ? r.thr : -__int_as_float(0x7f800000);
+                    if (__any_sync(0xffffffffu, fminf(fminf(m[0], m[1]), fminf(m[2], m[3])) < mt) &&
+                        __all_sync(0xffffffffu, info_ready())) {
+#pragma unroll
+                        for (int g = 0; g < 4; ++g)
+                            if (__any_sync(0xffffffffu, live && m[g] < r.thr))
+                                r = select_exact(r, rc, u[g], cid + g * 32, live, mylist - lane * (KN_SPLIT * KN_KMAX));
+                    }
+                } else if (rc.qid >= 0 && info_ready()) {
+#pragma unroll
+                    for (int g = 0; g < 4; ++g)
+                        r = select_bounded(r, rc, u[g], cid + g * 32, cnrm + g * 32, cncf + g * 32,
+                                           ct * KN_N + c0 + g * 32, S.nexact);
+                }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(EMPTY(s));
             }
             if (!ok) break;
-            for (int i = 0; i < S.k; ++i)
-                S.lists[state * S.k + i] = i < r.n ? mylist[i] : make_float2(0.f, __int_as_float(-1));
-            S.scount[state] = r.scount;
+            if constexpr (MODE == SEED) {
+                float* out = S.smin + state * S.seed_keys;
+                float g4[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    g4[i] = acc[i];
+#pragma unroll
+                    for (int t = 1; t < SEED_T; ++t) g4[i] = fminf(g4[i], acc[t * 4 + i]);
+                }
+                if (S.seed_keys == SEED_T * 4) {
+#pragma unroll
+                    for (int i = 0; i < SEED_T * 4; ++i) out[i] = acc[i];
+                } else if (S.seed_keys == 4) {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) out[i] = g4[i];
+                } else {
+                    out[0] = fminf(fminf(g4[0], g4[1]), fminf(g4[2], g4[3]));
+                }
+            } else {
+                for (int i = 0; i < S.k; ++i)
+                    S.lists[state * S.k + i] = i < r.n ? mylist[i] : make_float2(0.f, __int_as_float(-1));
+                S.scount[state] = r.scount;
+            }
         }
     }
     tc_fence_before();
@@ -712,22 +908,29 @@ __device__ __forceinline__ bool pair_less(uint64_t d1, int i1, uint64_t d2, int 
     return d1 < d2 || (d1 == d2 && i1 < i2);
 }
 
+constexpr int RERANK_ALL = (KN_SPLIT * (KN_KMAX + KN_SCAP) + 31) / 32, RERANK_FEW = 2;
+
 // One warp per (query slot, candidate range): exact distances of every kept
 // candidate, top-k of the range. With one range per query the rows go to the
 // output; otherwise to part_d2 / part_id ([qpad][nchunk][k]) for chunk_merge.
+// PER: candidates held per lane, the first 32 * PER of the query's; a launch
+// with PER = 1 leaves the queries that keep more to one with every candidate.
+template <int PER>
 __global__ void rerank_kernel(const uint32_t* __restrict__ theta_q, const uint32_t* __restrict__ theta_c, int D,
                               const int32_t* __restrict__ qv,
-                              const int32_t* __restrict__ qidx, int64_t qpad, int64_t nchunk, int k,
+                              const int32_t* __restrict__ qidx, int64_t qpad, Split W, int k,
                               const float2* __restrict__ lists, const int32_t* __restrict__ shortlist,
                               const int32_t* __restrict__ scount, const int* __restrict__ overflow,
                               int32_t* __restrict__ out_ids, uint64_t* __restrict__ out_d2,
                               int32_t* __restrict__ part_id, uint64_t* __restrict__ part_d2) {
     const int64_t grp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
+    const int64_t nchunk = W.nseg;
     if (grp >= qpad * nchunk) return;
     const int64_t slot = grp / nchunk;
     const int32_t v = qv[slot];
     if (v < 0 || overflow[slot]) return;   // padding, or handled by the brute-force fallback
+    if (grp % nchunk >= W.segments(slot / KN_M)) return;   // the tile has fewer segments
     int32_t* oid = nchunk == 1 ? out_ids + (int64_t)qidx[slot] * k : part_id + grp * k;
     uint64_t* od = nchunk == 1 ? out_d2 + (int64_t)qidx[slot] * k : part_d2 + grp * k;
     // candidates: the lists of the column slices, then their shortlists
@@ -740,8 +943,7 @@ __global__ void rerank_kernel(const uint32_t* __restrict__ theta_q, const uint32
     }
     const int nl = KN_SPLIT * k;
     const int total = nl + nst;
-    // each lane holds up to ceil(total/32) candidates
-    constexpr int PER = (KN_SPLIT * (KN_KMAX + KN_SCAP) + 31) / 32;
+    if (PER < RERANK_ALL ? total > 32 * PER : total <= 32 * RERANK_FEW) return;
     uint64_t dd[PER];
     int id[PER];
 #pragma unroll
@@ -813,31 +1015,44 @@ __global__ void __launch_bounds__(256) chunk_merge_kernel(const int32_t* __restr
                                                           const int32_t* __restrict__ qidx,
                                                           const int* __restrict__ overflow,
                                                           const int32_t* __restrict__ slots, int64_t count,
-                                                          int64_t nchunk, int k, const int32_t* __restrict__ part_id,
+                                                          Split W, int64_t nchunk, int k,
+                                                          const int32_t* __restrict__ part_id,
                                                           const uint64_t* __restrict__ part_d2,
                                                           int32_t* __restrict__ out_ids,
                                                           uint64_t* __restrict__ out_d2) {
-    __shared__ uint64_t sd[8];
-    __shared__ int si[8];
+    __shared__ uint64_t sd[2][8];
+    __shared__ int si[2][8];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t total = nchunk * k;
+    constexpr int HELD = 8;                           // entries kept in registers per thread
     for (int64_t e = blockIdx.x; e < count; e += gridDim.x) {
         const int64_t slot = slots ? slots[e] : e;
         if (qv[slot] < 0 || (!slots && overflow[slot])) continue;
-        const int64_t qi = qidx[slot], base = e * total;
+        const int64_t qi = qidx[slot], base = e * nchunk * k;
+        const int64_t total = (slots ? nchunk : W.segments(slot / KN_M)) * k;
+        uint64_t hd[HELD];
+        int hi[HELD];
+#pragma unroll
+        for (int j = 0; j < HELD; ++j) {
+            const int64_t t = threadIdx.x + 256 * j;
+            hi[j] = t < total ? part_id[base + t] : -1;
+            hd[j] = hi[j] >= 0 ? part_d2[base + t] : ~0ull;
+        }
         uint64_t lastd = 0;
         int lasti = -1;
         for (int r = 0; r < k; ++r) {
             uint64_t bd = ~0ull;
             int bi = 0x7fffffff;
-            for (int64_t t = threadIdx.x; t < total; t += 256) {
-                const int id = part_id[base + t];
-                if (id < 0) continue;
-                const uint64_t d = part_d2[base + t];
-                if ((r == 0 || pair_less(lastd, lasti, d, id)) && pair_less(d, id, bd, bi)) {
+            auto offer = [&](uint64_t d, int id) {
+                if (id >= 0 && (r == 0 || pair_less(lastd, lasti, d, id)) && pair_less(d, id, bd, bi)) {
                     bd = d;
                     bi = id;
                 }
+            };
+#pragma unroll
+            for (int j = 0; j < HELD; ++j) offer(hd[j], hi[j]);
+            for (int64_t t = threadIdx.x + 256 * HELD; t < total; t += 256) {
+                const int id = part_id[base + t];
+                if (id >= 0) offer(part_d2[base + t], id);
             }
 #pragma unroll
             for (int o = 16; o; o >>= 1) {
@@ -849,25 +1064,74 @@ __global__ void __launch_bounds__(256) chunk_merge_kernel(const int32_t* __restr
                 }
             }
             if (lane == 0) {
-                sd[warp] = bd;
-                si[warp] = bi;
+                sd[r & 1][warp] = bd;
+                si[r & 1][warp] = bi;
             }
-            __syncthreads();
-            bd = sd[0];
-            bi = si[0];
+            __syncthreads();                          // (two buffers: one barrier a rank)
+            bd = sd[r & 1][0];
+            bi = si[r & 1][0];
 #pragma unroll
             for (int w = 1; w < 8; ++w)
-                if (pair_less(sd[w], si[w], bd, bi)) {
-                    bd = sd[w];
-                    bi = si[w];
+                if (pair_less(sd[r & 1][w], si[r & 1][w], bd, bi)) {
+                    bd = sd[r & 1][w];
+                    bi = si[r & 1][w];
                 }
-            __syncthreads();
             if (threadIdx.x == 0) {
                 out_ids[qi * k + r] = bi == 0x7fffffff ? -1 : bi;
                 out_d2[qi * k + r] = bi == 0x7fffffff ? ~0ull : bd;
             }
             lastd = bd;
             lasti = bi;
+        }
+        __syncthreads();
+    }
+}
+
+// the same with a warp per query slot, for at most 256 entries
+__global__ void __launch_bounds__(256) chunk_merge_warp_kernel(const int32_t* __restrict__ qv,
+                                                               const int32_t* __restrict__ qidx,
+                                                               const int* __restrict__ overflow, int64_t qpad, Split W,
+                                                               int k, const int32_t* __restrict__ part_id,
+                                                               const uint64_t* __restrict__ part_d2,
+                                                               int32_t* __restrict__ out_ids,
+                                                               uint64_t* __restrict__ out_d2) {
+    const int64_t slot = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    if (slot >= qpad || qv[slot] < 0 || overflow[slot]) return;      // warp-uniform
+    const int64_t qi = qidx[slot], base = slot * W.nseg * k;
+    const int total = (int)W.segments(slot / KN_M) * k;
+    constexpr int HELD = 8;
+    uint64_t hd[HELD];
+    int hi[HELD];
+#pragma unroll
+    for (int j = 0; j < HELD; ++j) {
+        const int t = lane + 32 * j;
+        hi[j] = t < total ? part_id[base + t] : -1;
+        hd[j] = hi[j] >= 0 ? part_d2[base + t] : ~0ull;
+    }
+    for (int r = 0; r < k; ++r) {
+        uint64_t bd = ~0ull;
+        int bi = 0x7fffffff;
+#pragma unroll
+        for (int j = 0; j < HELD; ++j)
+            if (hi[j] >= 0 && pair_less(hd[j], hi[j], bd, bi)) {
+                bd = hd[j];
+                bi = hi[j];
+            }
+#pragma unroll
+        for (int o = 16; o; o >>= 1) {
+            const uint64_t od = __shfl_xor_sync(0xffffffffu, bd, o);
+            const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+            if (pair_less(od, oi, bd, bi)) {
+                bd = od;
+                bi = oi;
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < HELD; ++j) hi[j] = hi[j] == bi ? -1 : hi[j];   // ids are distinct
+        if (lane == 0) {
+            out_ids[qi * k + r] = bi == 0x7fffffff ? -1 : bi;
+            out_d2[qi * k + r] = bi == 0x7fffffff ? ~0ull : bd;
         }
     }
 }
@@ -932,41 +1196,162 @@ __global__ void __launch_bounds__(256) brute_warp_kernel(const uint32_t* __restr
     }
 }
 
-// query slots: exact queries first (stable), padded to a multiple of 128
-__global__ void query_slots_kernel(const int32_t* __restrict__ queries, int64_t q, const uint8_t* __restrict__ exact,
-                                   int64_t n, const int64_t* __restrict__ exscan, int64_t nexq,
-                                   int32_t* __restrict__ qv, int32_t* __restrict__ qidx, uint32_t* status) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= q) return;
-    int32_t v = queries ? queries[i] : (int32_t)i;
-    bool bad = v < 0 || v >= n;
-    if (bad) flag_status(status, ST_BAD_QUERY);
-    bool e = bad ? true : exact[v] != 0;
-    int64_t p = e ? exscan[i] : nexq + (i - exscan[i]);
-    qv[p] = bad ? -1 : v;
-    qidx[p] = (int32_t)i;
+// query slots: exact queries first (stable), padded to a multiple of 128.
+// exscan = exclusive scan of the queries' exact flags (an out-of-range query
+// counts as exact); the number of exact queries is read off its last entry, so
+// the host does not wait for it. Also each slot's query information.
+struct QuerySlots {
+    int32_t* qv;             // [qpad] query vertex (-1: padding or not a vertex)
+    int32_t* qidx;           // [qpad] query index
+    uint8_t* qexact;         // [qpad]
+    float* qnrm;             // [qpad]
+    int* overflow;           // [qpad], cleared
+    unsigned long long* sums;   // [0] kept pairs, [1] overflowed queries, cleared
+};
+
+__device__ __forceinline__ bool exact_query(int32_t v, const uint8_t* exact, int64_t n) {
+    return v < 0 || v >= n || exact[v] != 0;
 }
 
-__global__ void query_info_kernel(const int32_t* __restrict__ qv, int64_t qpad, const uint8_t* __restrict__ exact,
-                                  const float* __restrict__ nrm, uint8_t* __restrict__ qexact, float* __restrict__ qnrm) {
-    int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= qpad) return;
-    int32_t v = qv[s];
-    qexact[s] = v < 0 ? 1 : exact[v];
-    qnrm[s] = v < 0 ? 0.f : nrm[v];
+__device__ __forceinline__ void put_slot(const QuerySlots& Q, int64_t p, int32_t v, int32_t i, bool bad,
+                                         const uint8_t* exact, const float* nrm) {
+    Q.qv[p] = bad ? -1 : v;
+    Q.qidx[p] = i;
+    Q.qexact[p] = bad ? 1 : exact[v];
+    Q.qnrm[p] = bad ? 0.f : nrm[v];
+}
+
+__global__ void query_slots_kernel(const int32_t* __restrict__ queries, int64_t q, int64_t qpad,
+                                   const uint8_t* __restrict__ exact, const float* __restrict__ nrm, int64_t n,
+                                   const int64_t* __restrict__ exscan, QuerySlots Q, uint32_t* status) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= qpad) return;
+    Q.overflow[i] = 0;
+    if (i < 2) Q.sums[i] = 0;
+    if (i >= q) {
+        put_slot(Q, i, -1, 0, true, exact, nrm);
+        return;
+    }
+    const int32_t lastv = queries ? queries[q - 1] : (int32_t)(q - 1);
+    const int64_t nexq = exscan[q - 1] + (exact_query(lastv, exact, n) ? 1 : 0);
+    const int32_t v = queries ? queries[i] : (int32_t)i;
+    const bool bad = v < 0 || v >= n;
+    if (bad) flag_status(status, ST_BAD_QUERY);
+    const int64_t p = exact_query(v, exact, n) ? exscan[i] : nexq + (i - exscan[i]);
+    put_slot(Q, p, v, (int32_t)i, bad, exact, nrm);
 }
 
 __global__ void exact_flags_of_queries(const int32_t* __restrict__ queries, int64_t q, const uint8_t* __restrict__ exact,
                                        int64_t n, int64_t* __restrict__ f) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= q) return;
-    int32_t v = queries ? queries[i] : (int32_t)i;
-    f[i] = (v < 0 || v >= n) ? 1 : exact[v];
+    f[i] = exact_query(queries ? queries[i] : (int32_t)i, exact, n) ? 1 : 0;
 }
 
-__global__ void fill_i32(int32_t* p, int64_t n, int32_t v) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) p[i] = v;
+// the same for up to SLOTS_SMALL queries, flags, scan, slots and tile flags in
+// one CTA instead of seven launches
+constexpr int SLOTS_SMALL = 4096;
+__global__ void __launch_bounds__(1024) query_slots_small_kernel(const int32_t* __restrict__ queries, int q, int qpad,
+                                                                 const uint8_t* __restrict__ exact,
+                                                                 const float* __restrict__ nrm, int64_t n,
+                                                                 QuerySlots Q, uint8_t* __restrict__ qtile,
+                                                                 uint32_t* status) {
+    __shared__ int wsum[32];
+    constexpr int PER = SLOTS_SMALL / 1024;
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    int32_t v[PER];
+    bool ex[PER];
+    int mine = 0;
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+        const int i = t * PER + j;
+        v[j] = i < q ? queries[i] : -1;
+        ex[j] = i < q && exact_query(v[j], exact, n);
+        mine += ex[j] ? 1 : 0;
+    }
+    int inc = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += y;
+    }
+    if (lane == 31) wsum[w] = inc;
+    for (int i = t; i < qpad; i += 1024) Q.overflow[i] = 0;
+    for (int i = t; i < qpad / KN_M; i += 1024) qtile[i] = 1;
+    if (t < 2) Q.sums[t] = 0;
+    __syncthreads();
+    int before = inc - mine, nexq = 0;
+    for (int i = 0; i < 32; ++i) {
+        before += i < w ? wsum[i] : 0;
+        nexq += wsum[i];
+    }
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+        const int i = t * PER + j;
+        if (i < q) {
+            const bool bad = v[j] < 0 || v[j] >= n;
+            if (bad) flag_status(status, ST_BAD_QUERY);
+            const int p = ex[j] ? before : nexq + (i - before);
+            put_slot(Q, p, v[j], i, bad, exact, nrm);
+            if (!ex[j]) qtile[p / KN_M] = 0;
+            before += ex[j] ? 1 : 0;
+        }
+    }
+    for (int i = q + t; i < qpad; i += 1024) put_slot(Q, i, -1, 0, true, exact, nrm);
+}
+
+// thr0[slot] = the (k+1)-th smallest of the slot's sample minima (of disjoint
+// candidate sets; at most one is the query itself), +inf when there are fewer:
+// an upper bound of the k-th key over all candidates. A warp per slot, at most
+// 512 minima (seed_keys per segment and column slice).
+__global__ void __launch_bounds__(256) seed_bound_kernel(const float* __restrict__ smin, int64_t qpad, Split W,
+                                                         int seed_keys, int k, float* __restrict__ thr0) {
+    const int64_t slot = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    if (slot >= qpad) return;                        // warp-uniform
+    constexpr int PER = 16;
+    const int total = (int)W.segments(slot / KN_M) * KN_SPLIT * seed_keys;
+    const float* mine = smin + slot * W.nseg * KN_SPLIT * seed_keys;
+    const float inf = __int_as_float(0x7f800000);
+    float key[PER];
+#pragma unroll
+    for (int j = 0; j < PER; ++j) key[j] = lane + 32 * j < total ? mine[lane + 32 * j] : inf;
+    // k+1 times the smallest; equal ones count one by one (the lowest lane that
+    // holds it drops one)
+    float best = inf;
+    for (int r = 0; r <= k; ++r) {
+        float m = inf;
+#pragma unroll
+        for (int j = 0; j < PER; ++j) m = fminf(m, key[j]);
+        best = m;
+#pragma unroll
+        for (int o = 16; o; o >>= 1) best = fminf(best, __shfl_xor_sync(0xffffffffu, best, o));
+        if (best == inf) break;                      // warp-uniform
+        const unsigned have = __ballot_sync(0xffffffffu, m == best);
+        if (lane == __ffs(have) - 1) {
+            bool gone = false;
+#pragma unroll
+            for (int j = 0; j < PER; ++j)
+                if (!gone && key[j] == best) {
+                    key[j] = inf;
+                    gone = true;
+                }
+        }
+    }
+    if (lane == 0) thr0[slot] = best;
+}
+
+// kept pairs and overflowed slots of a call (their order does not matter)
+__global__ void knn_sums_kernel(const int32_t* __restrict__ scount, int64_t nstate, const int* __restrict__ overflow,
+                                int64_t qpad, unsigned long long* __restrict__ sums, int32_t* __restrict__ ovslots) {
+    unsigned long long kept = 0;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nstate; i += (int64_t)gridDim.x * blockDim.x) {
+        kept += (unsigned)scount[i];
+        if (i < qpad && overflow[i]) ovslots[atomicAdd(&sums[1], 1ull)] = (int32_t)i;
+    }
+#pragma unroll
+    for (int o = 16; o; o >>= 1) kept += __shfl_xor_sync(0xffffffffu, kept, o);
+    if ((threadIdx.x & 31) == 0 && kept) atomicAdd(&sums[0], kept);
 }
 
 }  // namespace
@@ -1038,7 +1423,7 @@ extern "C" panther_status pantherpp_vectors(panther_ctx* ctx, const panther_inde
         return fail(st);
     PCK(ctx, cudaMemsetAsync(maxv, 0, 4, s));
     unsigned gb = (unsigned)ceil_div(n, 256);
-    vec_stats_kernel<<<gb, 256, 0, s>>>(v->theta, n, D, v->norm2, v->nrm, v->exact, flag, maxv);
+    vec_stats_kernel<<<(unsigned)std::min<int64_t>(ceil_div(n, 32), (int64_t)ctx->num_sms * 16), 256, 0, s>>>(v->theta, n, D, v->norm2, v->nrm, v->exact, flag, maxv);
     ctx->launches++;
     // number of exact rows = sum of flags (read before the scan overwrites them)
     if ((st = scan_exclusive_i64(ctx, flag, n))) return fail(st);
@@ -1066,10 +1451,10 @@ extern "C" panther_status pantherpp_vectors(panther_ctx* ctx, const panther_inde
         return fail(st);
     }
     vec_perm_kernel<<<gb, 256, 0, s>>>(v->exact, flag, n, x.nexact, perm, pos);
-    vec_brow_kernel<<<(unsigned)ceil_div(x.npad, 256), 256, 0, s>>>(v->theta, v->norm2, v->nrm, perm,
+    vec_brow_kernel<<<(unsigned)ceil_div(x.npad, 32), 256, 0, s>>>(v->theta, v->norm2, v->nrm, perm,
                                                                     VecMeta{n, x.npad, x.nexact, D}, x.B, x.cid,
                                                                     x.cnrm, x.cncf);
-    tile_flags_kernel<<<(unsigned)ceil_div(x.npad / KN_N, 256), 256, 0, s>>>(v->exact, x.cid, x.npad, KN_N, x.ctile,
+    tile_flags_kernel<<<(unsigned)ceil_div(x.npad / KN_N, 8), 256, 0, s>>>(v->exact, x.cid, x.npad, KN_N, x.ctile,
                                                                              x.npad / KN_N);
     ctx->launches += 3;
     dev_free(ctx, perm);
@@ -1085,25 +1470,39 @@ extern "C" panther_status pantherpp_vectors(panther_ctx* ctx, const panther_inde
     return PANTHER_OK;
 }
 
-// Candidate ranges per query tile: with fewer query tiles than SMs, the
-// candidate tiles are cut into ranges so that tiles x ranges work items fill
-// the GPU; the choice minimises waves x range length, at least KN_STAGES
-// candidate tiles per range (both forms).
-static int64_t knn_ranges(int64_t nqt, int64_t nct, int num_sms, bool fp32) {
-    (void)fp32;   // both forms cut the candidates the same way
-    if (nqt >= num_sms) return 1;
+// The BF16 screen's work in equal runs, one per CTA, of at least KN_STAGES
+// candidate tiles. From 16 query tiles per SM on, whole tiles per CTA: the last
+// wave then costs at most 6%, and every segment more of a tile costs lists and
+// a shortlist of 2 KB per query.
+static Split knn_split(int64_t nqt, int64_t nct, int num_sms) {
+    Split W{nqt, nct, 0, 1};
+    if (nqt >= 16 * (int64_t)num_sms) return W;
+    W.G = std::max<int64_t>(1, std::min<int64_t>(num_sms, nqt * nct / KN_STAGES));
+    for (int64_t t = 0; t < nqt; ++t) W.nseg = std::max(W.nseg, W.segments(t));
+    return W;
+}
+
+// The FP32 form's candidate ranges: with fewer query tiles than SMs the choice
+// minimises waves x range length, at least KN_STAGES candidate tiles per range.
+static Split knn_ranges(int64_t nqt, int64_t nct, int num_sms) {
+    Split W{nqt, nct, 0, 1};
+    if (nqt >= num_sms) return W;
     const int64_t pmax = std::max<int64_t>(1, std::min<int64_t>(nct / KN_STAGES, 256));
-    int64_t best = 1;
     double best_cost = (double)ceil_div(nqt, num_sms);
     for (int64_t p = 2; p <= pmax; ++p) {
-        double cost = (double)ceil_div(nqt * p, num_sms) / (double)p;
+        const double cost = (double)ceil_div(nqt * p, num_sms) / (double)p;
         if (cost < best_cost * 0.999) {
-            best = p;
+            W.nseg = p;
             best_cost = cost;
         }
     }
-    return best;
+    return W;
 }
+
+// Candidate tiles of the sample that bounds the k-th keys (0: none): a 32nd,
+// a 16th of fewer than 2,048, none below 128 tiles (32,768 candidates), where
+// the screen itself is as short.
+static int64_t seed_tiles(int64_t nct) { return nct < 128 ? 0 : nct / (nct < 2048 ? 16 : 32); }
 
 // queries are vertices of vq, candidates every vertex of vc; `same` excludes
 // the candidate with the query's id (one graph: the query itself)
@@ -1114,140 +1513,155 @@ static panther_status knn_run(panther_ctx* ctx, const pantherpp_vecs* vq, const 
     const pantherpp_vecs* v = vq;
     cudaStream_t s = ctx->stream;
     const int64_t n = vq->n;
-    const int64_t qpad = ceil_div(q, KN_M) * KN_M;
-    const int64_t nch = knn_ranges(qpad / KN_M, x.npad / KN_N, ctx->num_sms, fp32);
+    const int64_t qpad = ceil_div(q, KN_M) * KN_M, nqt = qpad / KN_M, nct = x.npad / KN_N;
+    const Split W = fp32 ? knn_ranges(nqt, nct, ctx->num_sms) : knn_split(nqt, nct, ctx->num_sms);
+    const int64_t nch = W.nseg;
+    const int64_t ns = (fp32 || dump) ? 0 : seed_tiles(nct);
+    const Split WS = ns ? knn_split(nqt, ns, ctx->num_sms) : W;
+    // minima per segment and column slice: at most 512 a query, at least 40
+    const int seed_keys = WS.nseg <= 12 ? SEED_T * 4 : WS.nseg <= 64 ? 4 : 1;
     panther_status st;
     int64_t* qf = nullptr;
-    int32_t *qv = nullptr, *qidx = nullptr, *sl = nullptr, *sc = nullptr, *pid = nullptr;
-    int* ovf = nullptr;
-    uint8_t *qex = nullptr, *qtile = nullptr;
-    float* qn = nullptr;
+    int32_t *sl = nullptr, *sc = nullptr, *pid = nullptr, *ovs = nullptr;
+    uint8_t* qtile = nullptr;
     float2* lists = nullptr;
+    float *smin = nullptr, *thr0 = nullptr;
     uint16_t* A = nullptr;
     uint64_t* pd = nullptr;
+    QuerySlots Q{};
     auto cleanup = [&]() {
-        dev_free(ctx, qf); dev_free(ctx, qv); dev_free(ctx, qidx); dev_free(ctx, sl); dev_free(ctx, sc);
-        dev_free(ctx, ovf); dev_free(ctx, qex); dev_free(ctx, qtile); dev_free(ctx, qn); dev_free(ctx, lists);
-        dev_free(ctx, A); dev_free(ctx, pid); dev_free(ctx, pd);
+        dev_free(ctx, qf); dev_free(ctx, Q.qv); dev_free(ctx, Q.qidx); dev_free(ctx, sl); dev_free(ctx, sc);
+        dev_free(ctx, Q.overflow); dev_free(ctx, Q.qexact); dev_free(ctx, qtile); dev_free(ctx, Q.qnrm);
+        dev_free(ctx, lists); dev_free(ctx, smin); dev_free(ctx, thr0); dev_free(ctx, A); dev_free(ctx, pid);
+        dev_free(ctx, pd); dev_free(ctx, ovs); dev_free(ctx, Q.sums);
     };
     const int64_t nstate = qpad * nch * KN_SPLIT;
-    if ((st = dev_alloc(ctx, (void**)&qf, sizeof(int64_t) * q)) ||
-        (st = dev_alloc(ctx, (void**)&qv, sizeof(int32_t) * qpad)) ||
-        (st = dev_alloc(ctx, (void**)&qidx, sizeof(int32_t) * qpad)) ||
+    const bool small = q <= SLOTS_SMALL && queries;
+    if ((!small && (st = dev_alloc(ctx, (void**)&qf, sizeof(int64_t) * q))) ||
+        (st = dev_alloc(ctx, (void**)&Q.qv, sizeof(int32_t) * qpad)) ||
+        (st = dev_alloc(ctx, (void**)&Q.qidx, sizeof(int32_t) * qpad)) ||
         (st = dev_alloc(ctx, (void**)&sl, sizeof(int32_t) * nstate * KN_SCAP)) ||
         (st = dev_alloc(ctx, (void**)&sc, sizeof(int32_t) * nstate)) ||
-        (st = dev_alloc(ctx, (void**)&ovf, sizeof(int) * qpad)) || (st = dev_alloc(ctx, (void**)&qex, qpad)) ||
-        (st = dev_alloc(ctx, (void**)&qtile, qpad / KN_M)) || (st = dev_alloc(ctx, (void**)&qn, sizeof(float) * qpad)) ||
+        (st = dev_alloc(ctx, (void**)&Q.overflow, sizeof(int) * qpad)) ||
+        (st = dev_alloc(ctx, (void**)&ovs, sizeof(int32_t) * qpad)) ||
+        (st = dev_alloc(ctx, (void**)&Q.sums, 2 * sizeof(unsigned long long))) ||
+        (st = dev_alloc(ctx, (void**)&Q.qexact, qpad)) || (st = dev_alloc(ctx, (void**)&qtile, nqt)) ||
+        (st = dev_alloc(ctx, (void**)&Q.qnrm, sizeof(float) * qpad)) ||
         (st = dev_alloc(ctx, (void**)&lists, sizeof(float2) * nstate * k)) ||
         (nch > 1 && ((st = dev_alloc(ctx, (void**)&pid, sizeof(int32_t) * qpad * nch * k)) ||
                      (st = dev_alloc(ctx, (void**)&pd, sizeof(uint64_t) * qpad * nch * k)))) ||
+        (ns && ((st = dev_alloc(ctx, (void**)&smin, sizeof(float) * qpad * WS.nseg * KN_SPLIT * seed_keys)) ||
+                (st = dev_alloc(ctx, (void**)&thr0, sizeof(float) * qpad)))) ||
         (!fp32 && (st = dev_alloc(ctx, (void**)&A, (size_t)qpad * KN_K * 2)))) {
         cleanup();
         return st;
     }
-    unsigned gq = (unsigned)ceil_div(q, 256), gp = (unsigned)ceil_div(qpad, 256);
-    exact_flags_of_queries<<<gq, 256, 0, s>>>(queries, q, v->exact, n, qf);
-    if ((st = scan_exclusive_i64(ctx, qf, q))) { cleanup(); return st; }
-    // number of exact queries: recompute the last flag on the host side of the scan
-    int64_t last = 0;
-    int32_t lastq = 0;
-    PCK(ctx, cudaMemcpyAsync(&last, qf + q - 1, 8, cudaMemcpyDeviceToHost, s));
-    if (queries) PCK(ctx, cudaMemcpyAsync(&lastq, queries + q - 1, 4, cudaMemcpyDeviceToHost, s));
-    else lastq = (int32_t)(q - 1);
-    PCK(ctx, cudaStreamSynchronize(s));
-    uint8_t lastex = 1;
-    if (lastq >= 0 && lastq < n) {
-        PCK(ctx, cudaMemcpyAsync(&lastex, v->exact + lastq, 1, cudaMemcpyDeviceToHost, s));
-        PCK(ctx, cudaStreamSynchronize(s));
+    if (small) {
+        query_slots_small_kernel<<<1, 1024, 0, s>>>(queries, (int)q, (int)qpad, v->exact, v->nrm, n, Q, qtile,
+                                                    ctx->d_status);
+        ctx->launches++;
+    } else {
+        exact_flags_of_queries<<<(unsigned)ceil_div(q, 256), 256, 0, s>>>(queries, q, v->exact, n, qf);
+        if ((st = scan_exclusive_i64(ctx, qf, q))) { cleanup(); return st; }
+        query_slots_kernel<<<(unsigned)ceil_div(qpad, 256), 256, 0, s>>>(queries, q, qpad, v->exact, v->nrm, n, qf, Q,
+                                                                         ctx->d_status);
+        tile_flags_kernel<<<(unsigned)ceil_div(nqt, 8), 256, 0, s>>>(v->exact, Q.qv, qpad, KN_M, qtile, nqt);
+        ctx->launches += 3;
     }
-    const int64_t nexq = last + lastex;
-    fill_i32<<<gp, 256, 0, s>>>(qv, qpad, -1);
-    fill_i32<<<gp, 256, 0, s>>>(qidx, qpad, 0);
-    PCK(ctx, cudaMemsetAsync(ovf, 0, sizeof(int) * qpad, s));
-    query_slots_kernel<<<gq, 256, 0, s>>>(queries, q, v->exact, n, qf, nexq, qv, qidx, ctx->d_status);
-    query_info_kernel<<<gp, 256, 0, s>>>(qv, qpad, v->exact, v->nrm, qex, qn);
-    tile_flags_kernel<<<(unsigned)ceil_div(qpad / KN_M, 256), 256, 0, s>>>(v->exact, qv, qpad, KN_M, qtile,
-                                                                           qpad / KN_M);
-    ctx->launches += 6;
+    PCK(ctx, cudaMemsetAsync(sc, 0, sizeof(int32_t) * nstate, s));
     if (!fp32) {
-        vec_arow_kernel<<<gp, 256, 0, s>>>(v->theta, qv, qpad, v->D, A);
+        vec_arow_kernel<<<(unsigned)ceil_div(qpad, 8), 256, 0, s>>>(v->theta, Q.qv, qpad, v->D, A);
         ctx->launches++;
         CUtensorMap tmA, tmB;
         if (!make_map(ctx, &tmA, A, qpad, KN_M) || !make_map(ctx, &tmB, x.B, x.npad, KN_N)) {
             cleanup();
             return PANTHER_ECUDA;
         }
-        ScreenArgs S{x.cid, x.cnrm, x.cncf, x.ctile, x.npad / KN_N, x.nexact, qv, qn, qex, qtile, qpad / KN_M,
-                     nch, k, lists, sl, sc, ovf, ctx->d_status, same, dump, qidx, x.npad};
-        int64_t grid = std::min<int64_t>(qpad / KN_M * nch, ctx->num_sms);
+        ScreenArgs S{x.cid, x.cnrm, x.cncf, x.ctile, W, 0, 0, nullptr, x.nexact, Q.qv, Q.qnrm, Q.qexact, qtile,
+                     k, lists, sl, sc, nullptr, 0, Q.overflow, ctx->d_status, same, dump, Q.qidx, x.npad};
+        auto grid = [&](const Split& w) {
+            return (unsigned)(w.G ? w.G : std::min<int64_t>(nqt, ctx->num_sms));
+        };
         if (dump) {
-            PCK(ctx, cudaFuncSetAttribute(screen_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+            PCK(ctx, cudaFuncSetAttribute(screen_kernel<DUMP_FORM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                           (int)KN_SMEM_BYTES));
-            screen_kernel<true><<<(unsigned)grid, KN_THREADS, KN_SMEM_BYTES, s>>>(tmA, tmB, S);
+            screen_kernel<DUMP_FORM><<<grid(W), KN_THREADS, KN_SMEM_BYTES, s>>>(tmA, tmB, S);
         } else {
-            PCK(ctx, cudaFuncSetAttribute(screen_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+            PCK(ctx, cudaFuncSetAttribute(screen_kernel<SCREEN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                           (int)KN_SMEM_BYTES));
-            screen_kernel<false><<<(unsigned)grid, KN_THREADS, KN_SMEM_BYTES, s>>>(tmA, tmB, S);
+            if (ns) {
+                PCK(ctx, cudaFuncSetAttribute(screen_kernel<SEED>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                              (int)KN_SMEM_BYTES));
+                ScreenArgs SS = S;
+                SS.W = WS;
+                SS.seed_step = (uint32_t)(nct / ns);
+                SS.seed_mul = (uint32_t)std::max<int64_t>(1, ns * 618 / 1000);   // coprime to ns: a permutation
+                while (std::gcd(SS.seed_mul, (uint32_t)ns) != 1) ++SS.seed_mul;
+                SS.smin = smin;
+                SS.seed_keys = seed_keys;
+                screen_kernel<SEED><<<grid(WS), KN_THREADS, KN_SMEM_BYTES, s>>>(tmA, tmB, SS);
+                seed_bound_kernel<<<(unsigned)ceil_div(qpad, 8), 256, 0, s>>>(smin, qpad, WS, seed_keys, k, thr0);
+                ctx->launches += 2;
+                S.thr0 = thr0;
+            }
+            screen_kernel<SCREEN><<<grid(W), KN_THREADS, KN_SMEM_BYTES, s>>>(tmA, tmB, S);
         }
         ctx->launches++;
     } else {
+        const dim3 fg((unsigned)(qpad / F_T), (unsigned)nch);
         if (v->D <= KN_K)
-            fp32_kernel<64><<<dim3((unsigned)(qpad / F_T), (unsigned)nch), F_T, 0, s>>>(vq->theta, vc->theta, same, v->D, qv, qex, qn, qpad,
-                                                            x.nexact, x.cid,
-                                                            x.cnrm, x.cncf, x.npad, k, lists, sl, sc, ovf);
+            fp32_kernel<64><<<fg, F_T, 0, s>>>(vq->theta, vc->theta, same, v->D, Q.qv, Q.qexact, Q.qnrm, qpad,
+                                               x.nexact, x.cid, x.cnrm, x.cncf, x.npad, k, lists, sl, sc, Q.overflow);
         else
-            fp32_kernel<128><<<dim3((unsigned)(qpad / F_T), (unsigned)nch), F_T, 0, s>>>(vq->theta, vc->theta, same, v->D, qv, qex, qn, qpad,
-                                                            x.nexact, x.cid,
-                                                            x.cnrm, x.cncf, x.npad, k, lists, sl, sc, ovf);
+            fp32_kernel<128><<<fg, F_T, 0, s>>>(vq->theta, vc->theta, same, v->D, Q.qv, Q.qexact, Q.qnrm, qpad,
+                                                x.nexact, x.cid, x.cnrm, x.cncf, x.npad, k, lists, sl, sc, Q.overflow);
         ctx->launches++;
     }
     PCK(ctx, cudaGetLastError());
-    rerank_kernel<<<(unsigned)ceil_div(qpad * nch * 32, 256), 256, 0, s>>>(vq->theta, vc->theta, v->D, qv, qidx,
-                                                                            qpad, nch, k,
-                                                                            lists, sl, sc, ovf, ids, d2, pid, pd);
+    // (every list fits 64 candidates; a query with a shortlist may keep more)
+    const unsigned rg = (unsigned)ceil_div(qpad * nch * 32, 256);
+    rerank_kernel<RERANK_FEW><<<rg, 256, 0, s>>>(vq->theta, vc->theta, v->D, Q.qv, Q.qidx, qpad, W, k, lists, sl, sc,
+                                                 Q.overflow, ids, d2, pid, pd);
+    rerank_kernel<RERANK_ALL><<<rg, 256, 0, s>>>(vq->theta, vc->theta, v->D, Q.qv, Q.qidx, qpad, W, k, lists, sl, sc,
+                                                 Q.overflow, ids, d2, pid, pd);
     ctx->launches++;
-    if (nch > 1) {
+    ctx->launches++;
+    if (nch > 1 && nch * k <= 256) {
+        chunk_merge_warp_kernel<<<(unsigned)ceil_div(qpad, 8), 256, 0, s>>>(Q.qv, Q.qidx, Q.overflow, qpad, W, k, pid,
+                                                                            pd, ids, d2);
+        ctx->launches++;
+    } else if (nch > 1) {
         chunk_merge_kernel<<<(unsigned)std::min<int64_t>(qpad, 8 * ctx->num_sms), 256, 0, s>>>(
-            qv, qidx, ovf, nullptr, qpad, nch, k, pid, pd, ids, d2);
+            Q.qv, Q.qidx, Q.overflow, nullptr, qpad, W, nch, k, pid, pd, ids, d2);
         ctx->launches++;
     }
+    knn_sums_kernel<<<(unsigned)std::min<int64_t>(ceil_div(nstate, 256), 4 * ctx->num_sms), 256, 0, s>>>(
+        sc, nstate, Q.overflow, qpad, Q.sums, ovs);
+    ctx->launches++;
     PCK(ctx, cudaGetLastError());
-    // screening statistics (pairs screened, kept for rerank, overflowed queries)
-    std::vector<int32_t> hsc(nstate);
-    std::vector<int> hov(qpad);
-    PCK(ctx, cudaMemcpyAsync(hsc.data(), sc, sizeof(int32_t) * nstate, cudaMemcpyDeviceToHost, s));
-    PCK(ctx, cudaMemcpyAsync(hov.data(), ovf, sizeof(int) * qpad, cudaMemcpyDeviceToHost, s));
+    // screening statistics: pairs kept for rerank, overflowed queries
+    unsigned long long* hsum = (unsigned long long*)ctx->h_counts;      // pinned
+    PCK(ctx, cudaMemcpyAsync(hsum, Q.sums, 2 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
     PCK(ctx, cudaStreamSynchronize(s));
-    int64_t kept = 0, over = 0;
-    std::vector<int32_t> hslots;
-    for (int64_t i = 0; i < nstate; ++i) kept += hsc[i];
-    for (int64_t i = 0; i < qpad; ++i)
-        if (hov[i]) hslots.push_back((int32_t)i);
-    over = (int64_t)hslots.size();
+    const int64_t kept = (int64_t)hsum[0], over = (int64_t)hsum[1];
     if (over) {
         // the overflowed queries: exact brute force over all vertices, spread over the GPU
         const int64_t nparts = std::max<int64_t>(1, std::min<int64_t>(1024, ceil_div(vc->n, 4096)));
-        int32_t* dsl = nullptr;
         int32_t* bid = nullptr;
         uint64_t* bd = nullptr;
-        auto bfree = [&]() { dev_free(ctx, dsl); dev_free(ctx, bid); dev_free(ctx, bd); };
-        if ((st = dev_alloc(ctx, (void**)&dsl, sizeof(int32_t) * over)) ||
-            (st = dev_alloc(ctx, (void**)&bid, sizeof(int32_t) * over * nparts * k)) ||
+        auto bfree = [&]() { dev_free(ctx, bid); dev_free(ctx, bd); };
+        if ((st = dev_alloc(ctx, (void**)&bid, sizeof(int32_t) * over * nparts * k)) ||
             (st = dev_alloc(ctx, (void**)&bd, sizeof(uint64_t) * over * nparts * k))) {
             bfree();
             cleanup();
             return st;
         }
-        cudaError_t ce = cudaMemcpyAsync(dsl, hslots.data(), sizeof(int32_t) * over, cudaMemcpyHostToDevice, s);
-        if (!ce) {
-            brute_warp_kernel<<<(unsigned)ceil_div(over * nparts * 32, 256), 256, 0, s>>>(
-                vq->theta, vc->theta, same, v->D, vc->n, qv, dsl, over, nparts, k, bid, bd);
-            chunk_merge_kernel<<<(unsigned)std::min<int64_t>(over, 8 * ctx->num_sms), 256, 0, s>>>(
-                qv, qidx, ovf, dsl, over, nparts, k, bid, bd, ids, d2);
-            ctx->launches += 2;
-            ce = cudaGetLastError();
-        }
-        if (!ce) ce = cudaStreamSynchronize(s);   // the host slot list must outlive the copy
+        brute_warp_kernel<<<(unsigned)ceil_div(over * nparts * 32, 256), 256, 0, s>>>(
+            vq->theta, vc->theta, same, v->D, vc->n, Q.qv, ovs, over, nparts, k, bid, bd);
+        chunk_merge_kernel<<<(unsigned)std::min<int64_t>(over, 8 * ctx->num_sms), 256, 0, s>>>(
+            Q.qv, Q.qidx, Q.overflow, ovs, over, W, nparts, k, bid, bd, ids, d2);
+        ctx->launches += 2;
+        const cudaError_t ce = cudaGetLastError();
         bfree();
         if (ce) {
             cleanup();
