@@ -306,7 +306,7 @@ PANTHER_API panther_status panther_set_topk_shape(panther_ctx* ctx, int threads,
 
 /* theta(v) = the D largest counts cnt(v,u), u != v, descending, zero padded,
  * for every vertex (Algorithm 2's loop over V), plus the device data the
- * k-NN search needs (for D <= 56 a BF16 copy padded to 64 columns; exact
+ * k-NN search needs (a BF16 copy padded to 64, 128 or 192 columns; exact
  * squared norms).
  *   1 <= D <= 128 (D > 64 counts through the top-k path for k > 64).
  *   Errors: EINVAL, ENOMEM, EOVERFLOW (max count^2 * D reaches 2^64, so a
@@ -328,8 +328,7 @@ PANTHER_API panther_status pantherpp_vecs_view(const pantherpp_vecs* v, const ui
  *          candidate the bound cannot rule out) or PANTHER_KNN_FP32 (FP32
  *          CUDA-core brute force with the same bound and rerank), optionally
  *          | PANTHER_IO_HOST.
- * Vectors wider than the BF16 screen's 56 columns (D > 56) take the FP32
- * screen (64 or 128 columns) under either flag, with the same exact rerank.
+ * The BF16 screen pads vectors to 64, 128 or 192 columns (D up to 56, 120, 128).
  * Every form returns the exact answer. Errors: EINVAL, ENOMEM, ECUDA. */
 PANTHER_API panther_status pantherpp_knn(panther_ctx* ctx, const pantherpp_vecs* v, const int32_t* queries,
                              int64_t q, int k, int32_t* out_ids, uint64_t* out_dist2, int flags);

@@ -7,18 +7,20 @@
 // Nearest neighbours. For query a and candidate b (integer vectors) the
 // squared distance is d = |a|^2 + y with y = |b|^2 - 2 a.b; ranking by d is
 // ranking by y. y is screened on the tensor cores:
-//   A row (query)      = [bf16(a_0..a_{D-1}), 1 x 8, 0 ...]         (64 columns)
+//   A row (query)      = [bf16(a_0..a_{D-1}), 1 x 8, 0 ...]
 //   B row (candidate)  = [-2 bf16(b_0..b_{D-1}), p_0 .. p_7, 0 ...]
 // where p_i = ((|b|^2 >> 8i) & 255) << 8i are the eight 8-bit pieces of the
-// exact squared norm (each exactly representable in BF16). One tcgen05.mma
-// chain (M=128 queries, N=256 candidates, K=64, FP32 accumulation in TMEM)
+// exact squared norm (each exactly representable in BF16). Rows have K = 64
+// columns for D <= 56, 128 for D <= 120 and 192 for D <= 128. One tcgen05.mma
+// chain (M=128 queries, N=256 candidates, K, FP32 accumulation in TMEM)
 // produces y_hat = |b|^2 - 2 a_hat.b_hat directly.
 //
-// Error bound. With u = 2^-8 (BF16 round to nearest), gamma = 2^-16 (64
+// Error bound. With u = 2^-8 (BF16 round to nearest), gamma = K * 2^-22 (K
 // additions at a conservative 2^-22 each) and s = a.b <= |a||b|:
 //   |y_hat - y| <= [2(2u+u^2) + 2 gamma (1+u)^2] |a||b| + gamma |b|^2
 // If every entry of a and of b is <= 256, the BF16 inputs are exact and every
-// partial sum is an integer of magnitude < 2^24, so y_hat = y exactly.
+// partial sum is an integer of magnitude at most 2 D 2^16 <= 2^24, so y_hat = y
+// exactly.
 //
 // Selection (two threads per query row of the tile, half of the columns each)
 // keeps the k best keys in shared memory: exact pairs insert (y, id); other
@@ -44,14 +46,20 @@ namespace {
 
 constexpr int KN_M = 128;          // queries per tile
 constexpr int KN_N = 256;          // candidates per tile
-constexpr int KN_K = 64;           // padded vector length (bf16)
-constexpr int KN_STAGES = 4;
+constexpr int KN_K = 64;           // columns of one operand block (128 bytes of bf16)
+constexpr int KN_INFO = 4;         // candidate-information stages (tiles)
+constexpr int KN_MIN_RUN = 4;      // candidate tiles per work item at least
+// operand blocks of a row: the entries and the eight pieces of the squared norm
+__host__ __device__ constexpr int kn_blocks(int D) { return (D + 8 + KN_K - 1) / KN_K; }
+// ring stages of one 32 KB candidate block each: as many as fit next to A
+__host__ __device__ constexpr int kn_stages(int kb) { return kb == 1 ? 4 : 3; }
 constexpr int KN_KMAX = 32;
 constexpr int KN_SCAP = 256;       // shortlist capacity per query
 constexpr int KN_SPLIT = 2;        // selection warps per TMEM lane quarter (each takes one column slice)
 constexpr int KN_THREADS = 64 + 128 * KN_SPLIT;   // warp 0 TMA, warp 1 MMA, then the selection warps
-constexpr float KN_ALPHA = 0.0157f;    // >= 2(2u+u^2) + 2 gamma (1+u)^2
-constexpr float KN_BETA = 1.6e-5f;     // >= gamma = 2^-16
+// >= 2(2u+u^2) + 2 gamma (1+u)^2 and >= gamma for K = 64, 128, 192
+__host__ __device__ constexpr float kn_alpha(int kb) { return kb == 1 ? 0.0157f : kb == 2 ? 0.01573f : 0.01576f; }
+__host__ __device__ constexpr float kn_beta(int kb) { return kb == 1 ? 1.6e-5f : kb == 2 ? 3.1e-5f : 4.6e-5f; }
 constexpr uint32_t MAX_EXACT = 256;
 
 struct VecMeta {
@@ -135,29 +143,29 @@ __global__ void __launch_bounds__(256) vec_brow_kernel(const uint32_t* __restric
                                                        uint16_t* __restrict__ B, int32_t* __restrict__ cid,
                                                        float* __restrict__ cnrm, float* __restrict__ cncf) {
     const int64_t p = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / 8;
-    const int sub = threadIdx.x & 7;
+    const int sub = threadIdx.x & 7, kb = kn_blocks(M.D);
     if (p >= M.npad) return;
     const bool pad = p >= M.n;
     const int32_t v = pad ? -1 : perm[p];
     const uint64_t n2 = pad ? 0 : norm2[v];
-    if (B) {                                         // no BF16 rows when D > 56 (FP32 form only)
+    for (int blk = 0; blk < kb; ++blk) {
         uint32_t c[8];
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
-            const int d = sub * 8 + j;
+            const int d = blk * KN_K + sub * 8 + j;
             c[j] = !pad && d < M.D ? theta[(int64_t)v * M.D + d] : 0u;
         }
         uint32_t out[4];
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
-            const int d = sub * 8 + j;
+            const int d = blk * KN_K + sub * 8 + j;
             float f = -2.0f * (float)round8(c[j]);
             if (pad) f = d == M.D ? 1099511627776.0f : 0.f;   // padding: y = 2^40 for every query, id -1
             else if (d >= M.D) f = d < M.D + 8 ? ldexpf((float)((n2 >> (8 * (d - M.D))) & 255ull), 8 * (d - M.D)) : 0.f;
             const uint32_t b = bf16_bits_of(f);
             out[j / 2] = j & 1 ? out[j / 2] | (b << 16) : b;
         }
-        ((uint4*)(B + p * KN_K))[sub] = make_uint4(out[0], out[1], out[2], out[3]);
+        ((uint4*)(B + (p * kb + blk) * KN_K))[sub] = make_uint4(out[0], out[1], out[2], out[3]);
     }
     if (sub == 0) {
         cid[p] = v;
@@ -171,7 +179,7 @@ __global__ void __launch_bounds__(256) vec_arow_kernel(const uint32_t* __restric
                                                        const int32_t* __restrict__ qv, int64_t qpad, int D,
                                                        uint16_t* __restrict__ A) {
     const int64_t s = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
+    const int lane = threadIdx.x & 31, kb = kn_blocks(D);
     if (s >= qpad) return;                           // warp-uniform
     const int32_t v = qv[s];
     auto col = [&](int d) -> uint32_t {
@@ -180,7 +188,10 @@ __global__ void __launch_bounds__(256) vec_arow_kernel(const uint32_t* __restric
         else if (v >= 0 && d < D + 8) f = 1.0f;
         return bf16_bits_of(f);
     };
-    ((uint32_t*)(A + s * KN_K))[lane] = col(2 * lane) | (col(2 * lane + 1) << 16);
+    for (int blk = 0; blk < kb; ++blk) {
+        const int d = blk * KN_K + 2 * lane;
+        ((uint32_t*)(A + (s * kb + blk) * KN_K))[lane] = col(d) | (col(d + 1) << 16);
+    }
 }
 
 // out[t] = every id of tile t is padding or an exact row (a warp per tile)
@@ -326,7 +337,8 @@ struct RowConst {
     int qid;         // query vertex (-1: padding row)
     int self;        // candidate id excluded from the answer (the query itself; -2 across graphs)
     bool exact;
-    float anrm;      // KN_ALPHA * |a| (BF16) or 2 eps |a| (FP32)
+    float anrm;      // kn_alpha * |a| (BF16) or 2 eps |a| (FP32)
+    float beta;      // kn_beta (BF16 only)
     float2* list;    // k entries {key, id bits}
     int32_t* sl;     // shortlist
     int* overflow;
@@ -382,7 +394,7 @@ __device__ __forceinline__ float seed_bounded(const RowConst& c, const uint32_t 
     float m = __int_as_float(0x7f800000);
 #pragma unroll
     for (int j = 0; j < 32; ++j) {
-        const float E = fmaf(c.anrm, cnrm[j], fmaf(KN_BETA, cncf[j], 1.0f)) * 1.0001f;
+        const float E = fmaf(c.anrm, cnrm[j], fmaf(c.beta, cncf[j], 1.0f)) * 1.0001f;
         if (cid[j] >= 0) m = fminf(m, __fadd_ru(__uint_as_float(y[j]), E));
     }
     return m;
@@ -451,7 +463,7 @@ __device__ __forceinline__ Row select_bounded(Row r, const RowConst& c, const ui
                                               const float* cnrm, const float* cncf, int64_t pos0, int64_t nexact) {
 #pragma unroll
     for (int j = 0; j < 32; ++j) {
-        const float E = fmaf(c.anrm, cnrm[j], fmaf(KN_BETA, cncf[j], 1.0f)) * 1.0001f;
+        const float E = fmaf(c.anrm, cnrm[j], fmaf(c.beta, cncf[j], 1.0f)) * 1.0001f;
         if (__fsub_rd(__uint_as_float(y[j]), E) <= r.thr)
             r = take_bounded(r, c, __uint_as_float(y[j]), E, cid[j], pos0 + j < nexact);
     }
@@ -528,13 +540,17 @@ struct ScreenArgs {
 };
 
 // shared memory map (offsets from a 1024-aligned base)
-constexpr uint32_t SM_A = 0;                                   // 16 KB
-constexpr uint32_t SM_B = SM_A + KN_M * KN_K * 2;              // KN_STAGES x 32 KB
-constexpr uint32_t SM_INFO = SM_B + KN_STAGES * KN_N * KN_K * 2;  // KN_STAGES x 3 KB
-constexpr uint32_t SM_LIST = SM_INFO + KN_STAGES * KN_N * 12;  // 128 x SPLIT x KMAX x 8 B
-constexpr uint32_t SM_BAR = SM_LIST + KN_M * KN_SPLIT * KN_KMAX * 8;   // barriers
-constexpr uint32_t SM_TOTAL = SM_BAR + 256;
-constexpr uint32_t KN_SMEM_BYTES = SM_TOTAL + 1024;
+template <int KB>
+struct Smem {
+    static constexpr int ST = kn_stages(KB);
+    static constexpr uint32_t A = 0;                                     // KB x 16 KB
+    static constexpr uint32_t B = A + KB * KN_M * KN_K * 2;              // ST x 32 KB
+    static constexpr uint32_t INFO = B + ST * KN_N * KN_K * 2;           // KN_INFO x 3 KB
+    static constexpr uint32_t LIST = INFO + KN_INFO * KN_N * 12;         // 128 x SPLIT x KMAX x 8 B
+    static constexpr uint32_t BAR = LIST + KN_M * KN_SPLIT * KN_KMAX * 8;   // barriers
+    static constexpr uint32_t BYTES = BAR + 256 + 1024;
+    static_assert(BYTES <= 232448, "shared memory of one CTA");
+};
 
 // SCREEN is the k-NN path. DUMP is the measurement form
 // (pantherpp_debug_screen): it also writes every screened value y_hat to
@@ -555,7 +571,7 @@ constexpr uint32_t KN_SMEM_BYTES = SM_TOTAL + 1024;
 constexpr int SEED_T = 5;
 enum { SCREEN = 0, DUMP_FORM = 1, SEED = 2 };
 
-template <int MODE>
+template <int MODE, int KB>
 __global__ void __launch_bounds__(KN_THREADS, 1)
     screen_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, ScreenArgs S) {
     constexpr bool DUMP = MODE == DUMP_FORM;
@@ -567,22 +583,32 @@ __global__ void __launch_bounds__(KN_THREADS, 1)
     const uint32_t raw = smem_u32(smraw);
     const uint32_t base = (raw + 1023) & ~1023u;
     uint8_t* gbase = smraw + (base - raw);
-    // barriers: full[4], empty[4], tfull[2], tempty[2], afull, aempty
-    const uint32_t bar0 = base + SM_BAR;
+    using SM = Smem<KB>;
+    constexpr int ST = SM::ST;
+    // barriers: full[ST], empty[ST], tfull[2], tempty[2], ifull, iempty[KN_INFO], afull, aempty, drain
+    const uint32_t bar0 = base + SM::BAR;
     auto FULL = [&](int s) { return bar0 + 8 * s; };
-    auto EMPTY = [&](int s) { return bar0 + 8 * (KN_STAGES + s); };
-    auto TFULL = [&](int b) { return bar0 + 8 * (2 * KN_STAGES + b); };
-    auto TEMPTY = [&](int b) { return bar0 + 8 * (2 * KN_STAGES + 2 + b); };
-    const uint32_t AFULL = bar0 + 8 * (2 * KN_STAGES + 4), AEMPTY = AFULL + 8;
-    const uint32_t DRAIN = bar0 + 8 * (2 * KN_STAGES + 8);   // completion of this CTA's MMAs after an abort
-    volatile int* abort_flag = (volatile int*)(gbase + SM_BAR + 8 * (2 * KN_STAGES + 6));
-    uint32_t* tmem_slot = (uint32_t*)(gbase + SM_BAR + 8 * (2 * KN_STAGES + 7));
+    auto EMPTY = [&](int s) { return bar0 + 8 * (ST + s); };
+    auto TFULL = [&](int b) { return bar0 + 8 * (2 * ST + b); };
+    auto TEMPTY = [&](int b) { return bar0 + 8 * (2 * ST + 2 + b); };
+    auto IFULL = [&](int i) { return bar0 + 8 * (2 * ST + 4 + i); };
+    auto IEMPTY = [&](int i) { return bar0 + 8 * (2 * ST + 4 + KN_INFO + i); };
+    constexpr int NB = 2 * ST + 4 + 2 * KN_INFO;
+    const uint32_t AFULL = bar0 + 8 * NB, AEMPTY = AFULL + 8;
+    const uint32_t DRAIN = bar0 + 8 * (NB + 2);              // completion of this CTA's MMAs after an abort
+    volatile int* abort_flag = (volatile int*)(gbase + SM::BAR + 8 * (NB + 3));
+    uint32_t* tmem_slot = (uint32_t*)(gbase + SM::BAR + 8 * (NB + 4));
+    static_assert(8 * (NB + 5) <= 256, "barrier area");
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
-        for (int s = 0; s < KN_STAGES; ++s) {
+        for (int s = 0; s < ST; ++s) {
             mbar_init(FULL(s), 1);
-            mbar_init(EMPTY(s), 1 + 4 * KN_SPLIT);
+            mbar_init(EMPTY(s), 1);                  // the MMAs that read the block
+        }
+        for (int i = 0; i < KN_INFO; ++i) {
+            mbar_init(IFULL(i), 1);
+            mbar_init(IEMPTY(i), 4 * KN_SPLIT);      // the selection warps
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(TFULL(b), 1);
@@ -606,13 +632,14 @@ __global__ void __launch_bounds__(KN_THREADS, 1)
     // what was issued, for the drain after an abort: the parity of the last A
     // load and of the last B load per stage (-1: none), and whether MMAs ran
     int last_a = -1;
-    int last_b[KN_STAGES];
-    for (int st = 0; st < KN_STAGES; ++st) last_b[st] = -1;
+    int last_b[ST], last_i[KN_INFO];
+    for (int st = 0; st < ST; ++st) last_b[st] = -1;
+    for (int i = 0; i < KN_INFO; ++i) last_i[i] = -1;
     bool mma_issued = false;
     if (warp == 0) {
         // ------------------------------------------------ TMA producer ---
         if (lane == 0) {
-            int64_t it = 0;
+            uint32_t it = 0, ib = 0;                 // tiles, operand blocks
             int j = 0;
             bool ok = true;
             Item w;
@@ -621,62 +648,81 @@ __global__ void __launch_bounds__(KN_THREADS, 1)
                     ok = false;
                     break;
                 }
-                mbar_expect_tx(AFULL, KN_M * KN_K * 2);
-                tma_load_2d(base + SM_A, &tmA, 0, (int)(w.qt * KN_M), AFULL);
+                mbar_expect_tx(AFULL, KB * KN_M * KN_K * 2);
+                for (int blk = 0; blk < KB; ++blk)
+                    tma_load_2d(base + SM::A + blk * (KN_M * KN_K * 2), &tmA, blk * KN_K, (int)(w.qt * KN_M), AFULL);
                 last_a = j & 1;
-                for (int64_t c = w.ct0; c < w.ct1; ++c, ++it) {
+                for (int64_t c = w.ct0; c < w.ct1 && ok; ++c, ++it) {
                     const int64_t ct = tile_at(c);
-                    int s = (int)(it % KN_STAGES);
-                    uint32_t ph = (uint32_t)((it / KN_STAGES) & 1);
-                    if (!mbar_wait(EMPTY(s), ph ^ 1, S.status, abort_flag)) { ok = false; break; }
-                    mbar_expect_tx(FULL(s), KN_N * KN_K * 2 + 3 * KN_N * 4);
-                    tma_load_2d(base + SM_B + s * (KN_N * KN_K * 2), &tmB, 0, (int)(ct * KN_N), FULL(s));
-                    uint32_t info = base + SM_INFO + s * (KN_N * 12);
-                    bulk_load(info, S.cid + ct * KN_N, KN_N * 4, FULL(s));
-                    bulk_load(info + KN_N * 4, S.cnrm + ct * KN_N, KN_N * 4, FULL(s));
-                    bulk_load(info + KN_N * 8, S.cncf + ct * KN_N, KN_N * 4, FULL(s));
-                    last_b[s] = (int)ph;
+                    const int si = (int)(it % KN_INFO);
+                    const uint32_t pi = (it / KN_INFO) & 1;
+                    if (!mbar_wait(IEMPTY(si), pi ^ 1, S.status, abort_flag)) { ok = false; break; }
+                    mbar_expect_tx(IFULL(si), 3 * KN_N * 4);
+                    const uint32_t info = base + SM::INFO + si * (KN_N * 12);
+                    bulk_load(info, S.cid + ct * KN_N, KN_N * 4, IFULL(si));
+                    bulk_load(info + KN_N * 4, S.cnrm + ct * KN_N, KN_N * 4, IFULL(si));
+                    bulk_load(info + KN_N * 8, S.cncf + ct * KN_N, KN_N * 4, IFULL(si));
+                    last_i[si] = (int)pi;
+                    for (int blk = 0; blk < KB; ++blk, ++ib) {
+                        const int s = (int)(ib % ST);
+                        const uint32_t ph = (ib / ST) & 1;
+                        if (!mbar_wait(EMPTY(s), ph ^ 1, S.status, abort_flag)) { ok = false; break; }
+                        mbar_expect_tx(FULL(s), KN_N * KN_K * 2);
+                        tma_load_2d(base + SM::B + s * (KN_N * KN_K * 2), &tmB, blk * KN_K, (int)(ct * KN_N), FULL(s));
+                        last_b[s] = (int)ph;
+                    }
                 }
             }
         }
     } else if (warp == 1) {
         // --------------------------------------------------- MMA issuer ---
         if (lane == 0) {
-            int64_t it = 0;
+            uint32_t it = 0, ib = 0;
             int j = 0;
             Item w;
             for (; split_item(S.W, blockIdx.x, gridDim.x, j, &w); ++j) {
                 if (!mbar_wait(AFULL, j & 1, S.status, abort_flag)) break;
                 bool ok = true;
-                for (int64_t ct = w.ct0; ct < w.ct1; ++ct, ++it) {
-                    int s = (int)(it % KN_STAGES);
-                    uint32_t ph = (uint32_t)((it / KN_STAGES) & 1);
-                    int b = (int)(it & 1);
-                    uint32_t pb = (uint32_t)((it >> 1) & 1);
-                    if (!mbar_wait(FULL(s), ph, S.status, abort_flag) ||
-                        !mbar_wait(TEMPTY(b), pb ^ 1, S.status, abort_flag)) {
+                for (int64_t c = w.ct0; c < w.ct1 && ok; ++c, ++it) {
+                    const int b = (int)(it & 1);
+                    const uint32_t pb = (it >> 1) & 1;
+                    if (!mbar_wait(TEMPTY(b), pb ^ 1, S.status, abort_flag)) {
                         ok = false;
                         break;
                     }
-                    tc_fence_after();
-                    uint32_t a0 = base + SM_A, b0 = base + SM_B + s * (KN_N * KN_K * 2);
+                    for (int blk = 0; blk < KB; ++blk, ++ib) {
+                        const int s = (int)(ib % ST);
+                        if (!mbar_wait(FULL(s), (ib / ST) & 1, S.status, abort_flag)) {
+                            ok = false;
+                            break;
+                        }
+                        tc_fence_after();
+                        const uint32_t a0 = base + SM::A + blk * (KN_M * KN_K * 2), b0 = base + SM::B + s * (KN_N * KN_K * 2);
 #pragma unroll
-                    for (int kk = 0; kk < KN_K / 16; ++kk)
-                        umma_bf16(tmem + b * KN_N, sw128_desc(a0 + kk * 32), sw128_desc(b0 + kk * 32), kk > 0);
-                    umma_commit(EMPTY(s));
-                    umma_commit(TFULL(b));
-                    mma_issued = true;
+                        for (int kk = 0; kk < KN_K / 16; ++kk)
+                            umma_bf16(tmem + b * KN_N, sw128_desc(a0 + kk * 32), sw128_desc(b0 + kk * 32),
+                                      blk > 0 || kk > 0);
+                        umma_commit(EMPTY(s));
+                        mma_issued = true;
+                    }
+                    // the tile's information has landed before the tile is
+                    // handed on: selection warps release its stage without
+                    // looking at it, and no copy is in flight when the CTA ends
+                    if (ok && !mbar_wait(IFULL(it % KN_INFO), (it / KN_INFO) & 1, S.status, abort_flag)) ok = false;
+                    if (ok) umma_commit(TFULL(b));
                 }
                 umma_commit(AEMPTY);
                 if (!ok) break;
             }
+            // the last commit has arrived before the CTA's shared memory goes
+            if (j > 0 && !*abort_flag) mbar_wait(AEMPTY, (j - 1) & 1, S.status, abort_flag);
         }
     } else {
         // --------------------------------------------------- selection ---
         const int quarter = warp & 3;             // TMEM lanes 32*quarter .. +31
         const int half = (warp - 2) >> 2;         // column slice of every tile this warp screens
         const int row = quarter * 32 + lane;
-        float2* mylist = (float2*)(gbase + SM_LIST) + (row * KN_SPLIT + half) * KN_KMAX;
+        float2* mylist = (float2*)(gbase + SM::LIST) + (row * KN_SPLIT + half) * KN_KMAX;
         uint32_t it = 0;
         Item w;
         for (int64_t wj = 0; split_item(S.W, blockIdx.x, gridDim.x, wj, &w); ++wj) {
@@ -686,7 +732,7 @@ __global__ void __launch_bounds__(KN_THREADS, 1)
                   0x7fffffff, 0, 0};
             const int64_t state = (slot * S.W.nseg + w.seg) * KN_SPLIT + half;
             const RowConst rc{S.qv[slot], S.exclude_self ? S.qv[slot] : -2, S.qexact[slot] != 0,
-                              KN_ALPHA * S.qnrm[slot], mylist,
+                              kn_alpha(KB) * S.qnrm[slot], kn_beta(KB), mylist,
                               S.shortlist + state * KN_SCAP, S.overflow + slot, S.k};
             const bool qtile_exact = S.qtile[w.qt] != 0;
             float acc[SEED_T * 4];
@@ -698,8 +744,8 @@ __global__ void __launch_bounds__(KN_THREADS, 1)
             bool flag = S.ctile[tile_at(w.ct0)] != 0;    // of the coming tile, loaded a tile ahead
             for (int64_t c = w.ct0; c < w.ct1; ++c, ++it) {
                 const int64_t ct = tile_at(c);
-                const int s = (int)(it % KN_STAGES);
-                const uint32_t ph = (it / KN_STAGES) & 1;
+                const int si = (int)(it % KN_INFO);
+                const uint32_t pi = (it / KN_INFO) & 1;
                 const int b = (int)(it & 1);
                 const uint32_t pb = (it >> 1) & 1;
                 const bool fast = qtile_exact && flag;
@@ -709,15 +755,15 @@ __global__ void __launch_bounds__(KN_THREADS, 1)
                     break;
                 }
                 tc_fence_after();
-                const uint8_t* info = gbase + SM_INFO + s * (KN_N * 12);
+                const uint8_t* info = gbase + SM::INFO + si * (KN_N * 12);
                 const int c0 = half * 128;                // 128 columns per selection warp
                 const int32_t* cid = (const int32_t*)info + c0;
                 const float* cnrm = (const float*)(info + KN_N * 4) + c0;
                 const float* cncf = (const float*)(info + KN_N * 8) + c0;
                 const uint32_t tbase = tmem + ((uint32_t)(quarter * 32) << 16) + b * KN_N + c0;
-                // the candidates' ids and norms of stage s, seen through its
-                // barrier (complete: the MMAs that filled TFULL waited for it)
-                auto info_ready = [&]() { return mbar_wait(FULL(s), ph, S.status, abort_flag); };
+                // the candidates' ids and norms of the tile, needed by few tiles
+                // (they have landed: the wait makes them visible)
+                auto info_ready = [&]() { return mbar_wait(IFULL(si), pi, S.status, abort_flag); };
                 uint32_t u[4][32];
                 float m[4];
                 __syncwarp();
@@ -769,7 +815,7 @@ __global__ void __launch_bounds__(KN_THREADS, 1)
                                            ct * KN_N + c0 + g * 32, S.nexact);
                 }
                 __syncwarp();
-                if (lane == 0) mbar_arrive(EMPTY(s));
+                if (lane == 0) mbar_arrive(IEMPTY(si));
             }
             if (!ok) break;
             if constexpr (MODE == SEED) {
@@ -805,8 +851,10 @@ __global__ void __launch_bounds__(KN_THREADS, 1)
         // TMEM and exits (each drain is bounded too)
         if (warp == 0 && lane == 0) {
             if (last_a >= 0) mbar_drain(AFULL, (uint32_t)last_a);
-            for (int st = 0; st < KN_STAGES; ++st)
+            for (int st = 0; st < ST; ++st)
                 if (last_b[st] >= 0) mbar_drain(FULL(st), (uint32_t)last_b[st]);
+            for (int i = 0; i < KN_INFO; ++i)
+                if (last_i[i] >= 0) mbar_drain(IFULL(i), (uint32_t)last_i[i]);
         }
         if (warp == 1 && lane == 0 && mma_issued) {
             umma_commit(DRAIN);
@@ -850,7 +898,7 @@ __global__ void __launch_bounds__(F_T) fp32_kernel(const uint32_t* __restrict__ 
     // rows with every entry <= 256 give exact FP32 products and partial sums
     // (all integers below 2^24); other pairs carry the bound
     const bool qex = slot < qpad && qexact[slot] != 0;
-    const RowConst rc{qid, exclude_self ? qid : -2, qex, 2.0f * epsD * (slot < qpad ? qnrm[slot] : 0.f),
+    const RowConst rc{qid, exclude_self ? qid : -2, qex, 2.0f * epsD * (slot < qpad ? qnrm[slot] : 0.f), 0.f,
                       lst + threadIdx.x * KN_KMAX, shortlist + (slot < qpad ? state : 0) * KN_SPLIT * KN_SCAP,
                       overflow + (slot < qpad ? slot : 0), k};
     Row r{__int_as_float(0x7f800000), 0x7fffffff, 0, 0};
@@ -1372,11 +1420,11 @@ static PFN_cuTensorMapEncodeTiled_v12000 encode_fn(panther_ctx* ctx) {
     return fn;
 }
 
-static bool make_map(panther_ctx* ctx, CUtensorMap* m, const void* base, int64_t rows, int box_rows) {
+static bool make_map(panther_ctx* ctx, CUtensorMap* m, const void* base, int64_t rows, int box_rows, int kb) {
     auto fn = encode_fn(ctx);
     if (!fn) return false;
-    cuuint64_t dims[2] = {(cuuint64_t)KN_K, (cuuint64_t)rows};
-    cuuint64_t strides[1] = {(cuuint64_t)KN_K * 2};
+    cuuint64_t dims[2] = {(cuuint64_t)KN_K * kb, (cuuint64_t)rows};
+    cuuint64_t strides[1] = {(cuuint64_t)KN_K * kb * 2};
     cuuint32_t box[2] = {(cuuint32_t)KN_K, (cuuint32_t)box_rows};
     cuuint32_t estr[2] = {1, 1};
     CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
@@ -1442,7 +1490,7 @@ extern "C" panther_status pantherpp_vectors(panther_ctx* ctx, const panther_inde
     x.npad = ceil_div(n, KN_N) * KN_N;
     int32_t* perm = nullptr;
     if ((st = dev_alloc(ctx, (void**)&perm, sizeof(int32_t) * x.npad)) ||
-        (D <= KN_K - 8 && (st = dev_alloc(ctx, (void**)&x.B, (size_t)x.npad * KN_K * 2))) ||
+        (st = dev_alloc(ctx, (void**)&x.B, (size_t)x.npad * kn_blocks(D) * KN_K * 2)) ||
         (st = dev_alloc(ctx, (void**)&x.cid, sizeof(int32_t) * x.npad)) ||
         (st = dev_alloc(ctx, (void**)&x.cnrm, sizeof(float) * x.npad)) ||
         (st = dev_alloc(ctx, (void**)&x.cncf, sizeof(float) * x.npad)) ||
@@ -1470,24 +1518,24 @@ extern "C" panther_status pantherpp_vectors(panther_ctx* ctx, const panther_inde
     return PANTHER_OK;
 }
 
-// The BF16 screen's work in equal runs, one per CTA, of at least KN_STAGES
+// The BF16 screen's work in equal runs, one per CTA, of at least KN_MIN_RUN
 // candidate tiles. From 16 query tiles per SM on, whole tiles per CTA: the last
 // wave then costs at most 6%, and every segment more of a tile costs lists and
 // a shortlist of 2 KB per query.
 static Split knn_split(int64_t nqt, int64_t nct, int num_sms) {
     Split W{nqt, nct, 0, 1};
     if (nqt >= 16 * (int64_t)num_sms) return W;
-    W.G = std::max<int64_t>(1, std::min<int64_t>(num_sms, nqt * nct / KN_STAGES));
+    W.G = std::max<int64_t>(1, std::min<int64_t>(num_sms, nqt * nct / KN_MIN_RUN));
     for (int64_t t = 0; t < nqt; ++t) W.nseg = std::max(W.nseg, W.segments(t));
     return W;
 }
 
 // The FP32 form's candidate ranges: with fewer query tiles than SMs the choice
-// minimises waves x range length, at least KN_STAGES candidate tiles per range.
+// minimises waves x range length, at least KN_MIN_RUN candidate tiles per range.
 static Split knn_ranges(int64_t nqt, int64_t nct, int num_sms) {
     Split W{nqt, nct, 0, 1};
     if (nqt >= num_sms) return W;
-    const int64_t pmax = std::max<int64_t>(1, std::min<int64_t>(nct / KN_STAGES, 256));
+    const int64_t pmax = std::max<int64_t>(1, std::min<int64_t>(nct / KN_MIN_RUN, 256));
     double best_cost = (double)ceil_div(nqt, num_sms);
     for (int64_t p = 2; p <= pmax; ++p) {
         const double cost = (double)ceil_div(nqt * p, num_sms) / (double)p;
@@ -1503,6 +1551,16 @@ static Split knn_ranges(int64_t nqt, int64_t nct, int num_sms) {
 // a 16th of fewer than 2,048, none below 128 tiles (32,768 candidates), where
 // the screen itself is as short.
 static int64_t seed_tiles(int64_t nct) { return nct < 128 ? 0 : nct / (nct < 2048 ? 16 : 32); }
+
+template <int MODE, int KB>
+static panther_status launch_screen(panther_ctx* ctx, unsigned grid, const CUtensorMap& tmA, const CUtensorMap& tmB,
+                                    const ScreenArgs& S) {
+    PCK(ctx, cudaFuncSetAttribute(screen_kernel<MODE, KB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)Smem<KB>::BYTES));
+    screen_kernel<MODE, KB><<<grid, KN_THREADS, Smem<KB>::BYTES, ctx->stream>>>(tmA, tmB, S);
+    PLAUNCH(ctx);
+    return PANTHER_OK;
+}
 
 // queries are vertices of vq, candidates every vertex of vc; `same` excludes
 // the candidate with the query's id (one graph: the query itself)
@@ -1552,7 +1610,7 @@ static panther_status knn_run(panther_ctx* ctx, const pantherpp_vecs* vq, const 
                      (st = dev_alloc(ctx, (void**)&pd, sizeof(uint64_t) * qpad * nch * k)))) ||
         (ns && ((st = dev_alloc(ctx, (void**)&smin, sizeof(float) * qpad * WS.nseg * KN_SPLIT * seed_keys)) ||
                 (st = dev_alloc(ctx, (void**)&thr0, sizeof(float) * qpad)))) ||
-        (!fp32 && (st = dev_alloc(ctx, (void**)&A, (size_t)qpad * KN_K * 2)))) {
+        (!fp32 && (st = dev_alloc(ctx, (void**)&A, (size_t)qpad * kn_blocks(vq->D) * KN_K * 2)))) {
         cleanup();
         return st;
     }
@@ -1572,8 +1630,9 @@ static panther_status knn_run(panther_ctx* ctx, const pantherpp_vecs* vq, const 
     if (!fp32) {
         vec_arow_kernel<<<(unsigned)ceil_div(qpad, 8), 256, 0, s>>>(v->theta, Q.qv, qpad, v->D, A);
         ctx->launches++;
+        const int kb = kn_blocks(v->D);
         CUtensorMap tmA, tmB;
-        if (!make_map(ctx, &tmA, A, qpad, KN_M) || !make_map(ctx, &tmB, x.B, x.npad, KN_N)) {
+        if (!make_map(ctx, &tmA, A, qpad, KN_M, kb) || !make_map(ctx, &tmB, x.B, x.npad, KN_N, kb)) {
             cleanup();
             return PANTHER_ECUDA;
         }
@@ -1582,16 +1641,10 @@ static panther_status knn_run(panther_ctx* ctx, const pantherpp_vecs* vq, const 
         auto grid = [&](const Split& w) {
             return (unsigned)(w.G ? w.G : std::min<int64_t>(nqt, ctx->num_sms));
         };
-        if (dump) {
-            PCK(ctx, cudaFuncSetAttribute(screen_kernel<DUMP_FORM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)KN_SMEM_BYTES));
-            screen_kernel<DUMP_FORM><<<grid(W), KN_THREADS, KN_SMEM_BYTES, s>>>(tmA, tmB, S);
+        if (dump) {                                  // (D <= 56)
+            if ((st = launch_screen<DUMP_FORM, 1>(ctx, grid(W), tmA, tmB, S))) { cleanup(); return st; }
         } else {
-            PCK(ctx, cudaFuncSetAttribute(screen_kernel<SCREEN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)KN_SMEM_BYTES));
             if (ns) {
-                PCK(ctx, cudaFuncSetAttribute(screen_kernel<SEED>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              (int)KN_SMEM_BYTES));
                 ScreenArgs SS = S;
                 SS.W = WS;
                 SS.seed_step = (uint32_t)(nct / ns);
@@ -1599,14 +1652,19 @@ static panther_status knn_run(panther_ctx* ctx, const pantherpp_vecs* vq, const 
                 while (std::gcd(SS.seed_mul, (uint32_t)ns) != 1) ++SS.seed_mul;
                 SS.smin = smin;
                 SS.seed_keys = seed_keys;
-                screen_kernel<SEED><<<grid(WS), KN_THREADS, KN_SMEM_BYTES, s>>>(tmA, tmB, SS);
+                st = kb == 1 ? launch_screen<SEED, 1>(ctx, grid(WS), tmA, tmB, SS)
+                   : kb == 2 ? launch_screen<SEED, 2>(ctx, grid(WS), tmA, tmB, SS)
+                             : launch_screen<SEED, 3>(ctx, grid(WS), tmA, tmB, SS);
+                if (st) { cleanup(); return st; }
                 seed_bound_kernel<<<(unsigned)ceil_div(qpad, 8), 256, 0, s>>>(smin, qpad, WS, seed_keys, k, thr0);
-                ctx->launches += 2;
+                ctx->launches++;
                 S.thr0 = thr0;
             }
-            screen_kernel<SCREEN><<<grid(W), KN_THREADS, KN_SMEM_BYTES, s>>>(tmA, tmB, S);
+            st = kb == 1 ? launch_screen<SCREEN, 1>(ctx, grid(W), tmA, tmB, S)
+               : kb == 2 ? launch_screen<SCREEN, 2>(ctx, grid(W), tmA, tmB, S)
+                         : launch_screen<SCREEN, 3>(ctx, grid(W), tmA, tmB, S);
+            if (st) { cleanup(); return st; }
         }
-        ctx->launches++;
     } else {
         const dim3 fg((unsigned)(qpad / F_T), (unsigned)nch);
         if (v->D <= KN_K)
@@ -1685,9 +1743,7 @@ static panther_status knn_entry(panther_ctx* ctx, const pantherpp_vecs* v, const
     if (k < 1 || k > KN_KMAX) return set_err(ctx, PANTHER_EINVAL, "k must be in [1, 32]");
     int mode = flags & 0xff;
     if (mode != PANTHER_KNN_BF16_SCREEN && mode != PANTHER_KNN_FP32) return set_err(ctx, PANTHER_EINVAL, "bad flags");
-    // vectors wider than the BF16 screen's 56 columns take the FP32 screen
-    // (64 or 128 columns), with the same exact rerank
-    const bool fp32 = mode == PANTHER_KNN_FP32 || v->D > KN_K - 8;
+    const bool fp32 = mode == PANTHER_KNN_FP32;
     auto run = [&](const int32_t* qs, int32_t* oi, uint64_t* od) {
         return knn_run(ctx, v, vc, same, qs, q, k, oi, od, fp32);
     };
@@ -1744,7 +1800,7 @@ extern "C" panther_status pantherpp_debug_screen(panther_ctx* ctx, const panther
     if (!out_y && !out_cid) return PANTHER_OK;
     if (!queries || !out_y || !out_cid || q < 1 || q > KN_M)
         return set_err(ctx, PANTHER_EINVAL, "1 <= q <= 128 queries and both outputs are needed");
-    if (v->D > KN_K - 8) return set_err(ctx, PANTHER_EINVAL, "BF16 screening needs D <= 56");
+    if (kn_blocks(v->D) > 1) return set_err(ctx, PANTHER_EINVAL, "BF16 screening values are kept for D <= 56 only");
     cudaSetDevice(ctx->device);
     cudaStream_t s = ctx->stream;
     int32_t* ids = nullptr;

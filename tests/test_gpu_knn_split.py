@@ -29,8 +29,9 @@ def pk():
 
 # (n, R): 79 candidate tiles and no sample; 157 and a sample of 9; R = 4e5 puts
 # counts above 256 into the heaviest rows
+# D = 57, 120, 121 and 128: the edges of operand rows of 64, 128 and 192 columns
 @pytest.mark.parametrize("n,R", [(20_001, 60_000), (40_000, 400_000)])
-@pytest.mark.parametrize("D", [10, 50, 56])
+@pytest.mark.parametrize("D", [10, 50, 56, 57, 100, 120, 121, 128])
 def test_knn_batches(pk, n, R, D):
     g = synth.chung_lu(n, 10, 2.3, ("uniform", 1, 9), seed=4)
     ref = oracle.sample_paths(g, 2, R, 5, oracle.ALIAS, threads=THREADS)
