@@ -2709,7 +2709,7 @@ extern "C" panther_status panther_tune_topk(panther_ctx* ctx, const panther_inde
     if (ix->n != p->n || ix->R != p->R) return set_err(ctx, PANTHER_EINVAL, "index and paths do not belong together");
     cudaSetDevice(ctx->device);
     struct Shape { int threads, slots, bps; };
-    const Shape cand[] = {{128, 3840, 6}, {128, 3072, 7}, {128, 6144, 4}, {256, 3840, 6},
+    const Shape cand[] = {{128, 3840, 6}, {128, 3072, 7}, {128, 6144, 4}, {256, 4096, 5},
                           {256, 6144, 4}, {256, 8192, 3}, {512, 12288, 2}, {512, 24576, 1}};
     cudaEvent_t a, b;
     PCK(ctx, cudaEventCreate(&a));
