@@ -5,7 +5,10 @@
 //
 // PREFIX table: entry j of row v = {inclusive cumulative weight, neighbour}
 //   (uint2 when every S < 2^32, else uint4 {cum_lo, cum_hi, col, 0}).
-// ALIAS table: entry c of row v = {thr_lo, thr_hi, col[c], col[alias[c]]}.
+// ALIAS table: entry c of row v = {thr, S, col[c], col[alias[c]]} when every
+//   S < 2^32 (the usual graph), else {thr_lo, thr_hi, col[c], col[alias[c]]}.
+//   With S in the entry a walk step needs only {start, deg} of its vertex, so
+//   the sampler reads 8-byte records (vsmall) instead of 16-byte ones.
 //   It is the integer Vose table with LIFO worklists (q_j = w_j * deg against
 //   capacity S). A column popped as "small" gets the large that is current at
 //   that moment; that large is determined by prefix sums of the deficits of
@@ -182,6 +185,11 @@ __device__ __forceinline__ uint64_t edge_hash(uint64_t a, uint64_t b, uint64_t w
 }
 
 // -------------------------------------------------------- row stats ---
+// alias entry of threshold thr in a row of sum S (see the layouts above)
+__device__ __forceinline__ uint4 alias_entry(uint64_t thr, uint64_t S, int32_t self, int32_t other, bool narrow) {
+    return make_uint4((uint32_t)thr, narrow ? (uint32_t)S : (uint32_t)(thr >> 32), (uint32_t)self, (uint32_t)other);
+}
+
 struct StatsOut {
     uint4* vrec;
     uint32_t* status;
@@ -618,7 +626,7 @@ constexpr int ASSIGN_WAYS = 4;
 __device__ void alias_assign(int64_t start, int64_t deg, uint64_t S, int64_t nsm, const int32_t* __restrict__ col,
                              const uint32_t* __restrict__ w, uint4* __restrict__ tab,
                              const int32_t* __restrict__ sidx, const uint64_t* __restrict__ scum, int64_t tid,
-                             int64_t nthreads) {
+                             int64_t nthreads, bool narrow) {
     const uint64_t d = (uint64_t)deg;
     const int64_t nl = deg - nsm;
     const uint64_t* __restrict__ D = scum + start;
@@ -651,10 +659,9 @@ __device__ void alias_assign(int64_t start, int64_t deg, uint64_t S, int64_t nsm
                 while (i < nl && E[i] < dprev) ++i;
                 const uint64_t q = (uint64_t)wj * d;
                 if (nl == 0 || i >= nl)   // cannot happen for consistent integer weights
-                    tab[start + j] = make_uint4((uint32_t)S, (uint32_t)(S >> 32), (uint32_t)self, (uint32_t)self);
+                    tab[start + j] = alias_entry(S, S, self, self, narrow);
                 else
-                    tab[start + j] = make_uint4((uint32_t)q, (uint32_t)(q >> 32), (uint32_t)self,
-                                                (uint32_t)col[start + LI[i]]);
+                    tab[start + j] = alias_entry(q, S, self, col[start + LI[i]], narrow);
             };
             for (int64_t s2 = 0; s2 < len; ++s2)
 #pragma unroll
@@ -683,10 +690,9 @@ __device__ void alias_assign(int64_t start, int64_t deg, uint64_t S, int64_t nsm
                 while (js < nsm && D[js] <= Ei) ++js;
                 if (Dtot > Ei && i + 1 < nl) {
                     uint64_t thr = S - (D[js] - Ei);
-                    tab[start + j] = make_uint4((uint32_t)thr, (uint32_t)(thr >> 32), (uint32_t)self,
-                                                (uint32_t)col[start + jnext]);
+                    tab[start + j] = alias_entry(thr, S, self, col[start + jnext], narrow);
                 } else {
-                    tab[start + j] = make_uint4((uint32_t)S, (uint32_t)(S >> 32), (uint32_t)self, (uint32_t)self);
+                    tab[start + j] = alias_entry(S, S, self, self, narrow);
                 }
             };
             for (int64_t s2 = 0; s2 < len; ++s2)
@@ -700,10 +706,10 @@ __device__ void alias_assign(int64_t start, int64_t deg, uint64_t S, int64_t nsm
 
 template <class G>
 __device__ void row_alias(const G& g, int64_t start, int64_t deg, uint64_t S, const int32_t* col,
-                          const uint32_t* w, uint4* tab, int32_t* sidx, uint64_t* scum) {
+                          const uint32_t* w, uint4* tab, int32_t* sidx, uint64_t* scum, bool narrow) {
     if (deg == 0) return;
     int64_t nsm = row_alias_prep(g, start, deg, S, w, sidx, scum);
-    alias_assign(start, deg, S, nsm, col, w, tab, sidx, scum, g.rank(), G::size);
+    alias_assign(start, deg, S, nsm, col, w, tab, sidx, scum, g.rank(), G::size, narrow);
 }
 
 // rows of degree <= SMALL_DEG: one thread per row runs the sequential LIFO
@@ -713,7 +719,7 @@ constexpr int SMALL_DEG = 16;
 
 __global__ void __launch_bounds__(256) alias_thread_kernel(const uint4* __restrict__ vrec, int64_t n,
                                                            const int32_t* __restrict__ col,
-                                                           const uint32_t* __restrict__ w, uint4* tab) {
+                                                           const uint32_t* __restrict__ w, uint4* tab, bool narrow) {
     // the worklists and the row's columns live in shared memory, one column
     // per thread (no local memory, no bank conflicts)
     __shared__ uint64_t qs[SMALL_DEG][256];
@@ -751,31 +757,32 @@ __global__ void __launch_bounds__(256) alias_thread_kernel(const uint4* __restri
         while (ns > 0 && nl > 0) {
             const int a = sm(--ns), b = lg(--nl);
             const uint64_t qa = q(a);
-            tab[start + a] = make_uint4((uint32_t)qa, (uint32_t)(qa >> 32), (uint32_t)c(a), (uint32_t)c(b));
+            tab[start + a] = alias_entry(qa, S, c(a), c(b), narrow);
             const uint64_t qb = q(b) - (S - qa);
             q(b) = qb;
             if (qb < S) sm(ns++) = (int8_t)b; else lg(nl++) = (int8_t)b;
         }
         while (nl > 0) {
             const int b = lg(--nl);
-            tab[start + b] = make_uint4((uint32_t)S, (uint32_t)(S >> 32), (uint32_t)c(b), (uint32_t)c(b));
+            tab[start + b] = alias_entry(S, S, c(b), c(b), narrow);
         }
         while (ns > 0) {
             const int a = sm(--ns);
-            tab[start + a] = make_uint4((uint32_t)S, (uint32_t)(S >> 32), (uint32_t)c(a), (uint32_t)c(a));
+            tab[start + a] = alias_entry(S, S, c(a), c(a), narrow);
         }
     }
 }
 
 __global__ void alias_warp_kernel(const uint4* __restrict__ vrec, int64_t n, const int32_t* __restrict__ col,
                                   const uint32_t* __restrict__ w, const int32_t* __restrict__ mid, int64_t nmed,
-                                  uint4* tab, int32_t* sidx, uint64_t* scum) {
+                                  uint4* tab, int32_t* sidx, uint64_t* scum, bool narrow) {
     WarpG g;
     int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t i = wid; i < nmed; i += nw) {
         const uint4 r = vrec[mid[n - 1 - i]];
-        row_alias(g, (int64_t)r.x, (int64_t)r.y, (uint64_t)r.z | ((uint64_t)r.w << 32), col, w, tab, sidx, scum);
+        row_alias(g, (int64_t)r.x, (int64_t)r.y, (uint64_t)r.z | ((uint64_t)r.w << 32), col, w, tab, sidx, scum,
+                  narrow);
     }
 }
 
@@ -785,7 +792,7 @@ __global__ void alias_warp_kernel(const uint4* __restrict__ vrec, int64_t n, con
 template <int G>
 __global__ void alias_short_kernel(const uint4* __restrict__ vrec, int64_t n, const int32_t* __restrict__ col,
                                    const uint32_t* __restrict__ w, const int32_t* __restrict__ rows, bool back,
-                                   int64_t nrows, uint4* tab, int32_t* sidx, uint64_t* scum) {
+                                   int64_t nrows, uint4* tab, int32_t* sidx, uint64_t* scum, bool narrow) {
     SubG<G, 4> g;
     const int64_t gid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / G;
     const int64_t ng = ((int64_t)gridDim.x * blockDim.x) / G;
@@ -842,7 +849,7 @@ __global__ void alias_short_kernel(const uint4* __restrict__ vrec, int64_t n, co
             if (p < nl) scum[start + nsm + p] = x[j];
         }
         g.sync();
-        if (deg > 0) alias_assign(start, deg, S, nsm, col, w, tab, sidx, scum, rk, G);
+        if (deg > 0) alias_assign(start, deg, S, nsm, col, w, tab, sidx, scum, rk, G, narrow);
         g.sync();
     }
 }
@@ -991,12 +998,31 @@ __global__ void alias_assign_kernel(const uint4* __restrict__ vrec, const int32_
                                     const uint32_t* __restrict__ w, const int32_t* __restrict__ big,
                                     const int64_t* __restrict__ bign, const int64_t* __restrict__ seg_off,
                                     int64_t nbig, uint4* tab, const int32_t* __restrict__ sidx,
-                                    const uint64_t* __restrict__ scum) {
+                                    const uint64_t* __restrict__ scum, bool narrow) {
     const int64_t row = seg_owner(seg_off, nbig, blockIdx.x);
     const int64_t parts = seg_off[row + 1] - seg_off[row], part = blockIdx.x - seg_off[row];
     uint4 r = vrec[big[row]];
     alias_assign((int64_t)r.x, (int64_t)r.y, (uint64_t)r.z | ((uint64_t)r.w << 32), bign[row], col, w, tab, sidx,
-                 scum, part * blockDim.x + threadIdx.x, parts * blockDim.x);
+                 scum, part * blockDim.x + threadIdx.x, parts * blockDim.x, narrow);
+}
+
+// {start, deg} of every vertex: the records of the alias (S < 2^32) and the
+// unweighted walk
+__global__ void small_records_kernel(const uint4* __restrict__ vrec, int64_t n, uint2* __restrict__ vsmall) {
+    const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (v < n) {
+        const uint4 r = vrec[v];
+        vsmall[v] = make_uint2(r.x, r.y);
+    }
+}
+
+// narrow alias entries in the wide layout (threshold in the first two words)
+__global__ void widen_alias_kernel(const uint4* __restrict__ in, int64_t m, uint4* __restrict__ out) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < m) {
+        const uint4 e = in[i];
+        out[i] = make_uint4(e.x, 0u, e.z, e.w);
+    }
 }
 
 unsigned grid_for(panther_ctx* ctx, int64_t items_per_block_unit, int64_t n, int threads) {
@@ -1177,6 +1203,7 @@ extern "C" panther_status panther_build_graph(panther_ctx* ctx, int64_t n, int64
         return free_plan(), fail(set_err(ctx, PANTHER_EINVAL, "graph is not symmetric with equal weights"));
     g->max_row_sum = h_acc[0];
     g->prefix_wide = h_acc[0] >= (1ull << 32) ? 1 : 0;
+    const bool narrow = !g->prefix_wide;
 
     if (modes & PANTHER_MODE_PREFIX) {
         size_t esz = g->prefix_wide ? sizeof(uint4) : sizeof(uint2);
@@ -1201,26 +1228,26 @@ extern "C" panther_status panther_build_graph(panther_ctx* ctx, int64_t n, int64
             return free_plan(), fail(st);
         }
         alias_thread_kernel<<<(unsigned)std::min<int64_t>(ceil_div(n, 256), (int64_t)ctx->num_sms * 16), 256, 0, s>>>(
-            g->vrec, n, d_col, d_w, g->alias);
+            g->vrec, n, d_col, d_w, g->alias, narrow);
         ctx->launches++;
         if (nshort) {
             alias_short_kernel<8><<<rows_grid(nshort, 8), 256, 0, s>>>(g->vrec, n, d_col, d_w, mid, false, nshort,
-                                                                       g->alias, sidx, scum);
+                                                                       g->alias, sidx, scum, narrow);
             ctx->launches++;
         }
         if (n16) {
             alias_short_kernel<16><<<rows_grid(n16, 16), 256, 0, s>>>(g->vrec, n, d_col, d_w, mid2, false, n16,
-                                                                      g->alias, sidx, scum);
+                                                                      g->alias, sidx, scum, narrow);
             ctx->launches++;
         }
         if (n32) {
             alias_short_kernel<32><<<rows_grid(n32, 32), 256, 0, s>>>(g->vrec, n, d_col, d_w, mid2, true, n32,
-                                                                      g->alias, sidx, scum);
+                                                                      g->alias, sidx, scum, narrow);
             ctx->launches++;
         }
         if (nmed) {
             alias_warp_kernel<<<rows_grid(nmed, 32), 256, 0, s>>>(g->vrec, n, d_col, d_w, mid, nmed, g->alias, sidx,
-                                                                  scum);
+                                                                  scum, narrow);
             ctx->launches++;
         }
         if (h_nbig) {
@@ -1242,7 +1269,7 @@ extern "C" panther_status panther_build_graph(panther_ctx* ctx, int64_t n, int64
             big_place_kernel<<<(unsigned)nseg, BLK, 0, s>>>(g->vrec, d_w, big, seg_off, h_nbig, segsum, bign, sidx,
                                                             scum);
             alias_assign_kernel<<<(unsigned)nseg, 256, 0, s>>>(g->vrec, d_col, d_w, big, bign, seg_off, h_nbig,
-                                                               g->alias, sidx, scum);
+                                                               g->alias, sidx, scum, narrow);
             ctx->launches += 4;
             dev_free(ctx, segsum);
             dev_free(ctx, bign);
@@ -1260,6 +1287,17 @@ extern "C" panther_status panther_build_graph(panther_ctx* ctx, int64_t n, int64
             if ((st = dev_alloc(ctx, (void**)&g->col, sizeof(int32_t) * m))) return free_plan(), fail(st);
             if ((e = cudaMemcpyAsync(g->col, col, sizeof(int32_t) * m, cudaMemcpyDeviceToDevice, s)))
                 return free_plan(), fail(cuda_err(ctx, e, "column copy"));
+        }
+    }
+    if ((modes & PANTHER_MODE_UNWEIGHTED) || ((modes & PANTHER_MODE_ALIAS) && narrow)) {
+        if ((st = dev_alloc(ctx, (void**)&g->vsmall, sizeof(uint2) * n))) return free_plan(), fail(st);
+        small_records_kernel<<<(unsigned)ceil_div(n, 256), 256, 0, s>>>(g->vrec, n, g->vsmall);
+        ctx->launches++;
+        if ((e = cudaGetLastError())) return free_plan(), fail(cuda_err(ctx, e, "vertex records"));
+        // the prefix walk and wide alias entries need S of the 16-byte records
+        if (!(modes & PANTHER_MODE_PREFIX) && (narrow || !(modes & PANTHER_MODE_ALIAS))) {
+            dev_free(ctx, g->vrec);
+            g->vrec = nullptr;
         }
     }
     free_plan();
@@ -1288,7 +1326,10 @@ panther_status panther_debug_graph_tables(const panther_graph* g, void* dev_alia
     if (!g) return PANTHER_EINVAL;
     panther_ctx* ctx = g->ctx;
     if (prefix_wide) *prefix_wide = g->prefix_wide;
-    if (dev_alias16 && g->alias)
+    if (dev_alias16 && g->alias && !g->prefix_wide && g->m > 0) {
+        widen_alias_kernel<<<(unsigned)ceil_div(g->m, 256), 256, 0, ctx->stream>>>(g->alias, g->m, (uint4*)dev_alias16);
+        PLAUNCH(ctx);
+    } else if (dev_alias16 && g->alias)
         PCK(ctx, cudaMemcpyAsync(dev_alias16, g->alias, sizeof(uint4) * g->m, cudaMemcpyDeviceToDevice, ctx->stream));
     if (dev_prefix && g->prefix)
         PCK(ctx, cudaMemcpyAsync(dev_prefix, g->prefix, (g->prefix_wide ? 16 : 8) * g->m, cudaMemcpyDeviceToDevice,

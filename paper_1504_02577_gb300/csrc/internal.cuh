@@ -63,10 +63,11 @@ struct panther_graph {
     panther_ctx* ctx = nullptr;
     int64_t n = 0, m = 0;
     int modes = 0;
-    uint4* vrec = nullptr;           // [n]: {start, deg, S_lo, S_hi}
+    uint4* vrec = nullptr;           // [n]: {start, deg, S_lo, S_hi} (PREFIX, and ALIAS with a row sum from 2^32)
+    uint2* vsmall = nullptr;         // [n]: {start, deg} (UNWEIGHTED, and ALIAS otherwise)
     void* prefix = nullptr;          // [m]: uint2 {cum, col} or uint4 {cum_lo, cum_hi, col, 0}
     int prefix_wide = 0;             // 1 when a row sum reaches 2^32
-    uint4* alias = nullptr;          // [m]: {thr_lo, thr_hi, col_self, col_alias}
+    uint4* alias = nullptr;          // [m]: {thr, S, col_self, col_alias}, or {thr_lo, thr_hi, ..} when it does
     int32_t* col = nullptr;          // [m]: neighbours (UNWEIGHTED mode only)
     uint64_t max_row_sum = 0;
 };

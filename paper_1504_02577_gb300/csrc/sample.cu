@@ -1,10 +1,13 @@
 // Random path sampling (Algorithm 3).
 //
 // One thread walks one path at a time (grid-stride over path ids). Each step
-// is a dependent chain: the 16-byte vertex record (start, deg, S), then either
-// a binary search over the prefix table ending in a short unrolled scan whose
-// final sector also carries the neighbour id, or a single 16-byte alias entry
-// that already carries both candidate neighbour ids. The row is kept in
+// is a dependent chain: the vertex record (16 bytes {start, deg, S}, or 8
+// without S), then either a binary search over the prefix table ending in a
+// short unrolled scan whose final sector also carries the neighbour id, or a
+// single 16-byte alias entry that already carries both candidate neighbour ids
+// (and S). Paths of T = 5 on 20M / 5M vertices (R = 4e7 / 1e7, alias): 6.84 /
+// 1.43 ms with 16-byte records, 6.36 / 1.32 with 8-byte ones; unweighted T = 9
+// on 1M (R = 3e6): 335 / 314 us. The row is kept in
 // registers and stored as 32-byte vectors (stride 8/16/32 int32).
 #include "internal.cuh"
 
@@ -47,66 +50,94 @@ __device__ __forceinline__ uint32_t pick_prefix64(const uint4* __restrict__ e, u
     return v;
 }
 
-// MODE 1 = prefix, 2 = alias, 4 = unweighted (tab = the column array)
+// One step from vertex v at draw (r, t): the next vertex (v itself without
+// neighbours). MODE 1 = prefix, 2 = alias, 4 = unweighted (tab = the column
+// array); WIDE: a row sum reaches 2^32. The step is two dependent random reads,
+// the vertex record and the table entry, and the whole kernel waits for DRAM
+// (64-byte bursts for records of 8 or 16 bytes), so the records are kept as
+// small as the mode allows: {start, deg} where the entry carries S or S is not
+// needed. They are the part of the tables that L2 can hold.
+template <int MODE, bool WIDE>
+__device__ __forceinline__ uint64_t walk_step(const uint4* __restrict__ vrec, const uint2* __restrict__ vsmall,
+                                              const void* __restrict__ tab, uint64_t seed, uint64_t r, uint32_t t,
+                                              uint64_t v) {
+    if (MODE == 4) {
+        // t_ij = 1/deg: Uniform[0, deg) from the same words as the prefix
+        // draw, so the walk equals prefix selection with every weight 1
+        const uint2 rec = __ldg(&vsmall[v]);
+        if (rec.y == 0) return v;
+        uint64_t c = 0;
+        for (uint32_t att = 0;; ++att) {
+            const pword4 w = path_draw(seed, r, t, att);
+            if (lemire64((uint64_t)w.x | ((uint64_t)w.y << 32), (uint64_t)rec.y, &c)) break;
+        }
+        return (uint64_t)(uint32_t)__ldg((const int32_t*)tab + rec.x + c);
+    }
+    if (MODE == 2 && !WIDE) {
+        // the coin's range S comes with the drawn column's entry
+        const uint2 rec = __ldg(&vsmall[v]);
+        if (rec.y == 0) return v;
+        for (uint32_t att = 0;; ++att) {
+            const pword4 w = path_draw(seed, r, t, att);
+            uint64_t c = 0, u = 0;
+            if (!lemire64((uint64_t)w.x | ((uint64_t)w.y << 32), (uint64_t)rec.y, &c)) continue;
+            const uint4 e = __ldg((const uint4*)tab + rec.x + c);
+            if (!lemire64((uint64_t)w.z | ((uint64_t)w.w << 32), (uint64_t)e.y, &u)) continue;
+            return u < e.x ? e.z : e.w;
+        }
+    }
+    const uint4 rec = __ldg(&vrec[v]);
+    if (rec.y == 0) return v;
+    const uint64_t S = (uint64_t)rec.z | ((uint64_t)rec.w << 32);
+    if (MODE == 1) {
+        uint64_t x = 0;
+        for (uint32_t att = 0;; ++att) {
+            const pword4 w = path_draw(seed, r, t, att);
+            if (lemire64((uint64_t)w.x | ((uint64_t)w.y << 32), S, &x)) break;
+        }
+        return WIDE ? pick_prefix64((const uint4*)tab + rec.x, rec.y, x)
+                    : pick_prefix32((const uint2*)tab + rec.x, rec.y, (uint32_t)x);
+    }
+    uint64_t c = 0, u = 0;
+    for (uint32_t att = 0;; ++att) {
+        const pword4 w = path_draw(seed, r, t, att);
+        const bool ok0 = lemire64((uint64_t)w.x | ((uint64_t)w.y << 32), (uint64_t)rec.y, &c);
+        const bool ok1 = lemire64((uint64_t)w.z | ((uint64_t)w.w << 32), S, &u);
+        if (ok0 && ok1) break;
+    }
+    const uint4 e = __ldg((const uint4*)tab + rec.x + c);
+    return u < ((uint64_t)e.x | ((uint64_t)e.y << 32)) ? e.z : e.w;
+}
+
+__device__ __forceinline__ uint64_t walk_start(uint64_t seed, uint64_t r, int64_t n) {
+    uint64_t v = 0;
+    for (uint32_t att = 0;; ++att) {
+        const pword4 x = path_draw(seed, r, 0, att);
+        if (lemire64((uint64_t)x.x | ((uint64_t)x.y << 32), (uint64_t)n, &v)) return v;
+    }
+}
+
 template <int MODE, bool WIDE, int STRIDE>
-__global__ void __launch_bounds__(256, 5) sample_kernel(const uint4* __restrict__ vrec, const void* __restrict__ tab,
-                                                     int64_t n, uint64_t seed, int64_t r0, int64_t R, int T,
-                                                     int32_t* __restrict__ rows, uint32_t* status) {
+__global__ void __launch_bounds__(256, 5) sample_kernel(const uint4* __restrict__ vrec,
+                                                        const uint2* __restrict__ vsmall,
+                                                        const void* __restrict__ tab, int64_t n, uint64_t seed,
+                                                        int64_t r0, int64_t R, int T, int32_t* __restrict__ rows,
+                                                        uint32_t* status) {
     const int64_t nthreads = (int64_t)gridDim.x * blockDim.x;
     for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < R; r += nthreads) {
         int32_t p[STRIDE];
-        uint64_t v = 0;
-        for (uint32_t att = 0;; ++att) {
-            pword4 x = path_draw(seed, (uint64_t)(r0 + r), 0, att);
-            if (lemire64((uint64_t)x.x | ((uint64_t)x.y << 32), (uint64_t)n, &v)) break;
-        }
+        uint64_t v = walk_start(seed, (uint64_t)(r0 + r), n);
         p[0] = (int32_t)v;
 #pragma unroll
         for (int t = 1; t < STRIDE; ++t) {
+            p[t] = -1;
             if (t <= T) {
-                uint4 rec = __ldg(&vrec[v]);
-                if (rec.y != 0) {
-                    uint64_t S = (uint64_t)rec.z | ((uint64_t)rec.w << 32);
-                    if (MODE == 4) {
-                        // t_ij = 1/deg: Uniform[0, deg) from the same words as
-                        // the prefix draw, so the walk equals prefix selection
-                        // with every weight 1
-                        uint64_t c = 0;
-                        for (uint32_t att = 0;; ++att) {
-                            pword4 w = path_draw(seed, (uint64_t)(r0 + r), (uint32_t)t, att);
-                            if (lemire64((uint64_t)w.x | ((uint64_t)w.y << 32), (uint64_t)rec.y, &c)) break;
-                        }
-                        v = (uint64_t)(uint32_t)__ldg((const int32_t*)tab + rec.x + c);
-                    } else if (MODE == 1) {
-                        uint64_t x = 0;
-                        for (uint32_t att = 0;; ++att) {
-                            pword4 w = path_draw(seed, (uint64_t)(r0 + r), (uint32_t)t, att);
-                            if (lemire64((uint64_t)w.x | ((uint64_t)w.y << 32), S, &x)) break;
-                        }
-                        if (WIDE)
-                            v = pick_prefix64((const uint4*)tab + rec.x, rec.y, x);
-                        else
-                            v = pick_prefix32((const uint2*)tab + rec.x, rec.y, (uint32_t)x);
-                    } else {
-                        uint64_t c = 0, u = 0;
-                        for (uint32_t att = 0;; ++att) {
-                            pword4 w = path_draw(seed, (uint64_t)(r0 + r), (uint32_t)t, att);
-                            bool ok0 = lemire64((uint64_t)w.x | ((uint64_t)w.y << 32), (uint64_t)rec.y, &c);
-                            bool ok1 = lemire64((uint64_t)w.z | ((uint64_t)w.w << 32), S, &u);
-                            if (ok0 && ok1) break;
-                        }
-                        uint4 e = __ldg((const uint4*)tab + rec.x + c);
-                        uint64_t thr = (uint64_t)e.x | ((uint64_t)e.y << 32);
-                        v = u < thr ? e.z : e.w;
-                    }
-                    if (v >= (uint64_t)n) {   // a corrupt table entry: report, never index with it
-                        flag_status(status, ST_BAD_INDEX);
-                        v = 0;
-                    }
+                v = walk_step<MODE, WIDE>(vrec, vsmall, tab, seed, (uint64_t)(r0 + r), (uint32_t)t, v);
+                if (v >= (uint64_t)n) {   // a corrupt table entry: report, never index with it
+                    flag_status(status, ST_BAD_INDEX);
+                    v = 0;
                 }
                 p[t] = (int32_t)v;
-            } else {
-                p[t] = -1;
             }
         }
         int4* dst = (int4*)(rows + r * STRIDE);
@@ -118,64 +149,28 @@ __global__ void __launch_bounds__(256, 5) sample_kernel(const uint4* __restrict_
 // Rows of 64 or 128 entries (T >= 32): the same walk, but the row is not
 // held in registers; every 8 entries go out as two 16-byte stores.
 template <int MODE, bool WIDE>
-__global__ void __launch_bounds__(256) sample_long_kernel(const uint4* __restrict__ vrec, const void* __restrict__ tab,
-                                                          int64_t n, uint64_t seed, int64_t r0, int64_t R, int T,
-                                                          int stride, int32_t* __restrict__ rows, uint32_t* status) {
+__global__ void __launch_bounds__(256) sample_long_kernel(const uint4* __restrict__ vrec,
+                                                          const uint2* __restrict__ vsmall,
+                                                          const void* __restrict__ tab, int64_t n, uint64_t seed,
+                                                          int64_t r0, int64_t R, int T, int stride,
+                                                          int32_t* __restrict__ rows, uint32_t* status) {
     const int64_t nthreads = (int64_t)gridDim.x * blockDim.x;
     for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < R; r += nthreads) {
         int32_t buf[8];
         int4* dst = (int4*)(rows + r * stride);
-        uint64_t v = 0;
-        for (uint32_t att = 0;; ++att) {
-            pword4 x = path_draw(seed, (uint64_t)(r0 + r), 0, att);
-            if (lemire64((uint64_t)x.x | ((uint64_t)x.y << 32), (uint64_t)n, &v)) break;
-        }
+        uint64_t v = walk_start(seed, (uint64_t)(r0 + r), n);
         buf[0] = (int32_t)v;
         for (int t8 = 0; t8 < stride; t8 += 8) {
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
                 const int t = t8 + u;
                 if (t == 0) continue;
-                if (t > T) {
-                    buf[u] = -1;
-                    continue;
-                }
-                const uint4 rec = __ldg(&vrec[v]);
-                if (rec.y != 0) {
-                    const uint64_t S = (uint64_t)rec.z | ((uint64_t)rec.w << 32);
-                    if (MODE == 4) {
-                        uint64_t c = 0;
-                        for (uint32_t att = 0;; ++att) {
-                            pword4 w = path_draw(seed, (uint64_t)(r0 + r), (uint32_t)t, att);
-                            if (lemire64((uint64_t)w.x | ((uint64_t)w.y << 32), (uint64_t)rec.y, &c)) break;
-                        }
-                        v = (uint64_t)(uint32_t)__ldg((const int32_t*)tab + rec.x + c);
-                    } else if (MODE == 1) {
-                        uint64_t x = 0;
-                        for (uint32_t att = 0;; ++att) {
-                            pword4 w = path_draw(seed, (uint64_t)(r0 + r), (uint32_t)t, att);
-                            if (lemire64((uint64_t)w.x | ((uint64_t)w.y << 32), S, &x)) break;
-                        }
-                        if (WIDE)
-                            v = pick_prefix64((const uint4*)tab + rec.x, rec.y, x);
-                        else
-                            v = pick_prefix32((const uint2*)tab + rec.x, rec.y, (uint32_t)x);
-                    } else {
-                        uint64_t c = 0, uu = 0;
-                        for (uint32_t att = 0;; ++att) {
-                            pword4 w = path_draw(seed, (uint64_t)(r0 + r), (uint32_t)t, att);
-                            bool ok0 = lemire64((uint64_t)w.x | ((uint64_t)w.y << 32), (uint64_t)rec.y, &c);
-                            bool ok1 = lemire64((uint64_t)w.z | ((uint64_t)w.w << 32), S, &uu);
-                            if (ok0 && ok1) break;
-                        }
-                        const uint4 e = __ldg((const uint4*)tab + rec.x + c);
-                        const uint64_t thr = (uint64_t)e.x | ((uint64_t)e.y << 32);
-                        v = uu < thr ? e.z : e.w;
-                    }
-                    if (v >= (uint64_t)n) {
-                        flag_status(status, ST_BAD_INDEX);
-                        v = 0;
-                    }
+                buf[u] = -1;
+                if (t > T) continue;
+                v = walk_step<MODE, WIDE>(vrec, vsmall, tab, seed, (uint64_t)(r0 + r), (uint32_t)t, v);
+                if (v >= (uint64_t)n) {
+                    flag_status(status, ST_BAD_INDEX);
+                    v = 0;
                 }
                 buf[u] = (int32_t)v;
             }
@@ -190,13 +185,13 @@ void launch_sample(panther_ctx* ctx, const panther_graph* g, const void* tab, ui
                    int T, int stride, int32_t* rows, unsigned blocks) {
     cudaStream_t s = ctx->stream;
     if (stride == 8)
-        sample_kernel<MODE, WIDE, 8><<<blocks, 256, 0, s>>>(g->vrec, tab, g->n, seed, r0, R, T, rows, ctx->d_status);
+        sample_kernel<MODE, WIDE, 8><<<blocks, 256, 0, s>>>(g->vrec, g->vsmall, tab, g->n, seed, r0, R, T, rows, ctx->d_status);
     else if (stride == 16)
-        sample_kernel<MODE, WIDE, 16><<<blocks, 256, 0, s>>>(g->vrec, tab, g->n, seed, r0, R, T, rows, ctx->d_status);
+        sample_kernel<MODE, WIDE, 16><<<blocks, 256, 0, s>>>(g->vrec, g->vsmall, tab, g->n, seed, r0, R, T, rows, ctx->d_status);
     else if (stride == 32)
-        sample_kernel<MODE, WIDE, 32><<<blocks, 256, 0, s>>>(g->vrec, tab, g->n, seed, r0, R, T, rows, ctx->d_status);
+        sample_kernel<MODE, WIDE, 32><<<blocks, 256, 0, s>>>(g->vrec, g->vsmall, tab, g->n, seed, r0, R, T, rows, ctx->d_status);
     else
-        sample_long_kernel<MODE, WIDE><<<blocks, 256, 0, s>>>(g->vrec, tab, g->n, seed, r0, R, T, stride, rows,
+        sample_long_kernel<MODE, WIDE><<<blocks, 256, 0, s>>>(g->vrec, g->vsmall, tab, g->n, seed, r0, R, T, stride, rows,
                                                               ctx->d_status);
 }
 
@@ -238,7 +233,10 @@ extern "C" panther_status panther_sample_paths_range(panther_ctx* ctx, const pan
         else
             launch_sample<1, false>(ctx, g, g->prefix, seed, r0, R, T, p->stride, p->rows, blocks);
     } else if (mode == PANTHER_MODE_ALIAS) {
-        launch_sample<2, false>(ctx, g, g->alias, seed, r0, R, T, p->stride, p->rows, blocks);
+        if (g->prefix_wide)
+            launch_sample<2, true>(ctx, g, g->alias, seed, r0, R, T, p->stride, p->rows, blocks);
+        else
+            launch_sample<2, false>(ctx, g, g->alias, seed, r0, R, T, p->stride, p->rows, blocks);
     } else {
         launch_sample<4, false>(ctx, g, g->col, seed, r0, R, T, p->stride, p->rows, blocks);
     }
