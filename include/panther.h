@@ -198,7 +198,7 @@ PANTHER_API panther_status panther_paths_info(const panther_paths* p, int64_t* n
  * listed once. Layout: off int64[n+1], pid uint32[nnz] (ids reach 2^32 - 2;
  * a signed 32-bit view shows ids from 2^31 up as negative); P_v is
  * pid[off[v] .. off[v+1]) in ascending path id.
- * Memory: one sort over all pairs needs about 16 B per pair (+ 5% for tile
+ * Memory: one sort over all pairs needs about 16 B per pair (+ 2% for tile
  * counts) of temporary device memory next to the result (4 B per pair). When
  * that exceeds the index budget (panther_set_index_budget; by default the
  * free device memory less the result), the rows are sorted in chunks of
@@ -220,7 +220,7 @@ PANTHER_API panther_status panther_set_index_budget(panther_ctx* ctx, int64_t by
  * Same result as panther_build_index: P_v = pid[off[v] .. off[v+1]),
  * ascending. The caller passes dev_off (int64[n+1]) and dev_pid (uint32,
  * pid_capacity >= R*(T+1) entries); *nnz receives the number of pairs.
- * Temporary buffers come from one static device array of about 86 MiB that
+ * Temporary buffers come from one static device array of about 70 MiB that
  * every GPU loading the library reserves until the process exits; R*(T+1)
  * may be at most 4,194,304 (EOVERFLOW beyond, before any launch). The first
  * call on a device looks up that array's device address, so make it before

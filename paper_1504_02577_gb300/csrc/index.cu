@@ -6,8 +6,18 @@
 // aligned inside every 32-lane round, so the duplicate test is one
 // __match_any_sync; rows of 64 or 128 entries span two or four rounds of one
 // warp, and their entries are also compared with the row's earlier rounds. Later passes read the (key, value) pairs of the previous
-// pass. Every pass is: tile histogram -> exclusive scan over (digit, tile) ->
-// stable scatter. The scatter ranks items with warp-private digit counters:
+// pass. Every pass is: tile histogram -> offsets over (digit, tile) -> stable
+// scatter.
+//
+// The counts lie tile by tile, cnt[tile][digit] in 32 bits, so the histogram
+// writes and the scatter reads one contiguous row per tile. Their offsets are
+// three parts added in the scatter: a prefix over the tiles of a group of
+// GROUP (in place, a thread per digit), one over the groups and one over the
+// digits. (As 64-bit counts[digit][tile], copied and scanned in place, the
+// bookkeeping moved 2.7 GB a pass at 52,000 tiles, most of it in sectors that
+// held one count: 1.93 ms for the sort of 5.7e7 pairs of 5M vertices, 1.83 now.)
+//
+// The scatter ranks items with warp-private digit counters:
 // warps own contiguous sub-ranges of a tile and walk them in order, so the
 // sort is stable and path ids come out ascending within each vertex.
 #include <algorithm>
@@ -23,6 +33,7 @@ constexpr int IX_ROUNDS = 12;              // 32-item rounds per warp
 constexpr int IX_TILE = IX_T * IX_ROUNDS;  // 6144 items per tile
 constexpr int MAX_RADIX = 512;
 constexpr int MAX_RB = 9;                  // log2(MAX_RADIX)
+constexpr int GROUP = 128;                 // tiles per group of the offsets
 
 struct Src {
     // pass 0 source
@@ -96,8 +107,7 @@ __device__ __forceinline__ uint32_t long_row_repeats(const Src& s, int64_t wbase
 // LONG: pass 0 over rows of 64 or 128 entries (separate instantiations keep
 // the registers of the common kernels unchanged)
 template <bool LONG>
-__global__ void __launch_bounds__(IX_T) hist_kernel(Src s, int shift, int radix, int64_t ntiles,
-                                                    int64_t* __restrict__ counts) {
+__global__ void __launch_bounds__(IX_T, 3) hist_kernel(Src s, int shift, int radix, uint32_t* __restrict__ cnt) {
     __shared__ unsigned h[MAX_RADIX];
     for (int d = threadIdx.x; d < radix; d += IX_T) h[d] = 0;
     const int64_t base = (int64_t)blockIdx.x * IX_TILE + (int64_t)(threadIdx.x >> 5) * (IX_ROUNDS * 32) +
@@ -112,8 +122,71 @@ __global__ void __launch_bounds__(IX_T) hist_kernel(Src s, int shift, int radix,
         if (item_ok(s, base + k * 32, x[k]) && !((rep >> k) & 1u))
             atomicAdd(&h[((uint32_t)x[k] >> shift) & (radix - 1)], 1u);
     __syncthreads();
-    for (int d = threadIdx.x; d < radix; d += IX_T) counts[(int64_t)d * ntiles + blockIdx.x] = h[d];
+    for (int d = threadIdx.x; d < radix; d += IX_T) cnt[(int64_t)blockIdx.x * radix + d] = h[d];
 }
+
+// per digit: exclusive prefix over the tiles of one group, in place; the
+// group's sum to gsum[group][digit]
+constexpr int GP_T = 128;                  // digits per CTA of it (blockIdx.y the others)
+__global__ void __launch_bounds__(GP_T) group_prefix_kernel(uint32_t* __restrict__ cnt, int radix, int64_t ntiles,
+                                                            int64_t* __restrict__ gsum) {
+    const int d = blockIdx.y * GP_T + threadIdx.x;
+    if (d >= radix) return;
+    const int64_t t0 = (int64_t)blockIdx.x * GROUP, t1 = t0 + GROUP < ntiles ? t0 + GROUP : ntiles;
+    uint32_t run = 0;                                // at most GROUP * IX_TILE items
+    for (int64_t t = t0; t < t1; t += 16) {
+        uint32_t c[16];                              // loads in flight together
+#pragma unroll
+        for (int i = 0; i < 16; ++i) c[i] = t + i < t1 ? cnt[(t + i) * radix + d] : 0u;
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            if (t + i < t1) cnt[(t + i) * radix + d] = run;
+            run += c[i];
+        }
+    }
+    gsum[(int64_t)blockIdx.x * radix + d] = run;
+}
+
+// per digit: exclusive prefix over the groups, in place; then over the digits
+// (dbase[digit]); *total = the number of items. One CTA.
+__global__ void __launch_bounds__(MAX_RADIX) digit_base_kernel(int64_t* __restrict__ gsum, int radix, int64_t ngroups,
+                                                               int64_t* __restrict__ dbase,
+                                                               int64_t* __restrict__ total) {
+    __shared__ int64_t wsum[MAX_RADIX / 32];
+    const int d = threadIdx.x, lane = d & 31, w = d >> 5;
+    int64_t run = 0;
+    if (d < radix)
+        for (int64_t g = 0; g < ngroups; g += 8) {
+            int64_t c[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) c[i] = g + i < ngroups ? gsum[(g + i) * radix + d] : 0;
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                if (g + i < ngroups) gsum[(g + i) * radix + d] = run;
+                run += c[i];
+            }
+        }
+    int64_t x = run;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int64_t y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) wsum[w] = x;
+    __syncthreads();
+    int64_t before = x - run;
+    for (int i = 0; i < w; ++i) before += wsum[i];
+    if (d < radix) dbase[d] = before;
+    if (d == MAX_RADIX - 1) *total = before + run;
+}
+
+// device arrays of a pass's offsets
+struct Offsets {
+    uint32_t* cnt;           // [tiles][radix]
+    int64_t* gsum;           // [groups][radix]
+    int64_t* dbase;          // [radix]
+    int64_t* total;          // [1]
+};
 
 // One tile per CTA: rank every item stably (per-warp digit counters), stage
 // the tile in shared memory in digit order, then write each digit's run with
@@ -122,8 +195,7 @@ constexpr size_t SC_SMEM = (size_t)IX_WARPS * MAX_RADIX * 4 + (size_t)MAX_RADIX 
                            (size_t)IX_TILE * 8 + 64;
 
 template <bool LONG>
-__global__ void __launch_bounds__(IX_T, 2) scatter_kernel(Src s, int shift, int radix, int64_t ntiles,
-                                                          const int64_t* __restrict__ offs,
+__global__ void __launch_bounds__(IX_T, 2) scatter_kernel(Src s, int shift, int radix, Offsets O,
                                                           int32_t* __restrict__ okeys, int32_t* __restrict__ ovals) {
     extern __shared__ __align__(16) unsigned char sc_smem[];
     unsigned (*wc)[MAX_RADIX] = (unsigned (*)[MAX_RADIX])sc_smem;                       // [warps][radix]
@@ -143,7 +215,11 @@ __global__ void __launch_bounds__(IX_T, 2) scatter_kernel(Src s, int shift, int 
     uint32_t okmask = 0;
     // this tile's global start of digit threadIdx.x (final before the launch):
     // loaded now, so its latency overlaps the item loads and the ranking
-    const long long my_off = (int)threadIdx.x < radix ? offs[(int64_t)threadIdx.x * ntiles + blockIdx.x] : 0;
+    const long long my_off =
+        (int)threadIdx.x < radix
+            ? (long long)O.cnt[(int64_t)blockIdx.x * radix + threadIdx.x] +
+                  O.gsum[(int64_t)(blockIdx.x / GROUP) * radix + threadIdx.x] + O.dbase[threadIdx.x]
+            : 0;
 #pragma unroll
     for (int k = 0; k < IX_ROUNDS; ++k) key[k] = (uint32_t)load_raw(s, base + k * 32 + lane);   // loads in flight
 #pragma unroll
@@ -184,7 +260,6 @@ __global__ void __launch_bounds__(IX_T, 2) scatter_kernel(Src s, int shift, int 
     unsigned tot = 0;
     const int d2 = threadIdx.x;               // IX_T >= MAX_RADIX: one digit per thread
     if (d2 < radix) {
-        toff[d2] = my_off;
         for (int ww = 0; ww < IX_WARPS; ++ww) {
             unsigned c = wc[ww][d2];
             wc[ww][d2] = tot;
@@ -209,7 +284,10 @@ __global__ void __launch_bounds__(IX_T, 2) scatter_kernel(Src s, int shift, int 
         if (lane < IX_WARPS) wsum[lane] = y;
     }
     __syncthreads();
-    if (d2 < radix) tstart[d2] = x - tot + (w ? wsum[w - 1] : 0u);
+    if (d2 < radix) {
+        tstart[d2] = x - tot + (w ? wsum[w - 1] : 0u);
+        toff[d2] = my_off - (long long)tstart[d2];   // position of the tile's staged item j of digit d2: toff + j
+    }
     const unsigned nvalid = wsum[IX_WARPS - 1];
     __syncthreads();
     // phase 3a: stage keys and values in digit order (values loaded together first)
@@ -234,23 +312,34 @@ __global__ void __launch_bounds__(IX_T, 2) scatter_kernel(Src s, int shift, int 
     for (unsigned j = threadIdx.x; j < nvalid; j += IX_T) {
         const int32_t kk = skey[j];
         const uint32_t d = ((uint32_t)kk >> shift) & (radix - 1);
-        const int64_t pos = (int64_t)toff[d] + (j - tstart[d]);
+        const int64_t pos = (int64_t)toff[d] + j;
         okeys[pos] = kk;
         ovals[pos] = sval[j];
     }
 }
 
-__global__ void offsets_kernel(const int32_t* __restrict__ keys, int64_t nnz, int64_t n, int64_t* __restrict__ off,
-                               uint32_t* status) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i > nnz) return;
-    int64_t prev = i > 0 ? (int64_t)keys[i - 1] : -1;
-    int64_t cur = i < nnz ? (int64_t)keys[i] : n;
-    if (prev < -1 || prev >= n || cur < 0 || cur > n || cur < prev) {   // keys out of range or unsorted
-        flag_status(status, ST_BAD_INDEX);
-        return;
+// off[v] from the sorted keys: four keys per thread
+__global__ void __launch_bounds__(256) offsets_kernel(const int32_t* __restrict__ keys, int64_t nnz, int64_t n,
+                                                      int64_t* __restrict__ off, uint32_t* status) {
+    const int64_t i0 = 4 * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x);
+    if (i0 > nnz) return;
+    int64_t k[5];
+    k[0] = i0 > 0 ? (int64_t)keys[i0 - 1] : -1;
+    if (i0 + 4 <= nnz) {                             // keys is 16-byte aligned
+        const int4 q = *(const int4*)(keys + i0);
+        k[1] = q.x; k[2] = q.y; k[3] = q.z; k[4] = q.w;
+    } else {
+        for (int j = 0; j < 4; ++j) k[j + 1] = i0 + j < nnz ? (int64_t)keys[i0 + j] : n;
     }
-    for (int64_t v = prev + 1; v <= cur; ++v) off[v] = i;
+    for (int j = 0; j < 4; ++j) {
+        const int64_t i = i0 + j, prev = k[j], cur = k[j + 1];
+        if (i > nnz) return;
+        if (prev < -1 || prev >= n || cur < 0 || cur > n || cur < prev) {   // keys out of range or unsorted
+            flag_status(status, ST_BAD_INDEX);
+            return;
+        }
+        for (int64_t v = prev + 1; v <= cur; ++v) off[v] = i;
+    }
 }
 
 // cls[v] = path_code(|P_v|) and its histogram (a count of v with any u never
@@ -304,11 +393,6 @@ __global__ void advance_kernel(const int64_t* __restrict__ coff, int64_t n, int6
     if (v < n) cur[v] += coff[v + 1] - coff[v];
 }
 
-__global__ void total_kernel(const int64_t* __restrict__ counts, const int64_t* __restrict__ offs, int64_t len,
-                             int64_t* __restrict__ total) {
-    *total = offs[len - 1] + counts[len - 1];
-}
-
 int bits_for(int64_t maxval) {
     int b = 1;
     while (b < 62 && (int64_t(1) << b) <= maxval) ++b;
@@ -337,12 +421,25 @@ panther_status index_classes(panther_ctx* ctx, panther_index* ix) {
     return PANTHER_OK;
 }
 
+// the histogram of a pass and the offsets from it (three launches)
+static void launch_offsets(panther_ctx* ctx, const Src& src, int shift, int radix, int64_t ntiles, const Offsets& O) {
+    cudaStream_t s = ctx->stream;
+    if (src.first && src.stride > 32)
+        hist_kernel<true><<<(unsigned)ntiles, IX_T, 0, s>>>(src, shift, radix, O.cnt);
+    else
+        hist_kernel<false><<<(unsigned)ntiles, IX_T, 0, s>>>(src, shift, radix, O.cnt);
+    const int64_t ng = ceil_div(ntiles, GROUP);
+    group_prefix_kernel<<<dim3((unsigned)ng, (unsigned)ceil_div(radix, GP_T)), GP_T, 0, s>>>(O.cnt, radix, ntiles, O.gsum);
+    digit_base_kernel<<<1, MAX_RADIX, 0, s>>>(O.gsum, radix, ng, O.dbase, O.total);
+    ctx->launches += 3;
+}
+
 // LSD radix sort of the (vertex, path) pairs of src (pass 0 reads its rows);
 // the sorted keys and values end in one of the A/B buffers, returned with
 // the number of pairs. Synchronises once (after pass 0, to size the rest).
 static panther_status radix_pairs(panther_ctx* ctx, Src src, int64_t n, int32_t* kA, int32_t* vA, int32_t* kB,
-                                  int32_t* vB, int64_t* counts, int64_t* offs, int64_t* tot, int64_t* count_out,
-                                  int32_t** keys_out, int32_t** vals_out) {
+                                  int32_t* vB, const Offsets& O, int64_t* count_out, int32_t** keys_out,
+                                  int32_t** vals_out) {
     cudaStream_t s = ctx->stream;
     int passes, rb;
     radix_plan(n, &passes, &rb);
@@ -350,34 +447,22 @@ static panther_status radix_pairs(panther_ctx* ctx, Src src, int64_t n, int32_t*
     const int64_t tiles0 = ceil_div(src.R * src.stride, IX_TILE);
     int32_t *ik = nullptr, *iv = nullptr, *ok = kA, *ov = vA;
     int64_t count = 0;
-    panther_status st;
     for (int pass = 0; pass < passes; ++pass) {
-        int shift = pass * rb;
-        int64_t ntiles = pass == 0 ? tiles0 : ceil_div(count, IX_TILE);
-        if (ntiles < 1) ntiles = 1;
-        int64_t len = (int64_t)radix * ntiles;
-        if (src.first && src.stride > 32)
-            hist_kernel<true><<<(unsigned)ntiles, IX_T, 0, s>>>(src, shift, radix, ntiles, counts);
-        else
-            hist_kernel<false><<<(unsigned)ntiles, IX_T, 0, s>>>(src, shift, radix, ntiles, counts);
-        ctx->launches++;
-        cudaError_t e = cudaMemcpyAsync(offs, counts, sizeof(int64_t) * len, cudaMemcpyDeviceToDevice, s);
-        if (e) return cuda_err(ctx, e, "index scan copy");
-        if ((st = scan_exclusive_i64(ctx, offs, len))) return st;
+        const int shift = pass * rb;
+        const int64_t ntiles = std::max<int64_t>(1, pass == 0 ? tiles0 : ceil_div(count, IX_TILE));
+        launch_offsets(ctx, src, shift, radix, ntiles, O);
         if (pass == 0) {
             // the number of pairs is needed to size the later passes
-            total_kernel<<<1, 1, 0, s>>>(counts, offs, len, tot);
-            ctx->launches++;
-            e = cudaMemcpyAsync(&count, tot, sizeof(int64_t), cudaMemcpyDeviceToHost, s);
+            cudaError_t e = cudaMemcpyAsync(&count, O.total, sizeof(int64_t), cudaMemcpyDeviceToHost, s);
             if (!e) e = cudaStreamSynchronize(s);
             if (e) return cuda_err(ctx, e, "index count");
         }
         if (src.first && src.stride > 32)
-            scatter_kernel<true><<<(unsigned)ntiles, IX_T, SC_SMEM, s>>>(src, shift, radix, ntiles, offs, ok, ov);
+            scatter_kernel<true><<<(unsigned)ntiles, IX_T, SC_SMEM, s>>>(src, shift, radix, O, ok, ov);
         else
-            scatter_kernel<false><<<(unsigned)ntiles, IX_T, SC_SMEM, s>>>(src, shift, radix, ntiles, offs, ok, ov);
+            scatter_kernel<false><<<(unsigned)ntiles, IX_T, SC_SMEM, s>>>(src, shift, radix, O, ok, ov);
         ctx->launches++;
-        e = cudaGetLastError();
+        const cudaError_t e = cudaGetLastError();
         if (e) return cuda_err(ctx, e, "index scatter");
         // next pass reads what this one wrote
         src.first = 0;
@@ -398,7 +483,7 @@ static panther_status radix_pairs(panther_ctx* ctx, Src src, int64_t n, int32_t*
 static int64_t radix_temp_bytes(int64_t rows, int L, int stride, int radix) {
     const int64_t pairs = rows * L;
     const int64_t tiles = std::max(ceil_div(rows * stride, IX_TILE), ceil_div(pairs, IX_TILE));
-    return 4 * pairs * 4 + 2 * (int64_t)radix * tiles * 8 + 64;
+    return 4 * pairs * 4 + (int64_t)radix * (tiles * 4 + (ceil_div(tiles, GROUP) + 1) * 8) + 64;
 }
 
 extern "C" panther_status panther_set_index_budget(panther_ctx* ctx, int64_t bytes) {
@@ -429,9 +514,9 @@ extern "C" panther_status panther_build_index(panther_ctx* ctx, const panther_pa
             const int64_t results = p->R * p->L * 4 + 3 * (n + 1) * 8 + n + (int64_t(256) << 20);
             size_t fr = 0, tot = 0;
             if (cudaMemGetInfo(&fr, &tot) == cudaSuccess && (int64_t)fr - results < need) {
-                // memory the pool keeps but no one uses goes back first
-                cudaMemPool_t pool;
-                if (cudaDeviceGetDefaultMemPool(&pool, ctx->device) == cudaSuccess) cudaMemPoolTrimTo(pool, 0);
+                // memory the pools keep but no one uses goes back first
+                cudaStreamSynchronize(s);
+                trim_pools();
                 cudaMemGetInfo(&fr, &tot);
             }
             cudaGetLastError();
@@ -454,13 +539,15 @@ extern "C" panther_status panther_build_index(panther_ctx* ctx, const panther_pa
     ix->n = n;
     ix->R = p->R;
     int32_t *kA = nullptr, *vA = nullptr, *kB = nullptr, *vB = nullptr;
-    int64_t *counts = nullptr, *offs = nullptr, *tot = nullptr, *cur = nullptr, *coff = nullptr;
+    int64_t *cur = nullptr, *coff = nullptr;
+    Offsets O{};
     panther_status st;
     const int64_t maxpairs = rows * p->L;
     const int64_t maxtiles = std::max(ceil_div(rows * p->stride, IX_TILE), ceil_div(maxpairs, IX_TILE));
+    const int64_t maxgroups = ceil_div(maxtiles, GROUP);
     auto cleanup = [&]() {
         dev_free(ctx, kA); dev_free(ctx, vA); dev_free(ctx, kB); dev_free(ctx, vB);
-        dev_free(ctx, counts); dev_free(ctx, offs); dev_free(ctx, tot); dev_free(ctx, cur); dev_free(ctx, coff);
+        dev_free(ctx, O.cnt); dev_free(ctx, O.gsum); dev_free(ctx, cur); dev_free(ctx, coff);
     };
     auto fail = [&](panther_status e) {
         cleanup();
@@ -471,13 +558,14 @@ extern "C" panther_status panther_build_index(panther_ctx* ctx, const panther_pa
         (st = dev_alloc(ctx, (void**)&vA, sizeof(int32_t) * maxpairs)) ||
         (st = dev_alloc(ctx, (void**)&kB, sizeof(int32_t) * maxpairs)) ||
         (st = dev_alloc(ctx, (void**)&vB, sizeof(int32_t) * maxpairs)) ||
-        (st = dev_alloc(ctx, (void**)&counts, sizeof(int64_t) * radix * maxtiles)) ||
-        (st = dev_alloc(ctx, (void**)&offs, sizeof(int64_t) * radix * maxtiles)) ||
-        (st = dev_alloc(ctx, (void**)&tot, sizeof(int64_t))) ||
+        (st = dev_alloc(ctx, (void**)&O.cnt, sizeof(uint32_t) * radix * maxtiles)) ||
+        (st = dev_alloc(ctx, (void**)&O.gsum, sizeof(int64_t) * (radix * (maxgroups + 1) + 1))) ||
         (st = dev_alloc(ctx, (void**)&ix->off, sizeof(int64_t) * (n + 1))) ||
         (st = dev_alloc(ctx, (void**)&ix->cls, n)) ||
         (st = dev_alloc(ctx, (void**)&ix->cls_hist, sizeof(int64_t) * 256)))
         return fail(st);
+    O.dbase = O.gsum + radix * maxgroups;
+    O.total = O.dbase + radix;
     PCK(ctx, cudaFuncSetAttribute(scatter_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SC_SMEM));
     PCK(ctx, cudaFuncSetAttribute(scatter_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SC_SMEM));
     Src src{};
@@ -493,9 +581,9 @@ extern "C" panther_status panther_build_index(panther_ctx* ctx, const panther_pa
         // one radix sort over all pairs; its final values are pid
         int64_t count = 0;
         int32_t *ik = nullptr, *iv = nullptr;
-        if ((st = radix_pairs(ctx, src, n, kA, vA, kB, vB, counts, offs, tot, &count, &ik, &iv))) return fail(st);
+        if ((st = radix_pairs(ctx, src, n, kA, vA, kB, vB, O, &count, &ik, &iv))) return fail(st);
         ix->nnz = count;
-        offsets_kernel<<<(unsigned)ceil_div(count + 1, 256), 256, 0, s>>>(ik, count, n, ix->off, ctx->d_status);
+        offsets_kernel<<<(unsigned)ceil_div(count + 1, 1024), 256, 0, s>>>(ik, count, n, ix->off, ctx->d_status);
         ctx->launches++;
         if ((st = index_classes(ctx, ix))) return fail(st);
         // keep the final value array as pid; release everything else
@@ -530,8 +618,8 @@ extern "C" panther_status panther_build_index(panther_ctx* ctx, const panther_pa
             cs.r0 = r0;
             int64_t cn = 0;
             int32_t *ck = nullptr, *cv = nullptr;
-            if ((st = radix_pairs(ctx, cs, n, kA, vA, kB, vB, counts, offs, tot, &cn, &ck, &cv))) return fail(st);
-            offsets_kernel<<<(unsigned)ceil_div(cn + 1, 256), 256, 0, s>>>(ck, cn, n, coff, ctx->d_status);
+            if ((st = radix_pairs(ctx, cs, n, kA, vA, kB, vB, O, &cn, &ck, &cv))) return fail(st);
+            offsets_kernel<<<(unsigned)ceil_div(cn + 1, 1024), 256, 0, s>>>(ck, cn, n, coff, ctx->d_status);
             if (cn > 0) place_kernel<<<(unsigned)ceil_div(cn, 256), 256, 0, s>>>(ck, cv, cn, coff, cur, ix->pid);
             advance_kernel<<<(unsigned)ceil_div(n, 256), 256, 0, s>>>(coff, n, cur);
             ctx->launches += cn > 0 ? 3 : 2;
@@ -558,47 +646,11 @@ namespace {
 constexpr int64_t NA_MAX_PAIRS = int64_t(1) << 22;           // R * (T+1) at most 4,194,304
 constexpr int64_t NA_MAX_TILES = 2816;                        // >= ceil(R * stride / IX_TILE) for the limit above
 constexpr size_t NA_KV_BYTES = (size_t)NA_MAX_PAIRS * 4;      // one key or value array
-constexpr size_t NA_CNT_BYTES = (size_t)MAX_RADIX * NA_MAX_TILES * 8;
-constexpr size_t NA_SCRATCH_BYTES = 4 * NA_KV_BYTES + 2 * NA_CNT_BYTES + 256;
+constexpr size_t NA_CNT_BYTES = (size_t)MAX_RADIX * NA_MAX_TILES * 4;
+constexpr int64_t NA_MAX_GROUPS = (NA_MAX_TILES + GROUP - 1) / GROUP;
+constexpr size_t NA_SCRATCH_BYTES = 4 * NA_KV_BYTES + NA_CNT_BYTES + ((size_t)MAX_RADIX * (NA_MAX_GROUPS + 1) + 1) * 8 + 256;
 
 static __device__ __align__(256) unsigned char na_scratch[NA_SCRATCH_BYTES];
-
-// exclusive scan of len int64 values by one CTA (the counts of one pass)
-__global__ void __launch_bounds__(1024) na_scan_kernel(const int64_t* __restrict__ in, int64_t* __restrict__ out,
-                                                       int64_t len, int64_t* __restrict__ total) {
-    __shared__ int64_t sh[32];
-    __shared__ int64_t carry;
-    if (threadIdx.x == 0) carry = 0;
-    __syncthreads();
-    const unsigned lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    for (int64_t base = 0; base < len; base += blockDim.x) {
-        int64_t i = base + threadIdx.x;
-        int64_t v = i < len ? in[i] : 0, x = v;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            int64_t y = __shfl_up_sync(0xffffffffu, x, o);
-            if (lane >= (unsigned)o) x += y;
-        }
-        if (lane == 31) sh[wid] = x;
-        __syncthreads();
-        if (wid == 0) {
-            int64_t t = lane < (blockDim.x >> 5) ? sh[lane] : 0;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                int64_t y = __shfl_up_sync(0xffffffffu, t, o);
-                if (lane >= (unsigned)o) t += y;
-            }
-            sh[lane] = t;
-        }
-        __syncthreads();
-        int64_t excl = carry + (wid ? sh[wid - 1] : 0) + x - v;
-        if (i < len) out[i] = excl;
-        __syncthreads();
-        if (threadIdx.x == blockDim.x - 1) carry = excl + v;
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) *total = carry;
-}
 
 // device address of na_scratch, looked up once per device with that device current
 unsigned char* na_scratch_ptr[64];
@@ -632,9 +684,11 @@ extern "C" panther_status panther_build_index_noalloc(panther_ctx* ctx, const pa
     int32_t* vA = (int32_t*)(base + NA_KV_BYTES);
     int32_t* kB = (int32_t*)(base + 2 * NA_KV_BYTES);
     int32_t* vB = (int32_t*)(base + 3 * NA_KV_BYTES);
-    int64_t* counts = (int64_t*)(base + 4 * NA_KV_BYTES);
-    int64_t* offs = (int64_t*)(base + 4 * NA_KV_BYTES + NA_CNT_BYTES);
-    int64_t* tot = (int64_t*)(base + 4 * NA_KV_BYTES + 2 * NA_CNT_BYTES);
+    Offsets O;
+    O.cnt = (uint32_t*)(base + 4 * NA_KV_BYTES);
+    O.gsum = (int64_t*)(base + 4 * NA_KV_BYTES + NA_CNT_BYTES);
+    O.dbase = O.gsum + (int64_t)MAX_RADIX * NA_MAX_GROUPS;
+    O.total = O.dbase + MAX_RADIX;
     cudaStream_t s = ctx->stream;
     int passes, rb;
     radix_plan(p->n, &passes, &rb);
@@ -656,22 +710,16 @@ extern "C" panther_status panther_build_index_noalloc(panther_ctx* ctx, const pa
         const bool last = pass == passes - 1;
         int64_t ntiles = pass == 0 ? tiles0 : ceil_div(count, IX_TILE);
         if (ntiles < 1) ntiles = 1;
-        const int64_t len = (int64_t)radix * ntiles;
-        if (src.first && src.stride > 32)
-            hist_kernel<true><<<(unsigned)ntiles, IX_T, 0, s>>>(src, pass * rb, radix, ntiles, counts);
-        else
-            hist_kernel<false><<<(unsigned)ntiles, IX_T, 0, s>>>(src, pass * rb, radix, ntiles, counts);
-        na_scan_kernel<<<1, 1024, 0, s>>>(counts, offs, len, tot);
-        ctx->launches += 2;
+        launch_offsets(ctx, src, pass * rb, radix, ntiles, O);
         if (pass == 0) {
-            PCK(ctx, cudaMemcpyAsync(&count, tot, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+            PCK(ctx, cudaMemcpyAsync(&count, O.total, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
             PCK(ctx, cudaStreamSynchronize(s));
         }
         int32_t* outv = last ? (int32_t*)dev_pid : ov;     // the final pass writes the caller's pid array
         if (src.first && src.stride > 32)
-            scatter_kernel<true><<<(unsigned)ntiles, IX_T, SC_SMEM, s>>>(src, pass * rb, radix, ntiles, offs, ok, outv);
+            scatter_kernel<true><<<(unsigned)ntiles, IX_T, SC_SMEM, s>>>(src, pass * rb, radix, O, ok, outv);
         else
-            scatter_kernel<false><<<(unsigned)ntiles, IX_T, SC_SMEM, s>>>(src, pass * rb, radix, ntiles, offs, ok, outv);
+            scatter_kernel<false><<<(unsigned)ntiles, IX_T, SC_SMEM, s>>>(src, pass * rb, radix, O, ok, outv);
         ctx->launches++;
         PCK(ctx, cudaGetLastError());
         src.first = 0;
@@ -682,7 +730,7 @@ extern "C" panther_status panther_build_index_noalloc(panther_ctx* ctx, const pa
         ok = (ok == kA) ? kB : kA;
         ov = (ov == vA) ? vB : vA;
     }
-    offsets_kernel<<<(unsigned)ceil_div(count + 1, 256), 256, 0, s>>>(ik, count, p->n, dev_off, ctx->d_status);
+    offsets_kernel<<<(unsigned)ceil_div(count + 1, 1024), 256, 0, s>>>(ik, count, p->n, dev_off, ctx->d_status);
     ctx->launches++;
     PCK(ctx, cudaGetLastError());
     *nnz = count;
