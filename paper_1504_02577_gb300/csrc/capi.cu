@@ -299,6 +299,7 @@ void pantherpp_free_vecs(pantherpp_vecs* v) {
     dev_free(c, v->cnrm);
     dev_free(c, v->cncf);
     dev_free(c, v->ctile);
+    dev_free(c, v->ctmax);
     dev_free(c, v->norm2);
     dev_free(c, v->nrm);
     dev_free(c, v->exact);

@@ -108,6 +108,7 @@ struct pantherpp_vecs {
     float* cnrm = nullptr;           // [npad] |b| rounded up
     float* cncf = nullptr;           // [npad] |b|^2 rounded up
     uint8_t* ctile = nullptr;        // [npad/256] 1 if the tile holds only exact rows
+    float2* ctmax = nullptr;         // [npad/256] largest cnrm and cncf of the tile's rows
 };
 
 // ------------------------------------------------------------ host helpers ---

@@ -194,6 +194,30 @@ __global__ void __launch_bounds__(256) vec_arow_kernel(const uint32_t* __restric
     }
 }
 
+// largest norm and squared norm of each candidate tile (a warp per tile): the
+// error bound of any of its pairs is at most the one with these
+__global__ void __launch_bounds__(256) tile_max_kernel(const int32_t* __restrict__ cid, const float* __restrict__ cnrm,
+                                                       const float* __restrict__ cncf, float2* __restrict__ out,
+                                                       int64_t ntiles) {
+    const int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (t >= ntiles) return;                         // warp-uniform
+    float a = 0.f, b = 0.f;
+#pragma unroll
+    for (int j = 0; j < KN_N / 32; ++j) {
+        const int64_t i = t * KN_N + j * 32 + (threadIdx.x & 31);
+        if (cid[i] >= 0) {                           // padding has no pairs
+            a = fmaxf(a, cnrm[i]);
+            b = fmaxf(b, cncf[i]);
+        }
+    }
+#pragma unroll
+    for (int o = 16; o; o >>= 1) {
+        a = fmaxf(a, __shfl_xor_sync(0xffffffffu, a, o));
+        b = fmaxf(b, __shfl_xor_sync(0xffffffffu, b, o));
+    }
+    if ((threadIdx.x & 31) == 0) out[t] = make_float2(a, b);
+}
+
 // out[t] = every id of tile t is padding or an exact row (a warp per tile)
 __global__ void __launch_bounds__(256) tile_flags_kernel(const uint8_t* __restrict__ exact,
                                                          const int32_t* __restrict__ ids, int64_t count, int tile,
@@ -383,21 +407,10 @@ __device__ __noinline__ Row take_bounded(Row r, const RowConst& c, float y, floa
     return r;
 }
 
-// smallest upper bound of a group's keys (SEED), from the smallest of its
-// values when the tile is exact (+inf when it holds padding only: exact keys
-// lie below 2^24, padding's is 2^40)
-__device__ __forceinline__ float seed_exact(float m) {
-    return m < 1099511627776.0f ? m : __int_as_float(0x7f800000);
-}
-__device__ __forceinline__ float seed_bounded(const RowConst& c, const uint32_t (&y)[32], const int32_t* cid,
-                                              const float* cnrm, const float* cncf) {
-    float m = __int_as_float(0x7f800000);
-#pragma unroll
-    for (int j = 0; j < 32; ++j) {
-        const float E = fmaf(c.anrm, cnrm[j], fmaf(c.beta, cncf[j], 1.0f)) * 1.0001f;
-        if (cid[j] >= 0) m = fminf(m, __fadd_ru(__uint_as_float(y[j]), E));
-    }
-    return m;
+// an upper bound of a group's smallest key (SEED), from the smallest of its
+// values and the tile's error bound (+inf when it may be padding's, 2^40)
+__device__ __forceinline__ float seed_key(float m, float E) {
+    return m < 1099511627776.0f ? __fadd_ru(m, E) : __int_as_float(0x7f800000);
 }
 
 // One group of 32 screened values y of an exact tile, for the 32 rows of a
@@ -517,6 +530,7 @@ struct ScreenArgs {
     const float* cnrm;       // [npad]
     const float* cncf;       // [npad]
     const uint8_t* ctile;    // [npad/256] all-exact flags
+    const float2* ctmax;     // [npad/256] largest norm and squared norm
     Split W;                 // nct of it: candidate tiles screened (SEED: of the sample)
     uint32_t seed_step, seed_mul;   // SEED: tile j of the sample is candidate tile (j * mul mod nct) * step
     const float* thr0;       // [qpad] upper bound of the k-th key, or null
@@ -742,6 +756,7 @@ __global__ void __launch_bounds__(KN_THREADS, 1)
                 for (int i = 0; i < SEED_T * 4; ++i) acc[i] = __int_as_float(0x7f800000);
             bool ok = true;
             bool flag = S.ctile[tile_at(w.ct0)] != 0;    // of the coming tile, loaded a tile ahead
+            float2 top = S.ctmax[tile_at(w.ct0)];
             for (int64_t c = w.ct0; c < w.ct1; ++c, ++it) {
                 const int64_t ct = tile_at(c);
                 const int si = (int)(it % KN_INFO);
@@ -749,7 +764,12 @@ __global__ void __launch_bounds__(KN_THREADS, 1)
                 const int b = (int)(it & 1);
                 const uint32_t pb = (it >> 1) & 1;
                 const bool fast = qtile_exact && flag;
-                if (c + 1 < w.ct1) flag = S.ctile[tile_at(c + 1)] != 0;
+                // at least the error bound of any pair of this row and the tile
+                const float E = rc.exact && flag ? 0.f : fmaf(rc.anrm, top.x, fmaf(rc.beta, top.y, 1.0f)) * 1.0001f;
+                if (c + 1 < w.ct1) {
+                    flag = S.ctile[tile_at(c + 1)] != 0;
+                    top = S.ctmax[tile_at(c + 1)];
+                }
                 if (!__all_sync(0xffffffffu, mbar_wait(TFULL(b), pb, S.status, abort_flag))) {
                     ok = false;
                     break;
@@ -764,6 +784,9 @@ __global__ void __launch_bounds__(KN_THREADS, 1)
                 // the candidates' ids and norms of the tile, needed by few tiles
                 // (they have landed: the wait makes them visible)
                 auto info_ready = [&]() { return mbar_wait(IFULL(si), pi, S.status, abort_flag); };
+                // may a pair with a value from v up enter the list? (E = 0: exact
+                // pairs, of which a tie with the k-th key does not, as above)
+                auto may_enter = [&](float v) { return E == 0.f ? v < r.thr : __fsub_rd(v, E) <= r.thr; };
                 uint32_t u[4][32];
                 float m[4];
                 __syncwarp();
@@ -788,12 +811,7 @@ __global__ void __launch_bounds__(KN_THREADS, 1)
                 if constexpr (MODE == SEED) {
                     float v[4];
 #pragma unroll
-                    for (int g = 0; g < 4; ++g) v[g] = seed_exact(m[g]);
-                    if (!fast && info_ready()) {
-#pragma unroll
-                        for (int g = 0; g < 4; ++g)
-                            v[g] = seed_bounded(rc, u[g], cid + g * 32, cnrm + g * 32, cncf + g * 32);
-                    }
+                    for (int g = 0; g < 4; ++g) v[g] = seed_key(m[g], E);
 #pragma unroll
                     for (int i = 0; i < SEED_T * 4; ++i)
                         if (turn == i / 4) acc[i] = fminf(acc[i], v[i & 3]);
@@ -808,11 +826,16 @@ __global__ void __launch_bounds__(KN_THREADS, 1)
                             if (__any_sync(0xffffffffu, live && m[g] < r.thr))
                                 r = select_exact(r, rc, u[g], cid + g * 32, live, mylist - lane * (KN_SPLIT * KN_KMAX));
                     }
-                } else if (rc.qid >= 0 && info_ready()) {
+                } else if (rc.qid >= 0 && may_enter(fminf(fminf(m[0], m[1]), fminf(m[2], m[3]))) && info_ready()) {
+                    // (few groups hold a pair that the tile's bound cannot rule
+                    // out; with a bound per pair one query beyond BF16-exact
+                    // values among 20,011 made the call 50 ms instead of 4.9: its
+                    // query tile took 15 times as long as the others. 6.4 now.)
 #pragma unroll
                     for (int g = 0; g < 4; ++g)
-                        r = select_bounded(r, rc, u[g], cid + g * 32, cnrm + g * 32, cncf + g * 32,
-                                           ct * KN_N + c0 + g * 32, S.nexact);
+                        if (may_enter(m[g]))
+                            r = select_bounded(r, rc, u[g], cid + g * 32, cnrm + g * 32, cncf + g * 32,
+                                               ct * KN_N + c0 + g * 32, S.nexact);
                 }
                 __syncwarp();
                 if (lane == 0) mbar_arrive(IEMPTY(si));
@@ -945,9 +968,21 @@ __device__ __forceinline__ uint64_t exact_d2(const uint32_t* __restrict__ theta_
     uint64_t s = 0;
     const uint32_t* x = theta_q + (int64_t)a * D;
     const uint32_t* y = theta_c + (int64_t)b * D;
-    for (int d = 0; d < D; ++d) {
-        int64_t t = (int64_t)x[d] - (int64_t)y[d];
+    auto add = [&](uint32_t p, uint32_t q) {
+        const int64_t t = (int64_t)p - (int64_t)q;
         s += (uint64_t)(t * t);
+    };
+    if ((D & 1) == 0) {                              // rows are 8-byte aligned
+        const uint2 *x2 = (const uint2*)x, *y2 = (const uint2*)y;
+#pragma unroll 8
+        for (int d = 0; d < D / 2; ++d) {
+            const uint2 p = __ldg(x2 + d), q = __ldg(y2 + d);
+            add(p.x, q.x);
+            add(p.y, q.y);
+        }
+    } else {
+#pragma unroll 8
+        for (int d = 0; d < D; ++d) add(__ldg(x + d), __ldg(y + d));
     }
     return s;
 }
@@ -1494,7 +1529,8 @@ extern "C" panther_status pantherpp_vectors(panther_ctx* ctx, const panther_inde
         (st = dev_alloc(ctx, (void**)&x.cid, sizeof(int32_t) * x.npad)) ||
         (st = dev_alloc(ctx, (void**)&x.cnrm, sizeof(float) * x.npad)) ||
         (st = dev_alloc(ctx, (void**)&x.cncf, sizeof(float) * x.npad)) ||
-        (st = dev_alloc(ctx, (void**)&x.ctile, x.npad / KN_N))) {
+        (st = dev_alloc(ctx, (void**)&x.ctile, x.npad / KN_N)) ||
+        (st = dev_alloc(ctx, (void**)&x.ctmax, sizeof(float2) * (x.npad / KN_N)))) {
         dev_free(ctx, perm);
         return fail(st);
     }
@@ -1504,7 +1540,8 @@ extern "C" panther_status pantherpp_vectors(panther_ctx* ctx, const panther_inde
                                                                     x.cnrm, x.cncf);
     tile_flags_kernel<<<(unsigned)ceil_div(x.npad / KN_N, 8), 256, 0, s>>>(v->exact, x.cid, x.npad, KN_N, x.ctile,
                                                                              x.npad / KN_N);
-    ctx->launches += 3;
+    tile_max_kernel<<<(unsigned)ceil_div(x.npad / KN_N, 8), 256, 0, s>>>(x.cid, x.cnrm, x.cncf, x.ctmax, x.npad / KN_N);
+    ctx->launches += 4;
     dev_free(ctx, perm);
     dev_free(ctx, flag);
     dev_free(ctx, pos);
@@ -1636,7 +1673,7 @@ static panther_status knn_run(panther_ctx* ctx, const pantherpp_vecs* vq, const 
             cleanup();
             return PANTHER_ECUDA;
         }
-        ScreenArgs S{x.cid, x.cnrm, x.cncf, x.ctile, W, 0, 0, nullptr, x.nexact, Q.qv, Q.qnrm, Q.qexact, qtile,
+        ScreenArgs S{x.cid, x.cnrm, x.cncf, x.ctile, x.ctmax, W, 0, 0, nullptr, x.nexact, Q.qv, Q.qnrm, Q.qexact, qtile,
                      k, lists, sl, sc, nullptr, 0, Q.overflow, ctx->d_status, same, dump, Q.qidx, x.npad};
         auto grid = [&](const Split& w) {
             return (unsigned)(w.G ? w.G : std::min<int64_t>(nqt, ctx->num_sms));
@@ -1703,8 +1740,12 @@ static panther_status knn_run(panther_ctx* ctx, const pantherpp_vecs* vq, const 
     PCK(ctx, cudaStreamSynchronize(s));
     const int64_t kept = (int64_t)hsum[0], over = (int64_t)hsum[1];
     if (over) {
-        // the overflowed queries: exact brute force over all vertices, spread over the GPU
-        const int64_t nparts = std::max<int64_t>(1, std::min<int64_t>(1024, ceil_div(vc->n, 4096)));
+        // the overflowed queries: exact brute force over all vertices, spread
+        // over the GPU. A warp takes 4,096 vertices of a query, 512 when there
+        // are few queries (one query of 1.5M vertices kept 366 warps busy)
+        const int64_t nparts =
+            std::max({int64_t(1), std::min<int64_t>(1024, ceil_div(vc->n, 4096)),
+                      std::min<int64_t>(ceil_div(vc->n, 512), 32768 / over)});
         int32_t* bid = nullptr;
         uint64_t* bd = nullptr;
         auto bfree = [&]() { dev_free(ctx, bid); dev_free(ctx, bd); };
