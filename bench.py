@@ -300,7 +300,7 @@ def run_ours(args, ws, rank, local):
                         "frac": round(gbs / peak, 4), "traffic": _traffic(s, g.n / 5_000_000)}
     dom = max(stages, key=lambda s: stage_ms[s])
     kernel_name = {"sample": "sample_kernel (one launch)", "index": "index stage (radix passes)",
-                   "topk": "top-k stage (lane, group, persistent, hub kernels)",
+                   "topk": "top-k stage (lane, group, team, hub kernels)",
                    "tables": "tables stage (stats and alias kernels)"}[dom]
     traffic = _traffic(dom, g.n / 5_000_000)
     roofline = {"bound": "hbm", "kernel": kernel_name, "achieved": stage_obj[dom]["achieved_gbs"], "peak": peak,
