@@ -514,9 +514,9 @@ extern "C" panther_status panther_build_index(panther_ctx* ctx, const panther_pa
             const int64_t results = p->R * p->L * 4 + 3 * (n + 1) * 8 + n + (int64_t(256) << 20);
             size_t fr = 0, tot = 0;
             if (cudaMemGetInfo(&fr, &tot) == cudaSuccess && (int64_t)fr - results < need) {
-                // memory the pools keep but no one uses goes back first
-                cudaStreamSynchronize(s);
-                trim_pools();
+                // memory the pool keeps but no one uses goes back first
+                cudaMemPool_t pool;
+                if (cudaDeviceGetDefaultMemPool(&pool, ctx->device) == cudaSuccess) cudaMemPoolTrimTo(pool, 0);
                 cudaMemGetInfo(&fr, &tot);
             }
             cudaGetLastError();

@@ -26,7 +26,6 @@ struct panther_ctx {
     int num_sms = 0;
     cudaStream_t stream = nullptr;
     bool own_stream = false;
-    cudaMemPool_t pool = nullptr;     // of every dev_alloc of this context (null: the default pool)
     uint32_t* d_status = nullptr;     // [0] flags, [1..3] detail
     uint32_t* h_status = nullptr;     // pinned mirror
     int* h_counts = nullptr;          // pinned, behind it: tier sizes of a top-k call
@@ -131,7 +130,6 @@ panther_status cuda_err(panther_ctx* ctx, cudaError_t e, const char* what);
 
 panther_status dev_alloc(panther_ctx* ctx, void** p, size_t bytes);
 void dev_free(panther_ctx* ctx, void* p);
-void trim_pools();   // unused memory of every context's pool back to the device
 
 static inline int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }
 
