@@ -1141,14 +1141,17 @@ __device__ __forceinline__ void team_place(const TeamMem& M, const uint32_t (&u)
     __syncwarp();
 }
 
-// How a warp walks P_v, a round at a time. Rows of up to 32 entries: a lane
-// takes four entries, ceil((T+1)/4) lanes a path. With a whole row per lane a
-// query of fewer than 32 paths (most of the warp tier's) leaves lanes idle,
-// and the unrolled code of 8 to 32 entries, their probes and comparisons,
-// overflows the instruction cache: at T = 10 (1,000,003 vertices, R = 2e6) the
-// warp tier took 2.96 ms that way and 1.46 ms this way, at T = 5 the three
-// kernels 1.21 and 1.10 ms. Rows of 64 or 128: the warp takes 32 paths' ids
-// and walks them one by one (team_insert_long).
+// How a warp walks P_v, a round at a time: a lane takes four entries of a row,
+// ceil((T+1)/4) lanes a path. With a whole row per lane a query of fewer than 32
+// paths (most of the warp tier's) leaves lanes idle, and the unrolled code of 8
+// to 32 entries, their probes and comparisons, overflows the instruction cache:
+// at T = 10 (1,000,003 vertices, R = 2e6) the warp tier took 2.96 ms that way
+// and 1.46 ms this way, at T = 5 the three kernels 1.21 and 1.10 ms. Rows of 64
+// or 128 entries (T >= 32) once took 32 paths per warp, walked one by one with a
+// shuffle per earlier entry and lane to find repeats: a query of up to 32 paths
+// kept one warp of its CTA busy. All vertices of 100,000, R = 50,000, top-10:
+// T = 64 32.1 ms that way, 5.2 this way, T = 100 141 and 17 ms; 16 queries at
+// T = 100 (R = 3,000) 1,254 and 156 us.
 template <int STRIDE>
 struct Walk {
     static constexpr int XN = 4;                       // entries held per lane
@@ -1156,21 +1159,14 @@ struct Walk {
     int sub, c4;                                       // this lane's path of the round, its first entry
     __device__ __forceinline__ Walk(const PathsRef& P) {
         const int lane = threadIdx.x & 31;
-        if (STRIDE <= 32) {
-            const int lanes = (P.L + 3) >> 2;
-            ppr = 32 / lanes;
-            sub = lane / lanes;
-            c4 = 4 * (lane - sub * lanes);
-            if (sub >= ppr) sub = 1 << 30;             // spare lanes: past any list
-        } else {
-            ppr = 32;
-            sub = lane;
-            c4 = 0;
-        }
+        const int lanes = (P.L + 3) >> 2;              // at most 32 (T <= 127)
+        ppr = 32 / lanes;
+        sub = lane / lanes;
+        c4 = 4 * (lane - sub * lanes);
+        if (sub >= ppr) sub = 1 << 30;                 // spare lanes: past any list
     }
     // this lane's entries of path r (-1 everywhere when r is no path)
     __device__ __forceinline__ void load(const PathsRef& P, uint32_t r, int32_t (&x)[XN]) const {
-        if constexpr (STRIDE > 32) return;
         const bool act = r < (uint64_t)P.R;
         const int4* src = (const int4*)(P.rows + (uint64_t)(act ? r : 0u) * STRIDE + c4);
         const int4 q = (act && c4 < P.L) ? __ldg(src) : make_int4(-1, -1, -1, -1);
@@ -1204,42 +1200,6 @@ struct Walk {
         team_place<XN>(M, u, ok);
     }
 };
-
-// rows of 64 or 128 entries: the warp takes its lanes' paths one at a time,
-// lane l holding entries l, l+32, ... (as insert_paths_warp)
-template <int STRIDE>
-__device__ __forceinline__ void team_insert_long(const PathsRef& P, uint32_t r, int32_t v, const TeamMem& M,
-                                                     bool& ok) {
-    constexpr int NR = STRIDE / 32;
-    const unsigned lane = threadIdx.x & 31, lt = (1u << lane) - 1u;
-    unsigned pend = __ballot_sync(0xffffffffu, r < (uint64_t)P.R);
-    while (pend) {                                     // warp-uniform
-        const int src = __ffs(pend) - 1;
-        pend &= pend - 1;
-        const uint32_t rr = __shfl_sync(0xffffffffu, r, src);
-        const int32_t* row = P.rows + (uint64_t)rr * STRIDE;
-        int32_t y[NR];
-#pragma unroll
-        for (int m = 0; m < NR; ++m) y[m] = __ldg(row + m * 32 + lane);
-#pragma unroll
-        for (int m = 0; m < NR; ++m) {
-            if (m * 32 >= P.L) break;                  // warp-uniform: the rest is padding
-            bool take = m * 32 + (int)lane < P.L && y[m] >= 0 && y[m] != v;
-            take &= (__match_any_sync(0xffffffffu, y[m]) & lt) == 0;
-#pragma unroll
-            for (int mm = 0; mm < m; ++mm)
-#pragma unroll 8
-                for (int sl = 0; sl < 32; ++sl) take &= __shfl_sync(0xffffffffu, y[mm], sl) != y[m];
-            if (take) {
-                const uint32_t u = (uint32_t)y[m], s = hslot(u, M.ns);
-                const uint32_t p = atomicCAS(&M.key[s], EMPTYK, u);
-                if (p == u) team_bump(M, s);
-                else if (p != EMPTYK) team_probe(M, u, s, ok);
-            }
-            __syncwarp();
-        }
-    }
-}
 
 __device__ __forceinline__ uint64_t score_of(uint32_t id, uint32_t cnt) {
     return ((uint64_t)cnt << 32) | (uint64_t)(0xffffffffu - id);
@@ -1604,15 +1564,10 @@ __device__ __forceinline__ void cta_query(const PathsRef& P, int32_t v, int64_t 
     for (int64_t base = first; base < b; base += step) {
         const int64_t e2 = base + 2 * step + W.sub;
         const uint32_t r2 = e2 < b ? P.pid[e2] : NO_PATH;
-        if constexpr (STRIDE > 32) {
-            team_insert_long<STRIDE>(P, r0, v, M, ok);
-            r0 = r1;
-        } else {
-            W.load(P, r1, y);
-            W.count(P, x, v, M, ok);
+        W.load(P, r1, y);
+        W.count(P, x, v, M, ok);
 #pragma unroll
-            for (int j = 0; j < Walk<STRIDE>::XN; ++j) x[j] = y[j];
-        }
+        for (int j = 0; j < Walk<STRIDE>::XN; ++j) x[j] = y[j];
         r1 = r2;
     }
     team_finish<true>(P, b - a, M, ok, o, qi, status);
@@ -1697,15 +1652,10 @@ __global__ void __launch_bounds__(128) warp_tier_kernel(TeamArgs A) {
             bool ok = true;
             for (int64_t i = 0; i < np; i += W.ppr) {
                 const uint32_t r2 = next_ids();
-                if constexpr (STRIDE > 32) {
-                    team_insert_long<STRIDE>(A.P, r0, v, M, ok);
-                    r0 = r1;
-                } else {
-                    W.load(A.P, r1, y);
-                    W.count(A.P, x, v, M, ok);
+                W.load(A.P, r1, y);
+                W.count(A.P, x, v, M, ok);
 #pragma unroll
-                    for (int c = 0; c < Walk<STRIDE>::XN; ++c) x[c] = y[c];
-                }
+                for (int c = 0; c < Walk<STRIDE>::XN; ++c) x[c] = y[c];
                 r1 = r2;
             }
             team_finish<false>(A.P, np, M, ok, A.o, qi, A.status);
