@@ -420,7 +420,14 @@ __device__ __forceinline__ float seed_key(float m, float E) {
 // Mostly one row of the warp has one such candidate, so the warp inserts it
 // together, lane l holding entry l of the row's list: an insertion by the
 // row's own lane is a chain of up to k loads and stores the tile's other warps
-// soon wait for, and a call there saves the group's registers.
+// soon wait for, and a call there saves the group's registers. While lists
+// fill, most rows have one: with LANES and more than 1 + k/4 such rows (the chain
+// costs about 70 cycles a link, the warp's insertion about as much as three, and
+// half-full lists have short chains) every lane inserts its own. That costs
+// registers (72 bytes spilled
+// instead of 36; 100,000 queries against as many vertices 8.4 instead of 6.4 ms),
+// so only the form for few candidate tiles has it (FILL below).
+template <bool LANES>
 __device__ __forceinline__ Row select_exact(Row r, const RowConst& c, const uint32_t (&y)[32], const int32_t* cid,
                                             bool live, float2* warp_lists) {
     const int lane = threadIdx.x & 31;
@@ -440,6 +447,28 @@ __device__ __forceinline__ Row select_exact(Row r, const RowConst& c, const uint
         const int id = at >= 0 ? cid[at] : -1;
         last = at >= 0 ? at : 32;
         rows &= __ballot_sync(0xffffffffu, id >= 0 && id != c.self);
+        if (LANES && __popc(rows) > 1 + c.k / 4) {
+            if ((rows >> lane) & 1u) {
+                float2* list = warp_lists + lane * (KN_SPLIT * KN_KMAX);
+                int i = r.n < c.k ? r.n : c.k - 1;   // the entries worse than it move up one
+                r.n = i + 1;
+                float2 worst = make_float2(key, __int_as_float(id));
+#pragma unroll 1
+                for (bool top = true; i > 0; --i, top = false) {
+                    const float2 e = list[i - 1];
+                    if (e.x < key || (e.x == key && __float_as_int(e.y) < id)) break;
+                    list[i] = e;
+                    worst = top ? e : worst;
+                }
+                list[i] = make_float2(key, __int_as_float(id));
+                if (r.n == c.k) {
+                    r.thr = worst.x;
+                    r.thr_id = __float_as_int(worst.y);
+                }
+            }
+            __syncwarp();
+            continue;
+        }
         while (rows) {                               // warp-uniform
             const int l = __ffs(rows) - 1;
             rows &= rows - 1;
@@ -583,7 +612,11 @@ struct Smem {
 // (k+1)-th smallest over the query bounds its k-th key (one of them may be the
 // query itself).
 constexpr int SEED_T = 5;
-enum { SCREEN = 0, DUMP_FORM = 1, SEED = 2 };
+// FILL is the SCREEN form below 16 candidate tiles, where there is no sample and
+// filling the lists is the work: 1,000 queries against 1,000 vertices, k = 10,
+// 874 us with warp insertions alone, 310 with the lanes' own.
+enum { SCREEN = 0, DUMP_FORM = 1, SEED = 2, FILL = 3 };
+constexpr int64_t FILL_TILES = 16;
 
 template <int MODE, int KB>
 __global__ void __launch_bounds__(KN_THREADS, 1)
@@ -824,7 +857,7 @@ __global__ void __launch_bounds__(KN_THREADS, 1)
 #pragma unroll
                         for (int g = 0; g < 4; ++g)
                             if (__any_sync(0xffffffffu, live && m[g] < r.thr))
-                                r = select_exact(r, rc, u[g], cid + g * 32, live, mylist - lane * (KN_SPLIT * KN_KMAX));
+                                r = select_exact<MODE == FILL>(r, rc, u[g], cid + g * 32, live, mylist - lane * (KN_SPLIT * KN_KMAX));
                     }
                 } else if (rc.qid >= 0 && may_enter(fminf(fminf(m[0], m[1]), fminf(m[2], m[3]))) && info_ready()) {
                     // (few groups hold a pair that the tile's bound cannot rule
@@ -1556,13 +1589,13 @@ extern "C" panther_status pantherpp_vectors(panther_ctx* ctx, const panther_inde
 }
 
 // The BF16 screen's work in equal runs, one per CTA, of at least KN_MIN_RUN
-// candidate tiles. From 16 query tiles per SM on, whole tiles per CTA: the last
+// candidate tiles or a whole query tile. From 16 query tiles per SM on, whole tiles per CTA: the last
 // wave then costs at most 6%, and every segment more of a tile costs lists and
 // a shortlist of 2 KB per query.
 static Split knn_split(int64_t nqt, int64_t nct, int num_sms) {
     Split W{nqt, nct, 0, 1};
     if (nqt >= 16 * (int64_t)num_sms) return W;
-    W.G = std::max<int64_t>(1, std::min<int64_t>(num_sms, nqt * nct / KN_MIN_RUN));
+    W.G = std::min<int64_t>(num_sms, std::max(nqt, nqt * nct / KN_MIN_RUN));
     for (int64_t t = 0; t < nqt; ++t) W.nseg = std::max(W.nseg, W.segments(t));
     return W;
 }
@@ -1584,10 +1617,18 @@ static Split knn_ranges(int64_t nqt, int64_t nct, int num_sms) {
     return W;
 }
 
-// Candidate tiles of the sample that bounds the k-th keys (0: none): a 32nd,
-// a 16th of fewer than 2,048, none below 128 tiles (32,768 candidates), where
-// the screen itself is as short.
-static int64_t seed_tiles(int64_t nct) { return nct < 128 ? 0 : nct / (nct < 2048 ? 16 : 32); }
+// Candidate tiles of the sample that bounds the k-th keys (0: none): a 32nd of
+// the candidate tiles, a 16th of fewer than 2,048, an eighth of fewer than 128
+// but at least five (eight minima a tile; a bound for k = 32 needs 33). Below 16
+// tiles the sample would be as long as the screen. (32,000 queries against as
+// many vertices, 125 tiles, k = 10: 5.3 ms without a sample, 1.4 with one.
+// A 16th instead of an eighth leaves k = 32 without a bound at 16,000 vertices,
+// 4.8 ms instead of 2.0.)
+static int64_t seed_tiles(int64_t nct) {
+    if (nct < FILL_TILES) return 0;
+    if (nct < 128) return std::max<int64_t>(5, nct / 8);
+    return nct / (nct < 2048 ? 16 : 32);
+}
 
 template <int MODE, int KB>
 static panther_status launch_screen(panther_ctx* ctx, unsigned grid, const CUtensorMap& tmA, const CUtensorMap& tmB,
@@ -1697,9 +1738,14 @@ static panther_status knn_run(panther_ctx* ctx, const pantherpp_vecs* vq, const 
                 ctx->launches++;
                 S.thr0 = thr0;
             }
-            st = kb == 1 ? launch_screen<SCREEN, 1>(ctx, grid(W), tmA, tmB, S)
-               : kb == 2 ? launch_screen<SCREEN, 2>(ctx, grid(W), tmA, tmB, S)
-                         : launch_screen<SCREEN, 3>(ctx, grid(W), tmA, tmB, S);
+            if (nct < FILL_TILES)
+                st = kb == 1 ? launch_screen<FILL, 1>(ctx, grid(W), tmA, tmB, S)
+                   : kb == 2 ? launch_screen<FILL, 2>(ctx, grid(W), tmA, tmB, S)
+                             : launch_screen<FILL, 3>(ctx, grid(W), tmA, tmB, S);
+            else
+                st = kb == 1 ? launch_screen<SCREEN, 1>(ctx, grid(W), tmA, tmB, S)
+                   : kb == 2 ? launch_screen<SCREEN, 2>(ctx, grid(W), tmA, tmB, S)
+                             : launch_screen<SCREEN, 3>(ctx, grid(W), tmA, tmB, S);
             if (st) { cleanup(); return st; }
         }
     } else {
