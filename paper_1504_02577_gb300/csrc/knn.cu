@@ -859,8 +859,9 @@ __global__ void __launch_bounds__(KN_THREADS, 1)
                             if (__any_sync(0xffffffffu, live && m[g] < r.thr))
                                 r = select_exact<MODE == FILL>(r, rc, u[g], cid + g * 32, live, mylist - lane * (KN_SPLIT * KN_KMAX));
                     }
-                } else if (rc.qid >= 0 && may_enter(fminf(fminf(m[0], m[1]), fminf(m[2], m[3]))) && info_ready()) {
-                    // (few groups hold a pair that the tile's bound cannot rule
+                } else if (rc.qid >= 0 && r.scount <= KN_SCAP &&
+                           may_enter(fminf(fminf(m[0], m[1]), fminf(m[2], m[3]))) && info_ready()) {
+                    // (a row whose shortlist overflowed is brute_force's; few groups hold a pair that the tile's bound cannot rule
                     // out; with a bound per pair one query beyond BF16-exact
                     // values among 20,011 made the call 50 ms instead of 4.9: its
                     // query tile took 15 times as long as the others. 6.4 now.)
@@ -1252,8 +1253,8 @@ __global__ void __launch_bounds__(256) chunk_merge_warp_kernel(const int32_t* __
     }
 }
 
-// Exact brute force for the (rare) queries whose shortlist overflowed: the
-// vertex range of each such query is cut into nparts pieces, one warp each.
+// Exact brute force for the queries whose shortlist overflowed, few of them
+// (below BRUTE_TILE): the vertex range of each is cut into nparts pieces, one warp each.
 // A warp keeps its k best (d2, id) sorted across its lanes (lane l holds rank
 // l); a batch of 32 candidates costs one compare and a ballot unless one of
 // them beats the k-th entry. The nparts lists go through chunk_merge_kernel.
@@ -1310,6 +1311,120 @@ __global__ void __launch_bounds__(256) brute_warp_kernel(const uint32_t* __restr
         part_id[gw * k + lane] = li == 0x7fffffff ? -1 : li;
         part_d2[gw * k + lane] = ld;
     }
+}
+
+// The same for many queries: a thread per query, its row in registers, the
+// candidates of range blockIdx.y through shared memory, four dot products at a
+// time. Entries are non-negative, so d2 <= |a|^2 + |b|^2; while that is below
+// 2^32 the distance is exact in 32-bit arithmetic modulo 2^32 whatever the
+// entries. Other pairs are computed in 64 bits unless the norms alone,
+// (|a| - |b|)^2 <= d2, keep them from the list. A network whose counts are
+// mostly beyond BF16-exact values sends most of its queries here (all of 20,000,
+// D = 57, k = 10, R = 4e7, whole call: 31.5 ms with a warp per query and range,
+// 6.3 with this); the warp form reads every candidate row once per query.
+// A CTA costs the same for 1 and 128 queries, and its lists more the longer they
+// are: with k = 10 about what the warp form takes for 10 to 20 queries at
+// n = 200,000 (D = 128, 30 queries: 1.5 ms against 0.4) and for 60 to 130 at
+// n = 20,000, with k = 32 for 30 to 50 and for more than 160.
+constexpr int BT_T = 128, BT_C = 32;
+constexpr int64_t BRUTE_TILE = int64_t(1) << 18;      // queries x candidates / k from which it is taken
+template <int KK>
+struct BruteSmem {
+    uint32_t row[BT_C][KK];
+    uint64_t n2[BT_C];
+    float nrm[BT_C];
+    int id[BT_C];                      // -1: none
+    uint64_t ld[KN_KMAX][BT_T];        // the queries' lists, entry by entry
+    int li[KN_KMAX][BT_T];
+};
+
+template <int KK>
+__global__ void __launch_bounds__(BT_T) brute_tile_kernel(const uint32_t* __restrict__ theta_q,
+                                                          const uint64_t* __restrict__ norm2_q,
+                                                          const float* __restrict__ nrm_q,
+                                                          const uint32_t* __restrict__ theta_c,
+                                                          const uint64_t* __restrict__ norm2_c,
+                                                          const float* __restrict__ nrm_c, bool exclude_self, int D,
+                                                          int64_t n, const int32_t* __restrict__ qv,
+                                                          const int32_t* __restrict__ ovslots, int64_t nov, int k,
+                                                          int32_t* __restrict__ part_id,
+                                                          uint64_t* __restrict__ part_d2) {
+    extern __shared__ __align__(16) uint8_t bsm[];
+    BruteSmem<KK>& S = *(BruteSmem<KK>*)bsm;
+    const int t = threadIdx.x;
+    const int64_t q = (int64_t)blockIdx.x * BT_T + t, nparts = gridDim.y, part = blockIdx.y;
+    const int64_t u0 = part * n / nparts, u1 = (part + 1) * n / nparts;
+    const bool live = q < nov;
+    const int32_t v = live ? qv[ovslots[q]] : -1;
+    uint32_t a[KK];
+#pragma unroll
+    for (int d = 0; d < KK; ++d) a[d] = live && d < D ? theta_q[(int64_t)v * D + d] : 0u;
+    const uint64_t na2 = live ? norm2_q[v] : 0;
+    const float na = live ? nrm_q[v] : 0.f;
+    int held = 0;
+    uint64_t thr = ~0ull;              // the k-th entry (held == k)
+    int thr_id = 0x7fffffff;
+    for (int64_t c0 = u0; c0 < u1; c0 += BT_C) {
+        __syncthreads();
+        const int cnt = (int)(u1 - c0 < BT_C ? u1 - c0 : BT_C);
+        for (int i = t; i < BT_C * KK; i += BT_T) {
+            const int c = i / KK, d = i % KK;
+            S.row[c][d] = c < cnt && d < D ? theta_c[(c0 + c) * D + d] : 0u;
+        }
+        if (t < BT_C) {
+            S.id[t] = t < cnt ? (int)(c0 + t) : -1;
+            S.n2[t] = t < cnt ? norm2_c[c0 + t] : 0;
+            S.nrm[t] = t < cnt ? nrm_c[c0 + t] : 0.f;
+        }
+        __syncthreads();
+        if (!live) continue;
+        for (int c = 0; c < BT_C; c += 4) {
+            uint32_t dot[4] = {0, 0, 0, 0};
+#pragma unroll
+            for (int d = 0; d < KK; d += 4)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const uint4 b = *(const uint4*)&S.row[c + j][d];
+                    dot[j] += a[d] * b.x + a[d + 1] * b.y + a[d + 2] * b.z + a[d + 3] * b.w;
+                }
+#pragma unroll 1
+            for (int j = 0; j < 4; ++j) {
+                const int u = S.id[c + j];
+                if (u < 0 || (exclude_self && u == v)) continue;
+                const uint64_t nb2 = S.n2[c + j], sum = na2 + nb2;
+                const uint32_t dj = j == 0 ? dot[0] : j == 1 ? dot[1] : j == 2 ? dot[2] : dot[3];
+                uint64_t d2;
+                if ((na2 | nb2 | sum) >> 32) {       // (sum alone may wrap)
+                    const float gap = fabsf(na - S.nrm[c + j]) - 1e-6f * (na + S.nrm[c + j]);
+                    if (gap > 0.f && __fmul_rd(gap, gap) > __ull2float_ru(thr)) continue;
+                    d2 = exact_d2(theta_q, theta_c, D, v, u);
+                } else {
+                    d2 = (uint32_t)sum - 2u * dj;
+                }
+                if (!pair_less(d2, u, thr, thr_id)) continue;
+                int i = held < k ? held : k - 1;
+                held = i + 1;
+                for (; i > 0; --i) {
+                    const uint64_t ed = S.ld[i - 1][t];
+                    const int ei = S.li[i - 1][t];
+                    if (pair_less(ed, ei, d2, u)) break;
+                    S.ld[i][t] = ed;
+                    S.li[i][t] = ei;
+                }
+                S.ld[i][t] = d2;
+                S.li[i][t] = u;
+                if (held == k) {
+                    thr = S.ld[k - 1][t];
+                    thr_id = S.li[k - 1][t];
+                }
+            }
+        }
+    }
+    if (live)
+        for (int i = 0; i < k; ++i) {
+            part_id[(q * nparts + part) * k + i] = i < held ? S.li[i][t] : -1;
+            part_d2[(q * nparts + part) * k + i] = i < held ? S.ld[i][t] : ~0ull;
+        }
 }
 
 // query slots: exact queries first (stable), padded to a multiple of 128.
@@ -1640,6 +1755,19 @@ static panther_status launch_screen(panther_ctx* ctx, unsigned grid, const CUten
     return PANTHER_OK;
 }
 
+template <int KK>
+static panther_status launch_brute(panther_ctx* ctx, const pantherpp_vecs* vq, const pantherpp_vecs* vc, bool same,
+                                   const int32_t* qv, const int32_t* ovslots, int64_t over, int64_t nparts, int k,
+                                   int32_t* part_id, uint64_t* part_d2) {
+    constexpr int smem = (int)sizeof(BruteSmem<KK>);
+    PCK(ctx, cudaFuncSetAttribute(brute_tile_kernel<KK>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    brute_tile_kernel<KK><<<dim3((unsigned)ceil_div(over, BT_T), (unsigned)nparts), BT_T, smem, ctx->stream>>>(
+        vq->theta, vq->norm2, vq->nrm, vc->theta, vc->norm2, vc->nrm, same, vq->D, vc->n, qv, ovslots, over, k, part_id,
+        part_d2);
+    PLAUNCH(ctx);
+    return PANTHER_OK;
+}
+
 // queries are vertices of vq, candidates every vertex of vc; `same` excludes
 // the candidate with the query's id (one graph: the query itself)
 static panther_status knn_run(panther_ctx* ctx, const pantherpp_vecs* vq, const pantherpp_vecs* vc, bool same,
@@ -1788,10 +1916,13 @@ static panther_status knn_run(panther_ctx* ctx, const pantherpp_vecs* vq, const 
     if (over) {
         // the overflowed queries: exact brute force over all vertices, spread
         // over the GPU. A warp takes 4,096 vertices of a query, 512 when there
-        // are few queries (one query of 1.5M vertices kept 366 warps busy)
+        // are few queries (one query of 1.5M vertices kept 366 warps busy); a
+        // CTA of the many-query form 256 or more, three CTAs an SM
+        const bool tile = over >= 8 && over * vc->n >= BRUTE_TILE * k;
         const int64_t nparts =
-            std::max({int64_t(1), std::min<int64_t>(1024, ceil_div(vc->n, 4096)),
-                      std::min<int64_t>(ceil_div(vc->n, 512), 32768 / over)});
+            tile ? std::max<int64_t>(1, std::min<int64_t>(ceil_div(vc->n, 256), 3 * ctx->num_sms / ceil_div(over, BT_T)))
+                 : std::max({int64_t(1), std::min<int64_t>(1024, ceil_div(vc->n, 4096)),
+                             std::min<int64_t>(ceil_div(vc->n, 512), 32768 / over)});
         int32_t* bid = nullptr;
         uint64_t* bd = nullptr;
         auto bfree = [&]() { dev_free(ctx, bid); dev_free(ctx, bd); };
@@ -1801,11 +1932,22 @@ static panther_status knn_run(panther_ctx* ctx, const pantherpp_vecs* vq, const 
             cleanup();
             return st;
         }
-        brute_warp_kernel<<<(unsigned)ceil_div(over * nparts * 32, 256), 256, 0, s>>>(
-            vq->theta, vc->theta, same, v->D, vc->n, Q.qv, ovs, over, nparts, k, bid, bd);
+        if (tile) {
+            st = v->D <= 64 ? launch_brute<64>(ctx, vq, vc, same, Q.qv, ovs, over, nparts, k, bid, bd)
+                            : launch_brute<128>(ctx, vq, vc, same, Q.qv, ovs, over, nparts, k, bid, bd);
+        } else {
+            brute_warp_kernel<<<(unsigned)ceil_div(over * nparts * 32, 256), 256, 0, s>>>(
+                vq->theta, vc->theta, same, v->D, vc->n, Q.qv, ovs, over, nparts, k, bid, bd);
+            ctx->launches++;
+        }
+        if (st) {
+            bfree();
+            cleanup();
+            return st;
+        }
         chunk_merge_kernel<<<(unsigned)std::min<int64_t>(over, 8 * ctx->num_sms), 256, 0, s>>>(
             Q.qv, Q.qidx, Q.overflow, ovs, over, W, nparts, k, bid, bd, ids, d2);
-        ctx->launches += 2;
+        ctx->launches++;
         const cudaError_t ce = cudaGetLastError();
         bfree();
         if (ce) {
