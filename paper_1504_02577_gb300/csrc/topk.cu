@@ -1474,35 +1474,33 @@ __device__ __forceinline__ void team_select(const TeamMem& M, const OutRef& o, i
             __syncwarp();
             team_find_bin<CTA, true>(M, k);
             const uint32_t b = M.ctr[4];
-            const unsigned above = M.ctr[5], upto = M.ctr[6];   // above bin b (fewer than k), and with it
-            if (b >= 128u && upto > items) {
-                // a coded bin of large counts holds more than the buffer: one rank at a time
-                if (!CTA || threadIdx.x < 32) {
-                    const unsigned lane = threadIdx.x & 31;
-                    uint64_t last = ~0ull;
-                    for (unsigned rk = 0; rk < k; ++rk) {
-                        uint64_t best = 0;
-                        for (unsigned s = lane; s < M.ns; s += 32) {
-                            const uint32_t u = M.key[s], x = M.ext[s];
-                            const uint64_t sc = (u != EMPTYK && x) ? score_of(u, x + 1u) : 0ull;
-                            best = (sc < last && sc > best) ? sc : best;
-                        }
-#pragma unroll
-                        for (int d = 16; d; d >>= 1) best = umax64(best, __shfl_xor_sync(0xffffffffu, best, d));
-                        if (lane == 0) put_rank(o, qi, rk, 0xffffffffu - (uint32_t)best, (uint32_t)(best >> 32));
-                        last = best;
-                    }
-                }
-                done = k;                              // more than k candidates here
-                break;
+            unsigned above = M.ctr[5], upto = M.ctr[6];          // above bin b (fewer than k), and with it
+            uint32_t lo = (uint32_t)code_floor(b), hi = (uint32_t)code_floor(b + 1) - 1u;   // the bin's counts
+            // A coded bin of large counts (from 128 on) may hold more than the
+            // buffer: 256 equal steps of its range, until they fit or one count
+            // is left. (5,000 vertices, R = 8e7, 100 queries, k = 128: 1,575 us
+            // with ranks found one by one, by one warp, 486 this way.)
+#pragma unroll 1
+            while (lo < hi && upto > items) {
+                const unsigned shift = hi - lo < 256u ? 0u : 24u - (unsigned)__clz((int)(hi - lo));
+                team_clear_hist<CTA>(M);
+                each_rep([&](uint32_t, uint32_t c) {
+                    if (c >= lo && c <= hi) atomicAdd((uint32_t*)M.buf + ((c - lo) >> shift), 1u);
+                });
+                __syncwarp();
+                team_find_bin<CTA, true>(M, k - above);
+                upto = above + M.ctr[6];
+                above += M.ctr[5];
+                lo += M.ctr[4] << shift;
+                hi = min(hi, lo + (1u << shift) - 1u);
             }
-            // all of bin b with those above it, or (many share the count b) only those above
-            const bool split = b < 128u && upto > 64u;
-            const uint32_t from = split ? b + 1 : b;
-            if (split) level = b;
+            // all from lo on with those above it, or (many share the count lo) only those above
+            const bool split = lo == hi && upto > 64u;
+            const uint32_t from = split ? lo + 1u : lo;
+            if (split) level = lo;
             team_clear_hist<CTA>(M);
             each_rep([&](uint32_t id, uint32_t c) {
-                if (path_code(c) >= from) {
+                if (c >= from) {
                     const unsigned at = atomicAdd(&M.ctr[2], 1u);
                     if (at < items) put_score(M, at, id, c, idbits);
                 }
