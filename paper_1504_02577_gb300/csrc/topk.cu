@@ -1574,15 +1574,19 @@ __device__ __forceinline__ void cta_query(const PathsRef& P, int32_t v, int64_t 
 // What a query needs: 1 a team with a table of up to `ccap` candidates, 7 the
 // pass with the largest tables, 2 the hub tier, 0 nothing (no candidates),
 // -1 not a vertex
-__device__ __forceinline__ int query_tier(const PathsRef& P, int64_t v, int64_t ccap, int64_t ccap_big, int64_t* a,
-                                          int64_t* b) {
+struct SmallBounds {
+    int64_t ccap, ccap_big;      // candidates of a team, of the largest tables
+    int64_t np, np_big;          // paths of them
+    bool share;                  // long queries to the hub tier, whose CTAs share them (q < 32)
+};
+__device__ __forceinline__ int query_tier(const PathsRef& P, int64_t v, const SmallBounds& B, int64_t* a, int64_t* b) {
     if (v < 0 || v >= P.n) return -1;
     *a = P.off[v];
     *b = P.off[v + 1];
     const int64_t np = *b - *a, cap = min(np * (P.L - 1), P.n - 1);
     if (cap <= 0) return 0;
-    if (np > CTA_MAX_NP || cap > ccap_big) return 2;
-    return cap <= ccap && np <= MID_MAX_NP ? 1 : 7;
+    if (np > B.np_big || cap > B.ccap_big) return 2;
+    return cap <= B.ccap && np <= B.np ? 1 : 7;
 }
 
 struct TeamArgs {
@@ -1753,15 +1757,23 @@ __global__ void __launch_bounds__(1024, 1) single_kernel(PathsRef P, const int32
 // counts as in Tiers: [1] answered here, [2] hubs, [10] largest tables.
 template <int STRIDE>
 __global__ void __launch_bounds__(512) small_batch_kernel(PathsRef P, const int32_t* __restrict__ queries, int64_t q,
-                                                          int64_t ccap, int64_t ccap_big, uint32_t slots,
+                                                          SmallBounds B, uint32_t slots,
                                                           int32_t* __restrict__ hubs, int32_t* __restrict__ bigs,
                                                           int* __restrict__ counts, OutRef o, uint32_t* status) {
     extern __shared__ __align__(16) unsigned char tsm[];
     const TeamMem M = team_mem<true>(tsm, slots);
+    if (B.share) {                                     // by the longest query: those near it go the same way
+        const int lane = threadIdx.x & 31;
+        const int64_t v = lane < q ? (queries ? (int64_t)queries[lane] : lane) : -1;
+        const int64_t np = v >= 0 && v < P.n ? P.off[v + 1] - P.off[v] : 0;
+        const uint32_t top = __reduce_max_sync(0xffffffffu, (uint32_t)min(np, (int64_t)1 << 30));
+        const int64_t cut = 15'000'000 / ((64 - q) * P.L);
+        if (top > cut) B.np_big = min(min(B.np_big, cut), (int64_t)top / 8);
+    }
     for (int64_t i = blockIdx.x; i < q; i += gridDim.x) {
         const int64_t v = queries ? (int64_t)queries[i] : i;
         int64_t a = 0, b = 0;
-        const int tier = query_tier(P, v, ccap, ccap_big, &a, &b);      // the same for every thread
+        const int tier = query_tier(P, v, B, &a, &b);      // the same for every thread
         if (tier == 1) {
             if (threadIdx.x == 0) atomicAdd(&counts[1], 1);
             cta_query<STRIDE>(P, (int32_t)v, i, a, b, M, slots, o, status);
@@ -2123,17 +2135,35 @@ static panther_status set_smem_attr(panther_ctx* ctx) {
 // R = 2e6, k = 10: 97 / 134, 282 / 330, 479 / 479, 1,192 / 1,057 us.
 constexpr int64_t SMALL_Q = 16384, SMALL_Q_WIDE = 1024;
 
+// Bounds of that form's teams. While the batch leaves SMs idle, its longest
+// query is the call's time: a CTA of 128 threads counts about 0.4 entries of a
+// path a nanosecond, one of 1,024 up to 1.8 (2,000 vertices, R = 1e6, T = 20, 16
+// queries of 220,000 entries, k = 10: 586 and 258 us). The hub tier, whose CTAs
+// share a query, costs 150 us first; for k > 64, where it counts in device
+// tables, it then takes about 100 entries a nanosecond, so that it is the faster
+// one from some 15e6 / (64 - q) entries on (4 queries of 1.8M entries: 1,370 us in
+// CTAs, 353 there), but not on networks of a few hundred vertices, whose
+// device counters serialise.
+static SmallBounds small_bounds(const panther_ctx* ctx, const PathsRef& P, int64_t q, int k, int64_t ccap,
+                                int64_t ccap_big) {
+    SmallBounds B{ccap, ccap_big, MID_MAX_NP, CTA_MAX_NP, k > KMAX && q < 32 && P.n >= 512};
+    if (q <= 4 * (int64_t)ctx->num_sms) B.np = std::min<int64_t>(MID_MAX_NP, (1 << 15) / P.L);
+    return B;
+}
+
 template <int STRIDE>
 static void launch_small(panther_ctx* ctx, const PathsRef& P, const int32_t* queries, int64_t q, const Tiers& tiers,
-                         const OutRef& o, const TopkShape& sh, int64_t ccap, int64_t ccap_big) {
+                         const OutRef& o, const TopkShape& sh, const SmallBounds& B) {
     cudaStream_t s = ctx->stream;
     int* c = tiers.count;
     const unsigned blocks = (unsigned)std::min<int64_t>(q, (int64_t)ctx->num_sms * sh.blocks_per_sm);
     const int threads = std::min(sh.threads, 512);
     small_batch_kernel<STRIDE><<<blocks, threads, team_bytes(true, sh.cta_slots), s>>>(
-        P, queries, q, ccap, ccap_big, sh.cta_slots, tiers.list[2], tiers.list[7], c, o, ctx->d_status);
+        P, queries, q, B, sh.cta_slots, tiers.list[2], tiers.list[7], c, o, ctx->d_status);
     const TeamArgs big{P, queries, tiers.list[7], c + 10, c + 13, o, BIG_SLOTS, ctx->d_status};
-    cta_tier_kernel<STRIDE, 512><<<(unsigned)std::min<int64_t>(q, ctx->num_sms), BIG_T, BIG_SMEM, s>>>(big);
+    const unsigned bigs = (unsigned)std::min<int64_t>(q, ctx->num_sms);
+    if (q <= 4 * (int64_t)ctx->num_sms) cta_tier_kernel<STRIDE, 1024><<<bigs, 1024, BIG_SMEM, s>>>(big);
+    else cta_tier_kernel<STRIDE, 512><<<bigs, BIG_T, BIG_SMEM, s>>>(big);
     ctx->launches += 2;
 }
 
@@ -2458,11 +2488,12 @@ panther_status topk_run(panther_ctx* ctx, const panther_index* ix, const panther
     const bool lane_ok = p->stride == 8 && k <= LANE_K;
     PCK(ctx, cudaMemsetAsync(counts, 0, sizeof(int) * 16, s));
     if (q <= (wide_k ? SMALL_Q_WIDE : SMALL_Q)) {
-        if (p->stride == 8) launch_small<8>(ctx, P, queries, q, tiers, o, sh, ccap, ccap_big);
-        else if (p->stride == 16) launch_small<16>(ctx, P, queries, q, tiers, o, sh, ccap, ccap_big);
-        else if (p->stride == 32) launch_small<32>(ctx, P, queries, q, tiers, o, sh, ccap, ccap_big);
-        else if (p->stride == 64) launch_small<64>(ctx, P, queries, q, tiers, o, sh, ccap, ccap_big);
-        else launch_small<128>(ctx, P, queries, q, tiers, o, sh, ccap, ccap_big);
+        const SmallBounds sb = small_bounds(ctx, P, q, k, ccap, ccap_big);
+        if (p->stride == 8) launch_small<8>(ctx, P, queries, q, tiers, o, sh, sb);
+        else if (p->stride == 16) launch_small<16>(ctx, P, queries, q, tiers, o, sh, sb);
+        else if (p->stride == 32) launch_small<32>(ctx, P, queries, q, tiers, o, sh, sb);
+        else if (p->stride == 64) launch_small<64>(ctx, P, queries, q, tiers, o, sh, sb);
+        else launch_small<128>(ctx, P, queries, q, tiers, o, sh, sb);
     } else {
         classify_kernel<<<(unsigned)ceil_div(q, 256 * CL_PER), 256, 0, s>>>(queries, q, P, wcap, ccap, ccap_big, lane_ok,
                                                                              group_max, tiers, o, ctx->d_status);

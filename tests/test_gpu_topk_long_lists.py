@@ -1,7 +1,10 @@
-"""Top-k queries with very long path lists: counts so large that one coded bin of
-the ranking holds more candidates than its buffer. Results are integers and equal
-the oracle's."""
+"""Top-k queries with very long path lists, few at a time and many: teams of
+1,024 threads while the batch leaves SMs idle, for k > 64 device tables shared by
+many CTAs (ids and ties among their 128-entry lists included), and counts so
+large that one coded bin of the ranking holds more candidates than its buffer.
+Results are integers and equal the oracle's."""
 import os
+import time
 
 import numpy as np
 import pytest
@@ -38,6 +41,22 @@ def _check(pk, P, o, v, k):
     assert np.array_equal(cnt.cpu().numpy().astype(np.uint32), rcnt), (v.size, k)
 
 
+# lists of 60,000 paths (the hub tier shares them for k > 64), and a network too
+# small for it; 31 / 32 queries and four per SM are edges of the rules
+@pytest.mark.parametrize("n,R,T", [(600, 6_000_000, 5), (600, 1_500_000, 20), (400, 3_000_000, 5), (512, 3_000_000, 5)])
+def test_long_lists_match_the_oracle(pk, n, R, T):
+    g = synth.chung_lu(n, 60, 4.0, ("uniform", 1, 9), seed=3)
+    ref = oracle.sample_paths(g, 5, R, T, oracle.ALIAS, threads=THREADS)
+    o = oracle.Oracle(g.n, ref)
+    with pk.Panther(0) as P:
+        P.build_graph(g.row_ptr, g.col, g.w, pk.MODE_ALIAS)
+        P.sample_paths(5, R, T, pk.MODE_ALIAS)
+        P.build_index()
+        for q in (1, 5, 31, 32, n):
+            for k in (10, 65, 128):
+                _check(pk, P, o, np.resize(np.arange(n - 1, -1, -1, dtype=np.int32), q), k)
+
+
 def test_one_coded_bin_of_counts_above_4096(pk):
     # a complete graph: most of a row's 299 counts lie in one coded bin, 6,656 to
     # 7,167, more than the ranking buffer of 256
@@ -55,3 +74,28 @@ def test_one_coded_bin_of_counts_above_4096(pk):
         P.build_index()
         for k in (1, 10, 64, 65, 128):
             _check(pk, P, o, np.arange(0, n, 43, dtype=np.int32), k)
+
+
+def test_few_long_queries_above_64(pk):
+    # one query of about a million paths, 6e6 entries: 0.5 ms when many CTAs share
+    # it, 3.4 ms in one CTA
+    g = synth.chung_lu(600, 60, 4.0, ("uniform", 1, 9), seed=3)
+    t = {}
+    with pk.Panther(0) as P:
+        P.build_graph(g.row_ptr, g.col, g.w, pk.MODE_ALIAS)
+        P.sample_paths(9, 100_000_000, 5, pk.MODE_ALIAS)
+        P.build_index()
+        off = P.index_tensors()[0]
+        length = off[1:] - off[:-1]
+        q = torch.where(length <= 1_000_000, length, 0).argmax().to(torch.int32).reshape(1)
+        assert length[int(q)] > 500_000
+        for k in (128, ):
+            best = 1e9
+            for _ in range(5):
+                torch.cuda.synchronize()
+                t0 = time.perf_counter()
+                P.topk(q, k)
+                torch.cuda.synchronize()
+                best = min(best, time.perf_counter() - t0)
+            t[k] = best
+    assert t[128] < 1.5e-3, t
