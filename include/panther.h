@@ -329,6 +329,8 @@ PANTHER_API panther_status pantherpp_vecs_view(const pantherpp_vecs* v, const ui
  *          CUDA-core brute force with the same bound and rerank), optionally
  *          | PANTHER_IO_HOST.
  * The BF16 screen pads vectors to 64, 128 or 192 columns (D up to 56, 120, 128).
+ * Where pantherpp_vectors found no memory for the copy of more than 64 columns,
+ * the default form takes the FP32 one.
  * Every form returns the exact answer. Errors: EINVAL, ENOMEM, ECUDA. */
 PANTHER_API panther_status pantherpp_knn(panther_ctx* ctx, const pantherpp_vecs* v, const int32_t* queries,
                              int64_t q, int k, int32_t* out_ids, uint64_t* out_dist2, int flags);

@@ -102,7 +102,7 @@ struct pantherpp_vecs {
     uint32_t max_val = 0;
     // candidate side of the screening GEMM, exact rows first
     int64_t npad = 0, nexact = 0;    // positions (multiple of 256), exact positions
-    uint16_t* B = nullptr;           // [npad][64, 128 or 192] bf16 candidate rows
+    uint16_t* B = nullptr;           // [npad][64, 128 or 192] bf16 candidate rows (null: no memory, FP32 form)
     int32_t* cid = nullptr;          // [npad] vertex at each position (-1 padding)
     float* cnrm = nullptr;           // [npad] |b| rounded up
     float* cncf = nullptr;           // [npad] |b|^2 rounded up

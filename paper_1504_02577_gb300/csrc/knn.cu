@@ -165,7 +165,7 @@ __global__ void __launch_bounds__(256) vec_brow_kernel(const uint32_t* __restric
             const uint32_t b = bf16_bits_of(f);
             out[j / 2] = j & 1 ? out[j / 2] | (b << 16) : b;
         }
-        ((uint4*)(B + (p * kb + blk) * KN_K))[sub] = make_uint4(out[0], out[1], out[2], out[3]);
+        if (B) ((uint4*)(B + (p * kb + blk) * KN_K))[sub] = make_uint4(out[0], out[1], out[2], out[3]);
     }
     if (sub == 0) {
         cid[p] = v;
@@ -1672,8 +1672,11 @@ extern "C" panther_status pantherpp_vectors(panther_ctx* ctx, const panther_inde
     x.nexact = last_scan + last_flag;
     x.npad = ceil_div(n, KN_N) * KN_N;
     int32_t* perm = nullptr;
+    // Without memory for the operand rows of wide vectors (256 or 384 bytes per
+    // vertex) k-NN takes the FP32 form, which reads theta alone.
+    st = dev_alloc(ctx, (void**)&x.B, (size_t)x.npad * kn_blocks(D) * KN_K * 2);
+    if (st && (st != PANTHER_ENOMEM || kn_blocks(D) == 1)) return fail(st);
     if ((st = dev_alloc(ctx, (void**)&perm, sizeof(int32_t) * x.npad)) ||
-        (st = dev_alloc(ctx, (void**)&x.B, (size_t)x.npad * kn_blocks(D) * KN_K * 2)) ||
         (st = dev_alloc(ctx, (void**)&x.cid, sizeof(int32_t) * x.npad)) ||
         (st = dev_alloc(ctx, (void**)&x.cnrm, sizeof(float) * x.npad)) ||
         (st = dev_alloc(ctx, (void**)&x.cncf, sizeof(float) * x.npad)) ||
@@ -1774,6 +1777,7 @@ static panther_status knn_run(panther_ctx* ctx, const pantherpp_vecs* vq, const 
                               const int32_t* queries, int64_t q, int k, int32_t* ids, uint64_t* d2, bool fp32,
                               float* dump = nullptr) {
     const pantherpp_vecs& x = *vc;
+    if (!x.B) fp32 = true;
     const pantherpp_vecs* v = vq;
     cudaStream_t s = ctx->stream;
     const int64_t n = vq->n;
