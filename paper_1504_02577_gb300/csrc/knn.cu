@@ -64,7 +64,6 @@ constexpr uint32_t MAX_EXACT = 256;
 
 struct VecMeta {
     int64_t n, npad;                 // vertices, padded to a multiple of 256
-    int64_t nexact;                  // number of exact rows (they come first)
     int D;
 };
 
@@ -125,12 +124,11 @@ __global__ void __launch_bounds__(256) vec_stats_kernel(const uint32_t* __restri
 
 // position of every vertex: exact rows first (id ascending), then the rest
 __global__ void vec_perm_kernel(const uint8_t* __restrict__ exact, const int64_t* __restrict__ exscan, int64_t n,
-                                int64_t nexact, int32_t* __restrict__ perm, int64_t* __restrict__ pos) {
+                                int64_t nexact, int32_t* __restrict__ perm) {
     int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (v >= n) return;
     int64_t p = exact[v] ? exscan[v] : nexact + (v - exscan[v]);
     perm[p] = (int32_t)v;
-    pos[v] = p;
 }
 
 // B rows (candidate role) in permuted order + SoA candidate info: eight lanes
@@ -1636,11 +1634,9 @@ extern "C" panther_status pantherpp_vectors(panther_ctx* ctx, const panther_inde
     v->D = D;
     panther_status st;
     int64_t* flag = nullptr;
-    int64_t* pos = nullptr;
     unsigned* maxv = nullptr;
     auto fail = [&](panther_status x) {
         dev_free(ctx, flag);
-        dev_free(ctx, pos);
         dev_free(ctx, maxv);
         pantherpp_free_vecs(v);
         return x;
@@ -1650,7 +1646,7 @@ extern "C" panther_status pantherpp_vectors(panther_ctx* ctx, const panther_inde
     if ((st = dev_alloc(ctx, (void**)&v->norm2, sizeof(uint64_t) * n)) ||
         (st = dev_alloc(ctx, (void**)&v->nrm, sizeof(float) * n)) ||
         (st = dev_alloc(ctx, (void**)&v->exact, n)) || (st = dev_alloc(ctx, (void**)&flag, sizeof(int64_t) * n)) ||
-        (st = dev_alloc(ctx, (void**)&pos, sizeof(int64_t) * n)) || (st = dev_alloc(ctx, (void**)&maxv, 4)))
+        (st = dev_alloc(ctx, (void**)&maxv, 4)))
         return fail(st);
     PCK(ctx, cudaMemsetAsync(maxv, 0, 4, s));
     unsigned gb = (unsigned)ceil_div(n, 256);
@@ -1685,9 +1681,9 @@ extern "C" panther_status pantherpp_vectors(panther_ctx* ctx, const panther_inde
         dev_free(ctx, perm);
         return fail(st);
     }
-    vec_perm_kernel<<<gb, 256, 0, s>>>(v->exact, flag, n, x.nexact, perm, pos);
+    vec_perm_kernel<<<gb, 256, 0, s>>>(v->exact, flag, n, x.nexact, perm);
     vec_brow_kernel<<<(unsigned)ceil_div(x.npad, 32), 256, 0, s>>>(v->theta, v->norm2, v->nrm, perm,
-                                                                    VecMeta{n, x.npad, x.nexact, D}, x.B, x.cid,
+                                                                    VecMeta{n, x.npad, D}, x.B, x.cid,
                                                                     x.cnrm, x.cncf);
     tile_flags_kernel<<<(unsigned)ceil_div(x.npad / KN_N, 8), 256, 0, s>>>(v->exact, x.cid, x.npad, KN_N, x.ctile,
                                                                              x.npad / KN_N);
@@ -1695,10 +1691,8 @@ extern "C" panther_status pantherpp_vectors(panther_ctx* ctx, const panther_inde
     ctx->launches += 4;
     dev_free(ctx, perm);
     dev_free(ctx, flag);
-    dev_free(ctx, pos);
     dev_free(ctx, maxv);
     flag = nullptr;
-    pos = nullptr;
     maxv = nullptr;
     cudaError_t ce = cudaStreamSynchronize(s);
     if (ce) return fail(cuda_err(ctx, ce, "vector preparation"));

@@ -45,7 +45,6 @@ __device__ __forceinline__ uint32_t hslot(uint32_t key, uint32_t nslots) {
 }
 
 // add `amount` to the count of `key`; returns false if the table is full
-template <bool SHARED>
 __device__ __forceinline__ bool hash_add(unsigned long long* tab, uint32_t nslots, uint32_t key,
                                          uint32_t amount = 1) {
     uint32_t s = hslot(key, nslots);
@@ -353,7 +352,7 @@ struct PathsRef {
 
 // insert the distinct vertices u != v of path r into the table (with thr > 0
 // only the u with cls[u] >= thr)
-template <int STRIDE, bool SHARED>
+template <int STRIDE>
 __device__ __forceinline__ bool insert_path(const PathsRef& P, uint32_t r, int32_t v, unsigned long long* tab,
                                             uint32_t nslots, uint32_t thr = 0) {
     if (r >= (uint64_t)P.R) return false;             // corrupt index entry: the caller flags it, nothing is read
@@ -371,7 +370,7 @@ __device__ __forceinline__ bool insert_path(const PathsRef& P, uint32_t r, int32
             bool dup = false;
 #pragma unroll
             for (int i = 0; i < j; ++i) dup |= (x[i] == x[j]);
-            if (!dup && (thr == 0 || __ldg(P.cls + x[j]) >= thr)) ok &= hash_add<SHARED>(tab, nslots, (uint32_t)x[j]);
+            if (!dup && (thr == 0 || __ldg(P.cls + x[j]) >= thr)) ok &= hash_add(tab, nslots, (uint32_t)x[j]);
         }
     }
     return ok;
@@ -900,9 +899,9 @@ __global__ void __launch_bounds__(256) classify_kernel(const int32_t* __restrict
 // the counts (counts above 62 share bin 63), which also gives m = the slots
 // with count >= c*. With m <= 64 only those slots are compacted and one warp
 // sorts them; otherwise every slot is offered to per-warp lists, then merged.
-// CLEAR empties each filled slot once read (tables that are reused). The
+// Each filled slot is emptied once read (the tables are reused). The
 // list (ranks l and 32+l in lane l) goes to sink(t) in warp 0.
-template <bool CLEAR, class Sink>
+template <class Sink>
 __device__ void cta_select(unsigned long long* tab, uint32_t nslots, unsigned long long* lists, int k, Sink sink) {
     __shared__ unsigned hist[64];
     __shared__ int s_cstar, s_m, s_at;
@@ -949,7 +948,7 @@ __device__ void cta_select(unsigned long long* tab, uint32_t nslots, unsigned lo
         for (uint32_t base = (uint32_t)w * 32; base < nslots; base += (uint32_t)nw * 32) {   // warp-uniform
             const uint32_t s = base + lane;
             const unsigned long long x = s < nslots ? tab[s] : EMPTY;
-            if (CLEAR && x != EMPTY) tab[s] = EMPTY;
+            if (x != EMPTY) tab[s] = EMPTY;
             const bool pass = x != EMPTY && (uint32_t)x >= cstar;
             const unsigned mk = __ballot_sync(0xffffffffu, pass);
             if (!mk) continue;
@@ -975,7 +974,7 @@ __device__ void cta_select(unsigned long long* tab, uint32_t nslots, unsigned lo
         uint64_t sc = 0;
         if (s < nslots) {
             sc = slot_score(tab[s]);
-            if (CLEAR && sc) tab[s] = EMPTY;
+            if (sc) tab[s] = EMPTY;
         }
         t.offer(sc, k);
     }
@@ -1727,7 +1726,7 @@ __global__ void __launch_bounds__(1024, 1) single_kernel(PathsRef P, const int32
         }
     } else {
         for (int64_t e = P.off[v] + threadIdx.x; e < P.off[v + 1]; e += blockDim.x)
-            ok &= insert_path<STRIDE, false>(P, P.pid[e], (int32_t)v, gtab, gslots);
+            ok &= insert_path<STRIDE>(P, P.pid[e], (int32_t)v, gtab, gslots);
     }
     if (!ok) flag_status(status, ST_HASH_FULL);
     __syncthreads();
@@ -1835,7 +1834,7 @@ __global__ void g_count_kernel(PathsRef P, const int32_t* __restrict__ queries, 
         }
     } else {
         for (int64_t e = a + threadIdx.x; e < b; e += blockDim.x)
-            ok &= insert_path<STRIDE, false>(P, P.pid[e], v, tab, G.tab_n[g], thr);
+            ok &= insert_path<STRIDE>(P, P.pid[e], v, tab, G.tab_n[g], thr);
     }
     if (!ok) flag_status(status, ST_HASH_FULL);
 }
@@ -1850,7 +1849,7 @@ __global__ void __launch_bounds__(512) g_select_kernel(GPlan G, unsigned long lo
     const int64_t ns = G.tab_n[g];
     const uint32_t len = (uint32_t)(c0 + G_SLOTS < ns ? G_SLOTS : ns - c0);
     const unsigned lane = threadIdx.x & 31;
-    cta_select<true>(arena + G.tab_off[g] + c0, len, lists, k, [&](const WarpTopK& t) {
+    cta_select(arena + G.tab_off[g] + c0, len, lists, k, [&](const WarpTopK& t) {
         partial[item * KMAX + lane] = t.a;
         partial[item * KMAX + 32 + lane] = t.b;
     });
