@@ -247,8 +247,9 @@ PANTHER_API panther_status panther_index_view(const panther_index* ix, const int
  *   up to 16,384 queries (1,024 for k > 64) run as one launch with a CTA per
  *   query, larger ones by tiers; queries with more candidates than a shared
  *   memory table holds go to the hub tier in both. With k > 64 the hub tier
- *   uses device tables and 128-entry lists only, and the PLAIN form runs the
- *   batched one once per query.
+ *   uses device tables and 128-entry lists only, also takes long queries of
+ *   batches below 32 (networks of 512 vertices and more), and the PLAIN form
+ *   runs the batched one once per query.
  *   flags: PANTHER_TOPK_BATCHED or PANTHER_TOPK_PLAIN, optionally
  *          | PANTHER_IO_HOST (queries/outputs in host memory; the call then
  *          synchronises; batches of 4M queries or more run in four chunks

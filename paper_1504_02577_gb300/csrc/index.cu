@@ -14,8 +14,9 @@
 // three parts added in the scatter: a prefix over the tiles of a group of
 // GROUP (in place, a thread per digit), one over the groups and one over the
 // digits. (As 64-bit counts[digit][tile], copied and scanned in place, the
-// bookkeeping moved 2.7 GB a pass at 52,000 tiles, most of it in sectors that
-// held one count: 1.93 ms for the sort of 5.7e7 pairs of 5M vertices, 1.83 now.)
+// bookkeeping moved 2.7 GB a pass at the 52,000 tiles of 20M vertices, R = 4e7,
+// most of it in sectors that held one count: that index took 8.48 ms, 7.78 now;
+// 5M vertices, R = 1e7, 13,000 tiles: 2.02 and 1.91 ms.)
 //
 // The scatter ranks items with warp-private digit counters:
 // warps own contiguous sub-ranges of a tile and walk them in order, so the
