@@ -78,22 +78,22 @@ def _src_hash(*files):
 # unchanged (SHA-256 of the files), else reported as null. The capture and its
 # command are in profiles/.
 NCU_TRAFFIC = {
-    "tables": {"bytes_5M": 4311739648, "sources": {
-        "paper_1504_02577_gb300/csrc/graph.cu": "b6931b5c408e955ddf424f6cfd8c6481c3034578e74a627fbdca5f15e3f9914c",
-        "paper_1504_02577_gb300/csrc/internal.cuh": "3cae532383c14b26b3e266aa306722dccf3f619429e5d83d1545da44e042d3f1",
+    "tables": {"bytes_5M": 4335235584, "sources": {
+        "paper_1504_02577_gb300/csrc/graph.cu": "454e525003204290a735d722b2bbdf68eea72afdba3d0b4771618f33e904712b",
+        "paper_1504_02577_gb300/csrc/internal.cuh": "8f7574c282f1bb6c57ae419adfcb4163a1472578a2c6c8fbf91345a95cc80d4d",
     }},
-    "sample": {"bytes_5M": 8113694720, "sources": {
-        "paper_1504_02577_gb300/csrc/sample.cu": "6a0961deef0495fb013af3b4aeb2e2a7875ecf2ecd463668c9c638ff5ef5aaba",
-        "paper_1504_02577_gb300/csrc/internal.cuh": "3cae532383c14b26b3e266aa306722dccf3f619429e5d83d1545da44e042d3f1",
+    "sample": {"bytes_5M": 7362045184, "sources": {
+        "paper_1504_02577_gb300/csrc/sample.cu": "713f6a3de810b6439cc3f67742685cc10f2bb650aa47df9578a0ce4704370efe",
+        "paper_1504_02577_gb300/csrc/internal.cuh": "8f7574c282f1bb6c57ae419adfcb4163a1472578a2c6c8fbf91345a95cc80d4d",
     }},
-    "index": {"bytes_5M": 3644863232, "sources": {
-        "paper_1504_02577_gb300/csrc/index.cu": "fa0f5dab980d0de4713e0c3156ace87a85d808fb2021d8f29faa0242470ea345",
-        "paper_1504_02577_gb300/csrc/capi.cu": "597a6e25fa600a1f563883e2c94d998c5ec6145ce2ced5b02c85790390861551",
-        "paper_1504_02577_gb300/csrc/internal.cuh": "3cae532383c14b26b3e266aa306722dccf3f619429e5d83d1545da44e042d3f1",
+    "index": {"bytes_5M": 3492788224, "sources": {
+        "paper_1504_02577_gb300/csrc/index.cu": "b084c0c673378dfb48f331afd6dbea8bf88226e71da2f275fa676cace242a7bf",
+        "paper_1504_02577_gb300/csrc/capi.cu": "45d667fafa1397b074bd662cbe79470f1853af39c1839576f535105ef284bd6b",
+        "paper_1504_02577_gb300/csrc/internal.cuh": "8f7574c282f1bb6c57ae419adfcb4163a1472578a2c6c8fbf91345a95cc80d4d",
     }},
-    "topk": {"bytes_5M": 7915097600, "sources": {
-        "paper_1504_02577_gb300/csrc/topk.cu": "618c5a33fe00c1b2d814437a9ba960b86fb3649ceab6301ce516eaf347bd30ba",
-        "paper_1504_02577_gb300/csrc/internal.cuh": "3cae532383c14b26b3e266aa306722dccf3f619429e5d83d1545da44e042d3f1",
+    "topk": {"bytes_5M": 7926624768, "sources": {
+        "paper_1504_02577_gb300/csrc/topk.cu": "80d957df35b25bf69dafa94bd333bb988621e8257a5d1125e2fa6ac156c82676",
+        "paper_1504_02577_gb300/csrc/internal.cuh": "8f7574c282f1bb6c57ae419adfcb4163a1472578a2c6c8fbf91345a95cc80d4d",
     }},
 }
 
