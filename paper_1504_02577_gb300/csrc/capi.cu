@@ -224,7 +224,7 @@ void panther_free_graph(panther_graph* g) {
     if (!g) return;
     panther_ctx* c = g->ctx;
     dev_free(c, g->vrec);
-    dev_free(c, g->vsmall);
+    if (!g->one_block) dev_free(c, g->vsmall);
     dev_free(c, g->prefix);
     dev_free(c, g->alias);
     dev_free(c, g->col);

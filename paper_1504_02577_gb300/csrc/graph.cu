@@ -1006,6 +1006,12 @@ __global__ void alias_assign_kernel(const uint4* __restrict__ vrec, const int32_
                  scum, part * blockDim.x + threadIdx.x, parts * blockDim.x, narrow);
 }
 
+// Up to this many vertices both kinds of records are one allocation (100 MB at
+// most): a second one, and the first one's release, took 30 to 40 us of a small
+// build (200,000 vertices, unweighted: 422 us before the small records, 463 with
+// two allocations, 425 with one).
+constexpr int64_t ONE_BLOCK = int64_t(1) << 22;
+
 // {start, deg} of every vertex: the records of the alias (S < 2^32) and the
 // unweighted walk
 __global__ void small_records_kernel(const uint4* __restrict__ vrec, int64_t n, uint2* __restrict__ vsmall) {
@@ -1083,7 +1089,9 @@ extern "C" panther_status panther_build_graph(panther_ctx* ctx, int64_t n, int64
         panther_free_graph(g);
         return e;
     };
-    if ((st = dev_alloc(ctx, (void**)&g->vrec, sizeof(uint4) * n)) ||
+    // (small networks: the 8-byte records lie behind the 16-byte ones, which stay)
+    g->one_block = n <= ONE_BLOCK && (modes & (PANTHER_MODE_UNWEIGHTED | PANTHER_MODE_ALIAS));
+    if ((st = dev_alloc(ctx, (void**)&g->vrec, (sizeof(uint4) + (g->one_block ? sizeof(uint2) : 0)) * n)) ||
         (st = dev_alloc(ctx, (void**)&big, sizeof(int32_t) * (n + 1))) ||
         (st = dev_alloc(ctx, (void**)&mid, sizeof(int32_t) * n)) ||
         (st = dev_alloc(ctx, (void**)&mid2, sizeof(int32_t) * n)) ||
@@ -1290,12 +1298,13 @@ extern "C" panther_status panther_build_graph(panther_ctx* ctx, int64_t n, int64
         }
     }
     if ((modes & PANTHER_MODE_UNWEIGHTED) || ((modes & PANTHER_MODE_ALIAS) && narrow)) {
-        if ((st = dev_alloc(ctx, (void**)&g->vsmall, sizeof(uint2) * n))) return free_plan(), fail(st);
+        if (g->one_block) g->vsmall = (uint2*)(g->vrec + n);
+        else if ((st = dev_alloc(ctx, (void**)&g->vsmall, sizeof(uint2) * n))) return free_plan(), fail(st);
         small_records_kernel<<<(unsigned)ceil_div(n, 256), 256, 0, s>>>(g->vrec, n, g->vsmall);
         ctx->launches++;
         if ((e = cudaGetLastError())) return free_plan(), fail(cuda_err(ctx, e, "vertex records"));
         // the prefix walk and wide alias entries need S of the 16-byte records
-        if (!(modes & PANTHER_MODE_PREFIX) && (narrow || !(modes & PANTHER_MODE_ALIAS))) {
+        if (!g->one_block && !(modes & PANTHER_MODE_PREFIX) && (narrow || !(modes & PANTHER_MODE_ALIAS))) {
             dev_free(ctx, g->vrec);
             g->vrec = nullptr;
         }

@@ -65,6 +65,7 @@ struct panther_graph {
     int modes = 0;
     uint4* vrec = nullptr;           // [n]: {start, deg, S_lo, S_hi} (PREFIX, and ALIAS with a row sum from 2^32)
     uint2* vsmall = nullptr;         // [n]: {start, deg} (UNWEIGHTED, and ALIAS otherwise)
+    bool one_block = false;          // vsmall lies behind vrec in its allocation
     void* prefix = nullptr;          // [m]: uint2 {cum, col} or uint4 {cum_lo, cum_hi, col, 0}
     int prefix_wide = 0;             // 1 when a row sum reaches 2^32
     uint4* alias = nullptr;          // [m]: {thr, S, col_self, col_alias}, or {thr_lo, thr_hi, ..} when it does
