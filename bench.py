@@ -79,21 +79,21 @@ def _src_hash(*files):
 # command are in profiles/.
 NCU_TRAFFIC = {
     "tables": {"bytes_5M": 4335235584, "sources": {
-        "paper_1504_02577_gb300/csrc/graph.cu": "454e525003204290a735d722b2bbdf68eea72afdba3d0b4771618f33e904712b",
-        "paper_1504_02577_gb300/csrc/internal.cuh": "8f7574c282f1bb6c57ae419adfcb4163a1472578a2c6c8fbf91345a95cc80d4d",
+        "paper_1504_02577_gb300/csrc/graph.cu": "ddc27aec9543aed73a9bbb3c95e69ed8d2b2f7726b2d6f8367ca312527138159",
+        "paper_1504_02577_gb300/csrc/internal.cuh": "eeaad795871497f38ada3cdb5887cd4102974df9c5128b77b77d089a02da2b07",
     }},
     "sample": {"bytes_5M": 7362045184, "sources": {
         "paper_1504_02577_gb300/csrc/sample.cu": "713f6a3de810b6439cc3f67742685cc10f2bb650aa47df9578a0ce4704370efe",
-        "paper_1504_02577_gb300/csrc/internal.cuh": "8f7574c282f1bb6c57ae419adfcb4163a1472578a2c6c8fbf91345a95cc80d4d",
+        "paper_1504_02577_gb300/csrc/internal.cuh": "eeaad795871497f38ada3cdb5887cd4102974df9c5128b77b77d089a02da2b07",
     }},
     "index": {"bytes_5M": 3492788224, "sources": {
         "paper_1504_02577_gb300/csrc/index.cu": "b084c0c673378dfb48f331afd6dbea8bf88226e71da2f275fa676cace242a7bf",
-        "paper_1504_02577_gb300/csrc/capi.cu": "45d667fafa1397b074bd662cbe79470f1853af39c1839576f535105ef284bd6b",
-        "paper_1504_02577_gb300/csrc/internal.cuh": "8f7574c282f1bb6c57ae419adfcb4163a1472578a2c6c8fbf91345a95cc80d4d",
+        "paper_1504_02577_gb300/csrc/capi.cu": "a595da3269b103efb8a14db77228ffb4a30178e980ced7d39d500de1a1608e08",
+        "paper_1504_02577_gb300/csrc/internal.cuh": "eeaad795871497f38ada3cdb5887cd4102974df9c5128b77b77d089a02da2b07",
     }},
     "topk": {"bytes_5M": 7926624768, "sources": {
         "paper_1504_02577_gb300/csrc/topk.cu": "80d957df35b25bf69dafa94bd333bb988621e8257a5d1125e2fa6ac156c82676",
-        "paper_1504_02577_gb300/csrc/internal.cuh": "8f7574c282f1bb6c57ae419adfcb4163a1472578a2c6c8fbf91345a95cc80d4d",
+        "paper_1504_02577_gb300/csrc/internal.cuh": "eeaad795871497f38ada3cdb5887cd4102974df9c5128b77b77d089a02da2b07",
     }},
 }
 
